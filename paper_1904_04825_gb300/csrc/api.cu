@@ -5,6 +5,7 @@
 #include <cstring>
 #include <atomic>
 #include <new>
+#include <vector>
 
 #include "device.cuh"
 #include "internal.cuh"
@@ -90,6 +91,20 @@ int dalloc(fr_ctx* c, T** p, size_t count) {
   return FR_OK;
 }
 
+// element sizes h of n cells and, behind them, 2 / h (a division costs a kernel's
+// thread 5 FP64 issue slots, so it is taken once per mesh)
+int put_sizes(fr_ctx* c, const double* edges, int n, double** h, double** s) {
+  FRK_TRY(dalloc(c, h, 2 * (size_t)n));
+  *s = *h + n;
+  std::vector<double> v(2 * (size_t)n);
+  for (int i = 0; i < n; ++i) {
+    v[i] = edges[i + 1] - edges[i];
+    v[n + i] = 2.0 / v[i];
+  }
+  FRK_CUDA(c, cudaMemcpy(*h, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice));
+  return FR_OK;
+}
+
 int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   c->opts = *o;
   c->p = p;
@@ -103,19 +118,8 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   c->blk_chunk = c->ne;
   FRK_CUDA(c, cudaGetDevice(&c->device));
   build_tables(p, &c->tab);
-  double* hx = new double[mesh->nx];
-  double* hy = new double[mesh->ny];
-  for (int i = 0; i < mesh->nx; ++i) hx[i] = mesh->x_edges[i + 1] - mesh->x_edges[i];
-  for (int i = 0; i < mesh->ny; ++i) hy[i] = mesh->y_edges[i + 1] - mesh->y_edges[i];
-  int rc = dalloc(c, &c->hx, mesh->nx);
-  if (rc == FR_OK) rc = dalloc(c, &c->hy, mesh->ny);
-  if (rc == FR_OK && cudaMemcpy(c->hx, hx, mesh->nx * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
-    rc = set_error(c, FR_ERR_CUDA, "copying the mesh failed");
-  if (rc == FR_OK && cudaMemcpy(c->hy, hy, mesh->ny * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
-    rc = set_error(c, FR_ERR_CUDA, "copying the mesh failed");
-  delete[] hx;
-  delete[] hy;
-  FRK_TRY(rc);
+  FRK_TRY(put_sizes(c, mesh->x_edges, mesh->nx, &c->hx, &c->sx));
+  FRK_TRY(put_sizes(c, mesh->y_edges, mesh->ny, &c->hy, &c->sy));
   c->box[0] = mesh->x_edges[0];
   c->box[1] = mesh->x_edges[mesh->nx];
   c->box[2] = mesh->y_edges[0];
@@ -193,18 +197,9 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
               (mesh->z_edges[mesh->nz] - mesh->z_edges[0]);
   FRK_CUDA(c, cudaGetDevice(&c->device));
   build_tables(p, &c->tab);
-  const double* edges[3] = {mesh->x_edges, mesh->y_edges, mesh->z_edges};
-  const int counts[3] = {mesh->nx, mesh->ny, mesh->nz};
-  double** dst[3] = {&c->hx, &c->hy, &c->hz};
-  for (int d = 0; d < 3; ++d) {
-    double* h = new double[counts[d]];
-    for (int i = 0; i < counts[d]; ++i) h[i] = edges[d][i + 1] - edges[d][i];
-    int rc = dalloc(c, dst[d], counts[d]);
-    if (rc == FR_OK && cudaMemcpy(*dst[d], h, counts[d] * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
-      rc = set_error(c, FR_ERR_CUDA, "copying the mesh failed");
-    delete[] h;
-    FRK_TRY(rc);
-  }
+  FRK_TRY(put_sizes(c, mesh->x_edges, mesh->nx, &c->hx, &c->sx));
+  FRK_TRY(put_sizes(c, mesh->y_edges, mesh->ny, &c->hy, &c->sy));
+  FRK_TRY(put_sizes(c, mesh->z_edges, mesh->nz, &c->hz, &c->sz));
   const size_t n = (size_t)c->ndof;
   const int m = o->m_max;
   const size_t n2 = (size_t)c->n1 * c->n1;
@@ -571,8 +566,7 @@ extern "C" int fr_jv(fr_ctx* ctx, const double* U, const double* R0, const doubl
   if (y == U || y == R0 || y == z) return set_error(ctx, FR_ERR_INVALID_ARG, "fr_jv: y aliases an input");
   cudaStream_t s = as_stream(stream);
   FRK_TRY(launch_linearize(ctx, U, s));
-  FRK_TRY(launch_sumsq(ctx, U, ctx->scal + S_NU2, s));
-  FRK_TRY(launch_sumsq(ctx, z, ctx->scal + S_NZ2, s, true));
+  FRK_TRY(launch_norms_eps(ctx, U, z, s));
   return launch_residual(ctx, 1, U, z, R0, nullptr, y, shift, ctx->scal + S_EPS, nullptr, s);
 }
 

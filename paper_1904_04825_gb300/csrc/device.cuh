@@ -5,10 +5,52 @@
 
 namespace frk {
 
+// Reciprocal and square root for the FP64-issue-bound kernels.  GB300 starts 2
+// FP64 operations per clock and SM, and 1.0 / x and sqrt(x) take 5.3 and 8.8 of
+// those slots (measured: 0.40 and 0.24 per clock); rcp.approx / rsqrt.approx
+// run on another unit (16 per clock) and are good to 2^-19.9, so one step of
+// third order (1/x = r / (1 - e) ~ r (1 + e + e^2), 1/sqrt likewise with
+// 1 + e/2 + 3e^2/8) reaches FP64 in 3 and 5 slots.  Against the correctly
+// rounded results over 6.2e7 arguments: the reciprocal differs in 3e-4 of them,
+// the root in 0.125, by one unit in the last place.  Arguments at the ends of
+// the exponent range (zero, subnormal, infinite, NaN, negative under the root)
+// take the full operations.
+__device__ __forceinline__ bool mid_exponent(double x) {
+  return (unsigned)((__double2hiint(x) & 0x7ff00000) - 0x03000000) < 0x79000000u;
+}
+__device__ __forceinline__ double rcp_fast(double x) {
+  if (!mid_exponent(x)) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double sqrt_fast(double x) {
+  if (!mid_exponent(x) || __double2hiint(x) < 0) return sqrt(x);
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double g = x * r;
+  const double e = fma(-g, r, 1.0);
+  return fma(g, fma(e, 0.375, 0.5) * e, g);
+}
+// The larger of two non-negative values by their bit patterns (fmax takes 2.3
+// FP64 slots); a NaN wins.
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+// FAST selects them.  The finite-difference element blocks and the FP32-linear-
+// parts products keep the correctly rounded operations: they subtract fluxes
+// formed in several kernels, or round the difference to FP32.
+template <bool FAST>
+__device__ __forceinline__ double rcp_of(double x) { return FAST ? rcp_fast(x) : 1.0 / x; }
+template <bool FAST>
+__device__ __forceinline__ double sqrt_of(double x) { return FAST ? sqrt_fast(x) : sqrt(x); }
+
 // Inviscid fluxes f (x) and g (y) of the 2D Euler equations (Sec. 2).
+template <bool FAST = false>
 __device__ __forceinline__ void euler_fluxes(const double q[4], double gam, double f[4],
                                              double g[4]) {
-  const double rinv = 1.0 / q[0];
+  const double rinv = rcp_of<FAST>(q[0]);
   const double u = q[1] * rinv, v = q[2] * rinv;
   const double p = (gam - 1.0) * (q[3] - 0.5 * (q[1] * u + q[2] * v));
   f[0] = q[1];
@@ -16,14 +58,15 @@ __device__ __forceinline__ void euler_fluxes(const double q[4], double gam, doub
   f[2] = q[2] * u;
   f[3] = u * (q[3] + p);
   g[0] = q[2];
-  g[1] = q[1] * v;
+  g[1] = FAST ? f[2] : q[1] * v;
   g[2] = fma(q[2], v, p);
   g[3] = v * (q[3] + p);
 }
 
 // Normal flux along +x (dir 0) or +y (dir 1), plus |u_n| + c.
+template <bool FAST = false>
 __device__ __forceinline__ double normal_flux(const double q[4], int dir, double gam, double f[4]) {
-  const double rinv = 1.0 / q[0];
+  const double rinv = rcp_of<FAST>(q[0]);
   const double u = q[1] * rinv, v = q[2] * rinv;
   const double p = (gam - 1.0) * (q[3] - 0.5 * (q[1] * u + q[2] * v));
   const double un = dir == 0 ? u : v;
@@ -31,7 +74,7 @@ __device__ __forceinline__ double normal_flux(const double q[4], int dir, double
   f[1] = q[1] * un + (dir == 0 ? p : 0.0);
   f[2] = q[2] * un + (dir == 1 ? p : 0.0);
   f[3] = un * (q[3] + p);
-  return fabs(un) + sqrt(gam * p * rinv);
+  return fabs(un) + sqrt_of<FAST>(gam * p * rinv);
 }
 
 // Rusanov common flux f_n = (f(qm)+f(qp))/2 - lam/2 (qp - qm),
@@ -44,6 +87,18 @@ __device__ __forceinline__ void rusanov(const double qm[4], const double qp[4], 
   const double lam = fmax(am, ap);
 #pragma unroll
   for (int v = 0; v < 4; ++v) out[v] = 0.5 * (fm[v] + fp[v]) - 0.5 * lam * (qp[v] - qm[v]);
+}
+
+// Twice the Rusanov flux (the caller's coefficients carry the 1/2): 3 FP64
+// operations per variable instead of 4.
+__device__ __forceinline__ void rusanov2(const double qm[4], const double qp[4], int dir, double gam,
+                                         double out[4]) {
+  double fm[4], fp[4];
+  const double am = normal_flux<true>(qm, dir, gam, fm);
+  const double ap = normal_flux<true>(qp, dir, gam, fp);
+  const double lam = max_nonneg(am, ap);
+#pragma unroll
+  for (int v = 0; v < 4; ++v) out[v] = fma(-lam, qp[v] - qm[v], fm[v] + fp[v]);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -134,22 +189,24 @@ __device__ __forceinline__ void write_eps(const EpsArgs& ea, double nz2) {
 // |lambda_k| alpha_k r_k of the flux Jacobian at the Roe average
 // (sqrt(rho)-weighted velocity and total enthalpy; waves u_n - a, entropy
 // and shear at u_n, u_n + a).
+// FAST: twice that flux, with the fast reciprocals and roots.
+template <bool FAST = false>
 __device__ __forceinline__ void roe(const double qm[4], const double qp[4], int dir, double gam,
                                     double out[4]) {
   double fm[4], fp[4];
-  (void)normal_flux(qm, dir, gam, fm);
-  (void)normal_flux(qp, dir, gam, fp);
-  const double rim = 1.0 / qm[0], rip = 1.0 / qp[0];
+  (void)normal_flux<FAST>(qm, dir, gam, fm);
+  (void)normal_flux<FAST>(qp, dir, gam, fp);
+  const double rim = rcp_of<FAST>(qm[0]), rip = rcp_of<FAST>(qp[0]);
   const double um = qm[1] * rim, vm = qm[2] * rim, up = qp[1] * rip, vp = qp[2] * rip;
   const double pm = (gam - 1.0) * (qm[3] - 0.5 * (qm[1] * um + qm[2] * vm));
   const double pp = (gam - 1.0) * (qp[3] - 0.5 * (qp[1] * up + qp[2] * vp));
   const double Hm = (qm[3] + pm) * rim, Hp = (qp[3] + pp) * rip;
-  const double sm = sqrt(qm[0]), sp = sqrt(qp[0]);
-  const double w = 1.0 / (sm + sp);
+  const double sm = sqrt_of<FAST>(qm[0]), sp = sqrt_of<FAST>(qp[0]);
+  const double w = rcp_of<FAST>(sm + sp);
   const double u = (sm * um + sp * up) * w, v = (sm * vm + sp * vp) * w, H = (sm * Hm + sp * Hp) * w;
   const double rho = sm * sp;
   const double a2 = (gam - 1.0) * (H - 0.5 * (u * u + v * v));
-  const double a = sqrt(a2), ia2 = 1.0 / a2;
+  const double a = sqrt_of<FAST>(a2), ia2 = rcp_of<FAST>(a2);
   const double un = dir == 0 ? u : v;
   const double dun = dir == 0 ? up - um : vp - vm;
   const double dut = dir == 0 ? vp - vm : up - um;
@@ -172,7 +229,7 @@ __device__ __forceinline__ void roe(const double qm[4], const double qp[4], int 
     d[3] = l1 * (H - v * a) + l2 * k2 + l3 * u + l4 * (H + v * a);
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) out[k] = 0.5 * (fm[k] + fp[k]) - 0.5 * d[k];
+  for (int k = 0; k < 4; ++k) out[k] = FAST ? (fm[k] + fp[k]) - d[k] : 0.5 * (fm[k] + fp[k]) - 0.5 * d[k];
 }
 
 // the common inviscid flux selected by fr_opts.riemann (0 Rusanov, 1 Roe)
@@ -180,6 +237,12 @@ __device__ __forceinline__ void riemann_flux(int kind, const double qm[4], const
                                              double gam, double out[4]) {
   if (kind == 1) roe(qm, qp, dir, gam, out);
   else rusanov(qm, qp, dir, gam, out);
+}
+// twice that flux, by the fast operations
+__device__ __forceinline__ void riemann_flux2(int kind, const double qm[4], const double qp[4], int dir,
+                                              double gam, double out[4]) {
+  if (kind == 1) roe<true>(qm, qp, dir, gam, out);
+  else rusanov2(qm, qp, dir, gam, out);
 }
 
 // ---- asynchronous bulk copies (TMA engine) with mbarrier completion ----

@@ -118,6 +118,9 @@ struct fr_ctx {
   int dim3 = 0;              // 3D hexahedral Navier-Stokes path (5 variables, Np = (p+1)^3)
   int nz = 1;
   double* hz = nullptr;      // 3D: [nz] element depths (device)
+  double* sx = nullptr;      // 2 / hx, 2 / hy, 2 / hz (device; each behind its sizes)
+  double* sy = nullptr;
+  double* sz = nullptr;
   double volume = 0.0;       // 3D: volume of the periodic box
   double* diss = nullptr;    // 3D: the three quadrature sums of the dissipation rate
   long long ne = 0, ndof = 0;
@@ -250,6 +253,8 @@ int launch_solution_update(fr_ctx* ctx, double* x, cudaStream_t s);
 // krylov.cu
 int launch_sumsq(fr_ctx* ctx, const double* x, double* out, cudaStream_t s, bool with_eps = false);
 EpsArgs eps_args(fr_ctx* ctx, bool on);
+// ||U||^2, ||z||^2 and the FD step of the product A z in one launch
+int launch_norms_eps(fr_ctx* ctx, const double* U, const double* z, cudaStream_t s);
 int launch_lincomb(fr_ctx* ctx, double* out, int nterms, const double* const* xs,
                    const double* coefs, double* sumsq, cudaStream_t s);
 int launch_copy(fr_ctx* ctx, double* dst, const double* src, cudaStream_t s);

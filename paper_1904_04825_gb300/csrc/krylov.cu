@@ -20,18 +20,49 @@ unsigned vgrid(const fr_ctx* ctx, long long n) {
   return (unsigned)(g < 1 ? 1 : g);
 }
 
+// this thread's share of ||x||^2: one FMA chain in row order, eight loads in
+// flight (with one, 16.8 M rows ran at a tenth of HBM's rate)
+__device__ __forceinline__ double sumsq_rows(const double* __restrict__ x, long long n) {
+  const long long S = (long long)gridDim.x * blockDim.x;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  double ss = 0.0;
+  for (; i + 7 * S < n; i += 8 * S) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = x[i + u * S];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) ss = fma(v[u], v[u], ss);
+  }
+  for (; i < n; i += S) ss = fma(x[i], x[i], ss);
+  return ss;
+}
+
 __global__ void k_sumsq(const double* __restrict__ x, long long n, double* out, Reduce red,
                         EpsArgs ea) {
   __shared__ double sh[32];
-  double ss = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    ss = fma(x[i], x[i], ss);
-  const double bs = block_sum(ss, sh);
+  const double bs = block_sum(sumsq_rows(x, n), sh);
   if (threadIdx.x == 0) red.partials[(size_t)blockIdx.x * kMaxVec] = bs;
   if (last_block(red.counter)) {
     finish_sums(red, 1, out);
     if (threadIdx.x == 0) write_eps(ea, *out);
+  }
+}
+
+// out[0] = ||x||^2 (the FD step's ||U||^2), out[1] = ||y||^2 and the FD step from
+// both: one launch for the two norms of a product, each summed as k_sumsq sums it
+__global__ void k_sumsq2(const double* __restrict__ x, const double* __restrict__ y, long long n, double* out,
+                         Reduce red, EpsArgs ea) {
+  __shared__ double sh[32];
+  const double bx = block_sum(sumsq_rows(x, n), sh);
+  const double by = block_sum(sumsq_rows(y, n), sh);
+  if (threadIdx.x == 0) {
+    red.partials[(size_t)blockIdx.x * kMaxVec] = bx;
+    red.partials[(size_t)blockIdx.x * kMaxVec + 1] = by;
+  }
+  if (last_block(red.counter)) {
+    finish_sums(red, 2, out);
+    __syncthreads();
+    if (threadIdx.x == 0) write_eps(ea, out[1]);
   }
 }
 
@@ -427,6 +458,13 @@ EpsArgs eps_args(fr_ctx* ctx, bool on) {
 
 int launch_sumsq(fr_ctx* ctx, const double* x, double* out, cudaStream_t s, bool with_eps) {
   { ProfScope ps_(ctx, FR_KF_OTHER, s); k_sumsq<<<vgrid(ctx, ctx->ndof), kThreads, 0, s>>>(x, ctx->ndof, out, ctx->red, eps_args(ctx, with_eps)); }
+  FRK_LAUNCHED(ctx);
+  return FR_OK;
+}
+
+int launch_norms_eps(fr_ctx* ctx, const double* U, const double* z, cudaStream_t s) {
+  static_assert(S_NZ2 == S_NU2 + 1, "k_sumsq2 writes the two norms side by side");
+  { ProfScope ps_(ctx, FR_KF_OTHER, s); k_sumsq2<<<vgrid(ctx, ctx->ndof), kThreads, 0, s>>>(U, z, ctx->ndof, ctx->scal + S_NU2, ctx->red, eps_args(ctx, true)); }
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }

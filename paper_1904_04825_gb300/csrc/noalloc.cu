@@ -1,7 +1,7 @@
 // fr_jv_noalloc: the finite-difference operator of fr_jv for callers that
 // cannot allocate device memory.
 //
-// Its working memory (mesh edges and widths, the partial sums of the norm
+// Its working memory (mesh edges and 2 / widths, the partial sums of the norm
 // reductions, the FD step) lives in one file-scope static device array of
 // fixed size, so a call allocates nothing.  Every GPU that loads the library
 // holds that array until the process exits.  All calls share it and it keeps
@@ -16,19 +16,19 @@ constexpr int kNoAllocMaxCells = 4096;  // largest nx and ny
 // layout of the scratch array, in doubles
 constexpr size_t kOffXE = 0;                                     // x edges (nx+1)
 constexpr size_t kOffYE = kOffXE + kNoAllocMaxCells + 1;         // y edges (ny+1)
-constexpr size_t kOffHX = kOffYE + kNoAllocMaxCells + 1;         // widths (nx)
-constexpr size_t kOffHY = kOffHX + kNoAllocMaxCells;             // heights (ny)
-constexpr size_t kOffPart = kOffHY + kNoAllocMaxCells;           // reduction partials
+constexpr size_t kOffSX = kOffYE + kNoAllocMaxCells + 1;         // 2 / width (nx)
+constexpr size_t kOffSY = kOffSX + kNoAllocMaxCells;             // 2 / height (ny)
+constexpr size_t kOffPart = kOffSY + kNoAllocMaxCells;           // reduction partials
 constexpr size_t kOffScal = kOffPart + (size_t)kVecBlocks * kMaxVec;
 constexpr size_t kOffCount = kOffScal + S_COUNT;                 // completion counter
 constexpr size_t kScratchDoubles = ((kOffCount + 1 + 31) / 32) * 32;
 
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
 
-__global__ void k_widths(double* scratch, int nx, int ny) {
+__global__ void k_scales(double* scratch, int nx, int ny) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nx) scratch[kOffHX + i] = scratch[kOffXE + i + 1] - scratch[kOffXE + i];
-  if (i < ny) scratch[kOffHY + i] = scratch[kOffYE + i + 1] - scratch[kOffYE + i];
+  if (i < nx) scratch[kOffSX + i] = 2.0 / (scratch[kOffXE + i + 1] - scratch[kOffXE + i]);
+  if (i < ny) scratch[kOffSY + i] = 2.0 / (scratch[kOffYE + i + 1] - scratch[kOffYE + i]);
 }
 
 // Device address of the scratch array on the current device, looked up on
@@ -47,7 +47,7 @@ int scratch_for_device(double** out) {
 }
 
 // Stream-ordered body: clear the counter, bring the edges in, form the
-// widths, then ||U||^2, ||z||^2 with the FD step, and the operator itself.
+// scales, then ||U||^2, ||z||^2 with the FD step, and the operator itself.
 int run_jv(fr_ctx* ctx, const fr_mesh_desc* mesh, double* sp, const double* U, const double* R0,
            const double* z, double shift, double* y, cudaStream_t s) {
   FRK_CUDA(ctx, cudaMemsetAsync(ctx->red.counter, 0, sizeof(unsigned), s));
@@ -57,10 +57,9 @@ int run_jv(fr_ctx* ctx, const fr_mesh_desc* mesh, double* sp, const double* U, c
                                 cudaMemcpyHostToDevice, s));
   const int mx = ctx->nx > ctx->ny ? ctx->nx : ctx->ny;
   count_launch();
-  k_widths<<<(mx + 255) / 256, 256, 0, s>>>(sp, ctx->nx, ctx->ny);
+  k_scales<<<(mx + 255) / 256, 256, 0, s>>>(sp, ctx->nx, ctx->ny);
   FRK_LAUNCHED(ctx);
-  FRK_TRY(launch_sumsq(ctx, U, ctx->scal + S_NU2, s));
-  FRK_TRY(launch_sumsq(ctx, z, ctx->scal + S_NZ2, s, true));
+  FRK_TRY(launch_norms_eps(ctx, U, z, s));
   return launch_residual(ctx, 1, U, z, R0, nullptr, y, shift, ctx->scal + S_EPS, nullptr, s);
 }
 
@@ -141,8 +140,8 @@ extern "C" int fr_jv_noalloc(const fr_mesh_desc* mesh, int p, const fr_opts* opt
   c.ndof = c.ne * c.nb;
   c.opts = o;
   build_tables(p, &c.tab);
-  c.hx = sp + kOffHX;
-  c.hy = sp + kOffHY;
+  c.sx = sp + kOffSX;
+  c.sy = sp + kOffSY;
   c.scal = sp + kOffScal;
   c.red.partials = sp + kOffPart;
   c.red.counter = reinterpret_cast<unsigned*>(sp + kOffCount);

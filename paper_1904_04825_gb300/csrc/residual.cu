@@ -12,6 +12,11 @@
 // conservation holds to round-off).  The corrected divergence uses the
 // folded derivative matrix Dt (the local-flux traces F^l(+-1) are absorbed
 // into Dt, which removes their extrapolation from the flop count).
+//
+// Bound: FP64 issue (two operations per clock and SM).  At 512^2, p = 3, R and
+// A z with its two norms take 2241 us together; with IEEE divisions, roots and
+// fmax in the fluxes, two divisions per thread for the metric and one load in
+// flight in the norms they took 2718 us.
 #include "device.cuh"
 
 namespace frk {
@@ -23,8 +28,8 @@ struct ResArgs {
   const double* R0;
   const double* b;
   double* out;
-  const double* hx;
-  const double* hy;
+  const double* sx;    // 2 / hx per element column
+  const double* sy;    // 2 / hy per element row
   const double* eps2;  // (eps, 1/eps) of the FD product
   const int* done;
   long long ne;
@@ -75,6 +80,12 @@ template <> struct Tile<5, 0> { static constexpr int TX = 2, TY = 3; };
 template <> struct Tile<5, 1> { static constexpr int TX = 3, TY = 2; };
 template <> struct Tile<6, 0> { static constexpr int TX = 2, TY = 2; };
 template <> struct Tile<6, 1> { static constexpr int TX = 5, TY = 1; };
+// Shape 2: small meshes, whose shape-0 tiles would leave most SMs idle (see use_small_tile).
+template <> struct Tile<2, 2> { static constexpr int TX = 2, TY = 2; };
+template <> struct Tile<3, 2> { static constexpr int TX = 2, TY = 2; };
+template <> struct Tile<4, 2> { static constexpr int TX = 2, TY = 1; };
+template <> struct Tile<5, 2> { static constexpr int TX = 2, TY = 1; };
+template <> struct Tile<6, 2> { static constexpr int TX = 1, TY = 1; };
 
 template <int P, int MODE, int TV, int RM>
 __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restrict__ out, int bid) {
@@ -83,6 +94,10 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
   constexpr int NXF = (TX + 1) * TY * N;  // points on the tile's x-faces (normal +x)
   constexpr int NYF = (TY + 1) * TX * N;  // points on the tile's y-faces (normal +y)
   constexpr bool PERTURB = MODE == 1 || MODE == 2;  // MODE 3: R's fluxes at U into the caches
+  // MODE 3 feeds the FP32-linear-parts product, which repeats its fluxes with
+  // the correctly rounded operations; the others take the fast ones, whose
+  // common flux comes out doubled (sdgL, sdgR carry the 1/2)
+  constexpr bool FAST = MODE != 3;
   __shared__ double sq[NE][4][NP];
   __shared__ double sF[NE][4][NP];
   __shared__ double sG[NE][4][NP];
@@ -100,8 +115,8 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
   if (threadIdx.x < N) {
     slm[threadIdx.x] = a.tab.lm[threadIdx.x];
     slp[threadIdx.x] = a.tab.lp[threadIdx.x];
-    sdgL[threadIdx.x] = a.tab.dgL[threadIdx.x];
-    sdgR[threadIdx.x] = a.tab.dgR[threadIdx.x];
+    sdgL[threadIdx.x] = 0.5 * a.tab.dgL[threadIdx.x];
+    sdgR[threadIdx.x] = 0.5 * a.tab.dgR[threadIdx.x];
   }
 
   const int tiles_x = (a.nx + TX - 1) / TX;
@@ -127,7 +142,7 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
       q[v] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
       sq[el][v][t] = q[v];
     }
-    euler_fluxes(q, a.gam, f, g);
+    euler_fluxes<FAST>(q, a.gam, f, g);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       sF[el][v][t] = f[v];
@@ -197,7 +212,8 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
         qm[v] = pm[v * N];
         qp[v] = pp[v * N];
       }
-      riemann_flux(RM, qm, qp, 0, a.gam, fc);
+      if (FAST) riemann_flux2(RM, qm, qp, 0, a.gam, fc);
+      else riemann_flux(RM, qm, qp, 0, a.gam, fc);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sfx[fy][xf][v][k] = fc[v];
       if (MODE == 3 && xf < ax) {  // the west face of tile element xf
@@ -221,7 +237,8 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
         qm[v] = pm[v * N];
         qp[v] = pp[v * N];
       }
-      riemann_flux(RM, qm, qp, 1, a.gam, fc);
+      if (FAST) riemann_flux2(RM, qm, qp, 1, a.gam, fc);
+      else riemann_flux(RM, qm, qp, 1, a.gam, fc);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sfy[fx][yf][v][k] = fc[v];
       if (MODE == 3 && yf < ay) {  // the south face of tile element yf
@@ -239,10 +256,9 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, double* __restri
 
   // ---- 3: corrected divergence and the output ----
   if (MODE == 3 || !active) return;
-  const double hx = a.hx[ix0 + lx], hy = a.hy[iy0 + ly];
   const int i = t % N, j = t / N;
   // with unscaled fluxes, -(1/|J|)(dF~/dxi + dG~/deta) = -(2/hx) df~ - (2/hy) dg~
-  const double sx = 2.0 / hx, sy = 2.0 / hy;
+  const double sx = a.sx[ix0 + lx], sy = a.sy[iy0 + ly];
   const long long base = e * 4 * NP + t;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
@@ -443,7 +459,7 @@ __global__ void __launch_bounds__(256) k_jv32(const ResArgs a) {
   __syncthreads();
   // ---- 3: corrected divergence of the differences (FP32), output (FP64) ----
   if (!active) return;
-  const float sx = (float)(2.0 / a.hx[ix0 + lx]), sy = (float)(2.0 / a.hy[iy0 + ly]);
+  const float sx = (float)a.sx[ix0 + lx], sy = (float)a.sy[iy0 + ly];
   const int i = t % N, j = t / N;
   const long long base = e * 4 * NP + t;
 #pragma unroll
@@ -477,14 +493,27 @@ int launch_pvr(fr_ctx* ctx, int mode, const ResArgs& a, cudaStream_t s) {
   const double wb = in_cycle ? 0.0 : (mode == 0 ? 16.0 : (mode == 1 ? 32.0 : 40.0)) * nd;
   const double wf = in_cycle ? 0.0 : (mode == 0 ? fl : fl + 6.0 * nd);
   const bool mixed = ctx->opts.jv_precision == 1;
+  if constexpr (TV != 2) {
+    if (mode == 3) { ProfScope ps_(ctx, FR_KF_OTHER, s); k_residual<P, 3, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
+    else if (mode == 1 && mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_jv32<P, 1, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
+    else if (mode == 2 && mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_jv32<P, 2, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
+  }
   if (mode == 0) { ProfScope ps_(ctx, FR_KF_RESIDUAL, s, wb, wf); k_residual<P, 0, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
-  else if (mode == 3) { ProfScope ps_(ctx, FR_KF_OTHER, s); k_residual<P, 3, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
-  else if (mode == 1 && mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_jv32<P, 1, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
-  else if (mode == 1) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_residual<P, 1, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
-  else if (mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_jv32<P, 2, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
-  else { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_residual<P, 2, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
+  else if (mode == 1 && !mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_residual<P, 1, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
+  else if (mode == 2 && !mixed) { ProfScope ps_(ctx, FR_KF_JV, s, wb, wf); k_residual<P, 2, TV, RM><<<(unsigned)grid, blk, 0, s>>>(a); }
   FRK_LAUNCHED(ctx);
   return FR_OK;
+}
+
+// Shape-0 tiles of 9 to 25 elements keep a CTA busy for 20 us, so a mesh with
+// fewer of them than the chip has SMs runs on a fraction of its FP64 units; the
+// small tiles repeat more halo traces (about a third more FP64 work) but spread.
+template <int P>
+bool use_small_tile(const fr_ctx* ctx, int mode) {
+  if (ctx->tile_variant != 0 || mode == 3 || (mode != 0 && ctx->opts.jv_precision == 1)) return false;
+  constexpr int TX = Tile<P, 0>::TX, TY = Tile<P, 0>::TY;
+  const long long tiles = (long long)((ctx->nx + TX - 1) / TX) * ((ctx->ny + TY - 1) / TY);
+  return tiles < ctx->num_sms;
 }
 
 // the common flux is a template parameter so each flux gets its own register allocation
@@ -495,6 +524,7 @@ int launch_pv(fr_ctx* ctx, int mode, const ResArgs& a, cudaStream_t s) {
 
 template <int P>
 int launch_p(fr_ctx* ctx, int mode, const ResArgs& a, cudaStream_t s) {
+  if (use_small_tile<P>(ctx, mode)) return launch_pv<P, 2>(ctx, mode, a, s);
   return ctx->tile_variant == 1 ? launch_pv<P, 1>(ctx, mode, a, s) : launch_pv<P, 0>(ctx, mode, a, s);
 }
 
@@ -507,7 +537,7 @@ int launch_residual(fr_ctx* ctx, int mode, const double* U, const double* z, con
   if (ctx->viscous) return launch_ns_residual(ctx, mode, U, z, R0, b, out, shift, eps2, done, s);
   ResArgs a;
   a.U = U; a.z = z; a.R0 = R0; a.b = b; a.out = out;
-  a.hx = ctx->hx; a.hy = ctx->hy; a.eps2 = eps2; a.done = done;
+  a.sx = ctx->sx; a.sy = ctx->sy; a.eps2 = eps2; a.done = done;
   a.ne = ctx->ne; a.nx = ctx->nx; a.ny = ctx->ny;
   a.gam = ctx->opts.gamma; a.shift = shift;
   a.eps_rel = ctx->opts.eps_rel; a.eps_fixed = ctx->opts.eps_fixed;
@@ -544,7 +574,7 @@ int fill_batch_residual(fr_ctx* ctx, const double* U, const double* R0, double s
   if (ctx->dim3 || ctx->viscous || ctx->opts.jv_precision != 0 || ctx->p < 2 || ctx->p > 4) return FR_ERR_UNSUPPORTED;
   ResArgs a{};
   a.U = U; a.z = ctx->z; a.R0 = R0; a.b = nullptr; a.out = ctx->V;
-  a.hx = ctx->hx; a.hy = ctx->hy; a.eps2 = ctx->scal + S_EPS; a.done = ctx->gd.done;
+  a.sx = ctx->sx; a.sy = ctx->sy; a.eps2 = ctx->scal + S_EPS; a.done = ctx->gd.done;
   a.ne = ctx->ne; a.nx = ctx->nx; a.ny = ctx->ny;
   a.gam = ctx->opts.gamma; a.shift = shift;
   a.eps_rel = ctx->opts.eps_rel; a.eps_fixed = ctx->opts.eps_fixed;
