@@ -64,9 +64,9 @@ __device__ __forceinline__ void euler_fluxes(const double q[4], double gam, doub
 }
 
 // Normal flux along +x (dir 0) or +y (dir 1), plus |u_n| + c.
-template <bool FAST = false>
+template <bool FR = false, bool FS = FR>
 __device__ __forceinline__ double normal_flux(const double q[4], int dir, double gam, double f[4]) {
-  const double rinv = rcp_of<FAST>(q[0]);
+  const double rinv = rcp_of<FR>(q[0]);
   const double u = q[1] * rinv, v = q[2] * rinv;
   const double p = (gam - 1.0) * (q[3] - 0.5 * (q[1] * u + q[2] * v));
   const double un = dir == 0 ? u : v;
@@ -74,7 +74,7 @@ __device__ __forceinline__ double normal_flux(const double q[4], int dir, double
   f[1] = q[1] * un + (dir == 0 ? p : 0.0);
   f[2] = q[2] * un + (dir == 1 ? p : 0.0);
   f[3] = un * (q[3] + p);
-  return fabs(un) + sqrt_of<FAST>(gam * p * rinv);
+  return fabs(un) + sqrt_of<FS>(gam * p * rinv);
 }
 
 // Rusanov common flux f_n = (f(qm)+f(qp))/2 - lam/2 (qp - qm),
@@ -90,12 +90,14 @@ __device__ __forceinline__ void rusanov(const double qm[4], const double qp[4], 
 }
 
 // Twice the Rusanov flux (the caller's coefficients carry the 1/2): 3 FP64
-// operations per variable instead of 4.
+// operations per variable instead of 4.  FR: the fast reciprocal (the root is
+// always the fast one; it only scales the jump).
+template <bool FR>
 __device__ __forceinline__ void rusanov2(const double qm[4], const double qp[4], int dir, double gam,
                                          double out[4]) {
   double fm[4], fp[4];
-  const double am = normal_flux<true>(qm, dir, gam, fm);
-  const double ap = normal_flux<true>(qp, dir, gam, fp);
+  const double am = normal_flux<FR, true>(qm, dir, gam, fm);
+  const double ap = normal_flux<FR, true>(qp, dir, gam, fp);
   const double lam = max_nonneg(am, ap);
 #pragma unroll
   for (int v = 0; v < 4; ++v) out[v] = fma(-lam, qp[v] - qm[v], fm[v] + fp[v]);
@@ -242,7 +244,7 @@ __device__ __forceinline__ void riemann_flux(int kind, const double qm[4], const
 __device__ __forceinline__ void riemann_flux2(int kind, const double qm[4], const double qp[4], int dir,
                                               double gam, double out[4]) {
   if (kind == 1) roe<true>(qm, qp, dir, gam, out);
-  else rusanov2(qm, qp, dir, gam, out);
+  else rusanov2<true>(qm, qp, dir, gam, out);
 }
 
 // ---- asynchronous bulk copies (TMA engine) with mbarrier completion ----

@@ -27,6 +27,8 @@ struct Tables {
   double Dt[kMaxN][kMaxN];
   double lm[kMaxN];   // l_k(-1)
   double lp[kMaxN];   // l_k(+1)
+  double dlm[kMaxN];  // l_k'(-1)
+  double dlp[kMaxN];  // l_k'(+1)
   double dgL[kMaxN];  // g_L'(xi_i)
   double dgR[kMaxN];  // g_R'(xi_i)
   double xi[kMaxN];   // solution points

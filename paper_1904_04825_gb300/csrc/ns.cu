@@ -1,21 +1,32 @@
 // Viscous (Navier-Stokes) FR residual with BR2 common gradients, Sec. 2-3
 // (Eqs. com_q, com_grad_q and the BR2 lifting with g'(+-1) = +-(P+1)(P+2)/2).
 //
-// R(U), A z and b - A z take three kernels:
-//  k_ns_trace: per element, the (possibly perturbed) state and its own
-//    polynomial gradient traced to the 4 (p+1) face points -> trace buffer.
+// R(U), A z and b - A z take three kernels, FP64-issue bound:
+//  k_ns_trace: per element, the (possibly perturbed) state q and its normal
+//    derivative traced to the 4 (p+1) face points -> trace buffer.  The
+//    tangential derivative is not traced: it is the derivative along the face
+//    of the common solution, which k_ns_face takes once for both elements.
 //  k_ns_face:  per west / south face point (and north wall), the common
-//    solution, BR2 common gradient and common total flux (Rusanov inviscid
-//    minus viscous) from the two traces -> face buffer, each face once.
+//    solution, the BR2 common gradient and the common total flux (Rusanov
+//    inviscid minus viscous) -> face buffer, each face once.
 //  k_ns_cell:  per element, the FR-corrected gradient and total flux at the
 //    solution points, the corrected divergence with the four faces' common
 //    fluxes, the body-force source and the output.  Both elements of a face
 //    read the same stored flux, so conservation holds to round-off.
-// Element-Jacobi columns use k_ns_res (its mode 3) after a trace pass of the
-// unperturbed state: slot = (element, column c), own state perturbed in DOF
+// Bound: FP64 issue.  R + A z at 256 x 128, p = 3: 660 us; 963 us when all
+// three derivatives were traced from both sides, both viscous fluxes formed on
+// every face, q_com - q subtracted at every point, a third of the face threads
+// kept for walls, and 2 / h divided out by every thread.
+// Element-Jacobi columns use k_ns_res after k_ns_fulltrace, which traces q and
+// its whole gradient: slot = (element, column c), own state perturbed in DOF
 // c by eps_c = beps (1 + |q_c|), own traces recomputed, neighbour traces
 // frozen; it forms the element's four face fluxes itself and stages column c
-// of shift*I - J_ee for the inversion kernel.
+// of shift*I - J_ee for the inversion kernel.  The unperturbed residual of the
+// difference quotients comes from the same kernel (mode 0), by the same
+// operations.
+// In a thin wall cell the heat flux carries the rounding of D q on the total
+// energy (44.6 at Mach 0.2) times (2 / h)^2, which is what limits R: the normal
+// derivatives, the liftings and q_com - q keep one order of operations.
 // Walls (isothermal, no slip) at the y ends: boundary state
 // (rho_int, 0, 0, rho_int R T_w / (gamma - 1)), common gradient = own
 // gradient + own lifting, inviscid wall flux g(q_b).  Gas constant R = 1.
@@ -30,10 +41,12 @@ struct NsArgs {
   const double* R0;
   const double* b;
   double* out;
-  double* tb;          // traces [ne][4 faces][N][4 vars][3] = (q, q_x, q_y)
-  double* fb;          // common data per element's W, S (and top-wall N) face [ne][3][N][8] = (q_com, f_n)
+  double* tb;          // traces [ne][4 faces][N][q 4, q_n 4]; for the blocks [ne][4][N][4 vars][q, q_x, q_y]
+  double* fb;          // [ne][W, S][N][q_com 4, f_n 4], then the north wall's [nx][N][8]
   const double* hx;
   const double* hy;
+  const double* sx;    // 2 / hx
+  const double* sy;    // 2 / hy
   const double* eps2;
   const int* done;
   long long ne;
@@ -92,8 +105,9 @@ __device__ __forceinline__ void face_trace(const double* sq, const double* dxi, 
   }
 }
 
-template <int P, bool PERTURB>
-__global__ void __launch_bounds__(256) k_ns_trace(const NsArgs a) {
+// traces of the unperturbed state and of its gradient, for the block columns
+template <int P>
+__global__ void __launch_bounds__(256) k_ns_fulltrace(const NsArgs a) {
   constexpr int N = P + 1, NP = N * N, E = NsSlots<P>::E;
   __shared__ double sq[E][4 * NP], dxi[E][4 * NP], deta[E][4 * NP];
   __shared__ double sD[N][N], slm[N], slp[N];
@@ -102,16 +116,14 @@ __global__ void __launch_bounds__(256) k_ns_trace(const NsArgs a) {
     slm[threadIdx.x] = a.tab.lm[threadIdx.x];
     slp[threadIdx.x] = a.tab.lp[threadIdx.x];
   }
-  if (a.done && *a.done) return;
   const int el = threadIdx.x / NP, t = threadIdx.x % NP;
   const long long e = (long long)blockIdx.x * E + el;
   const bool active = el < E && e < a.ne;
-  const double eps = PERTURB ? a.eps2[0] : 0.0;
   if (active) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const long long o = e * 4 * NP + v * NP + t;
-      sq[el][v * NP + t] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+      sq[el][v * NP + t] = a.U[o];
     }
   }
   __syncthreads();
@@ -132,7 +144,7 @@ __global__ void __launch_bounds__(256) k_ns_trace(const NsArgs a) {
   __syncthreads();
   if (!active) return;
   const int ix = (int)(e % a.nx), iy = (int)(e / a.nx);
-  const double sx = 2.0 / a.hx[ix], sy = 2.0 / a.hy[iy];
+  const double sx = a.sx[ix], sy = a.sy[iy];
   for (int fp = t; fp < 4 * N; fp += NP) {
     const int face = fp / N, k = fp % N;
     double tr[4][3];
@@ -145,7 +157,7 @@ __global__ void __launch_bounds__(256) k_ns_trace(const NsArgs a) {
   }
 }
 
-// common total flux across a face from the left (-) and right (+) data;
+// (block columns) common total flux across a face from the left (-) and right (+) data;
 // dir 0: x-face (normal +x), 1: y-face (normal +y); hm, hp: element sizes
 // normal to the face; cbr2 = (P+1)(P+2)/2.
 __device__ __forceinline__ void common_flux(const double m[4][3], const double pp[4][3], int dir,
@@ -200,7 +212,7 @@ __device__ __forceinline__ void wall_flux(const double o[4][3], bool south, doub
 template <int P, int MODE>
 __global__ void __launch_bounds__(256) k_ns_res(const NsArgs a) {
   constexpr int N = P + 1, NP = N * N, E = NsSlots<P>::E, NB = 4 * NP;
-  constexpr bool PERTURB = MODE == 1 || MODE == 2;
+  static_assert(MODE == 0 || MODE == 3, "R(U) or the block columns");
   constexpr double cbr2 = (P + 1) * (P + 2) / 2.0;
   __shared__ double sq[E][4 * NP], dxi[E][4 * NP], deta[E][4 * NP];  // dxi/deta reused for F, G
   __shared__ double tr[E][4][N][4][3];   // own face traces
@@ -224,11 +236,6 @@ __global__ void __launch_bounds__(256) k_ns_res(const NsArgs a) {
   const bool active = el < E && slot < nslots;
   const long long e = MODE == 3 ? slot / NB : slot;
   const int col = MODE == 3 ? (int)(slot % NB) : 0;
-  double eps = 0.0, ieps = 0.0;
-  if (PERTURB) {
-    eps = a.eps2[0];
-    ieps = a.eps2[1];
-  }
   int ix = 0, iy = 0;
   double hx = 1.0, hy = 1.0;
   double ceps = 0.0;
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(256) k_ns_res(const NsArgs a) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const long long o = e * 4 * NP + v * NP + t;
-      double qv = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+      double qv = a.U[o];
       if (MODE == 3 && v * NP + t == col) qv += ceps;
       sq[el][v * NP + t] = qv;
     }
@@ -262,7 +269,7 @@ __global__ void __launch_bounds__(256) k_ns_res(const NsArgs a) {
     }
   }
   __syncthreads();
-  const double sx = 2.0 / hx, sy = 2.0 / hy;
+  const double sx = active ? a.sx[ix] : 0.0, sy = active ? a.sy[iy] : 0.0;
   if (active) {
     for (int fp = t; fp < 4 * N; fp += NP) {
       const int face = fp / N, k = fp % N;
@@ -356,72 +363,165 @@ __global__ void __launch_bounds__(256) k_ns_res(const NsArgs a) {
     const long long o = base + v * NP;
     if (MODE == 0) {
       a.out[o] = R;
-    } else if (MODE == 3) {
+    } else {
       // column col of M = shift I - J_ee, staged column-major [col][row]
       const int row = v * NP + t;
       const double m = (row == col ? a.shift : 0.0) - (R - a.R0[o]) / ceps;
       a.out[(e * NB + col) * NB + row] = m;
-    } else {
-      const double zo = a.z[o];
-      const double Az = eps > 0.0 ? fma(-(R - a.R0[o]), ieps, a.shift * zo) : a.shift * zo;
-      a.out[o] = MODE == 2 ? a.b[o] - Az : Az;
     }
   }
 }
 
-// Modes 0-2 in two passes so every face's common data is formed once:
-// k_ns_face: one thread per (element, face W or S, point): q_com and the
-//   common total flux from the two traces in the trace buffer (or the wall
-//   state), into the face buffer; top-row elements also form their north
-//   wall face.
-// k_ns_cell: per element the FR-corrected gradient with q_com of its four
-//   faces, the point fluxes, the corrected divergence with the common fluxes
-//   of its four faces (W, S own; E, N the neighbours' W, S), body force and
-//   the output.  Both elements of a face read the same stored flux, so
-//   conservation holds to round-off.
+// q and its normal derivative at the face points; work items over the CTA's
+// E elements x 4N points, so no degree leaves threads with a second round alone
+template <int P, bool PERTURB>
+__global__ void __launch_bounds__(256) k_ns_trace(const NsArgs a) {
+  constexpr int N = P + 1, NP = N * N, E = NsSlots<P>::E;
+  __shared__ double sq[E][4 * NP], dd[2][E][4 * NP];
+  __shared__ double sD[N][N], sl[2][N];  // l_k(-+1)
+  if (a.done && *a.done) return;
+  if (threadIdx.x < N * N) sD[threadIdx.x / N][threadIdx.x % N] = a.tab.D[threadIdx.x / N][threadIdx.x % N];
+  if (threadIdx.x < N) {
+    sl[0][threadIdx.x] = a.tab.lm[threadIdx.x];
+    sl[1][threadIdx.x] = a.tab.lp[threadIdx.x];
+  }
+  const long long e0 = (long long)blockIdx.x * E;
+  const int ne = a.ne - e0 < E ? (int)(a.ne - e0) : E;
+  const double eps = PERTURB ? a.eps2[0] : 0.0;
+  for (int i = threadIdx.x; i < ne * 4 * NP; i += blockDim.x) {
+    const long long o = e0 * 4 * NP + i;
+    sq[0][i] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+  }
+  __syncthreads();
+  {
+    const int el = threadIdx.x / NP, t = threadIdx.x % NP, i = t % N, j = t / N;
+    if (el < ne) {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        double d1 = 0.0, d2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          d1 = fma(sD[i][k], sq[el][v * NP + k + N * j], d1);
+          d2 = fma(sD[j][k], sq[el][v * NP + i + N * k], d2);
+        }
+        dd[0][el][v * NP + t] = d1;
+        dd[1][el][v * NP + t] = d2;
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * 4 * N; i += blockDim.x) {
+    const int el = i / (4 * N), face = (i / N) % 4, k = i % N;
+    const long long e = e0 + el;
+    const double s = face < 2 ? a.sx[e % a.nx] : a.sy[e / a.nx];
+    const int off = face < 2 ? N * k : k, stride = face < 2 ? 1 : N;
+    double* dst = a.tb + ((e * 4 + face) * N + k) * 8;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      dst[v] = tsum<N>(sq[el] + v * NP + off, stride, sl[face & 1]);
+      dst[4 + v] = s * tsum<N>(dd[face >> 1][el] + v * NP + off, stride, sl[face & 1]);
+    }
+  }
+}
+
+// Viscous flux along a face normal from the common state, its normal gradient
+// gn and tangential gradient gt (dir 0: normal x, 1: normal y), R = 1.
+__device__ __forceinline__ void visc_normal(const double q[4], const double gn[4], const double gt[4], int dir,
+                                            const NsArgs& a, double fv[4]) {
+  const double rinv = rcp_fast(q[0]);
+  const double vn = (dir == 0 ? q[1] : q[2]) * rinv, vt = (dir == 0 ? q[2] : q[1]) * rinv, e = q[3] * rinv;
+  const double n_n = fma(-vn, gn[0], dir == 0 ? gn[1] : gn[2]) * rinv;  // d v_n / d n
+  const double t_n = fma(-vt, gn[0], dir == 0 ? gn[2] : gn[1]) * rinv;  // d v_t / d n
+  const double n_t = fma(-vn, gt[0], dir == 0 ? gt[1] : gt[2]) * rinv;
+  const double t_t = fma(-vt, gt[0], dir == 0 ? gt[2] : gt[1]) * rinv;
+  const double Tn = (a.gam - 1.0) * fma(-vt, t_n, fma(-vn, n_n, fma(-e, gn[0], gn[3]) * rinv));
+  const double tnn = a.mu * fma(4.0 / 3.0, n_n, (-2.0 / 3.0) * t_t);
+  const double tnt = a.mu * (t_n + n_t);
+  fv[0] = 0.0;
+  fv[1] = dir == 0 ? tnn : tnt;
+  fv[2] = dir == 0 ? tnt : tnn;
+  fv[3] = fma(a.kappa, Tn, fma(vt, tnt, vn * tnn));
+}
+
+// threads of k_ns_face: whole faces of N points per CTA
+template <int P> struct FaceThreads { static constexpr int value = 256 / (P + 1) * (P + 1); };
+
+// one thread per point of the west and south faces of every element, then of
+// the north wall; the N threads of a face exchange its common solution in
+// shared memory for the tangential derivative
 template <int P>
 __global__ void __launch_bounds__(256) k_ns_face(const NsArgs a) {
   constexpr int N = P + 1;
   constexpr double cbr2 = (P + 1) * (P + 2) / 2.0;
+  __shared__ double sD[N][N], sc[FaceThreads<P>::value][4];
   if (a.done && *a.done) return;
-  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = a.ne * 3 * N;
-  if (tid >= total) return;
-  const int k = (int)(tid % N);
-  const int slot = (int)((tid / N) % 3);  // 0: west face, 1: south face, 2: north wall
-  const long long e = tid / (3 * N);
+  if (threadIdx.x < N * N) sD[threadIdx.x / N][threadIdx.x % N] = a.tab.D[threadIdx.x / N][threadIdx.x % N];
+  const long long tid = (long long)blockIdx.x * FaceThreads<P>::value + threadIdx.x;
+  const long long inner = a.ne * 2 * N;
+  const bool active = tid < inner + (a.wall_y ? (long long)a.nx * N : 0);
+  const bool north = tid >= inner;
+  const int k = threadIdx.x % N;
+  const int slot = north ? 1 : (int)((tid / N) % 2);  // 0: west face, 1: south face (or the north wall)
+  const long long e = north ? a.ne - a.nx + (tid - inner) / N : tid / (2 * N);
   const int ix = (int)(e % a.nx), iy = (int)(e / a.nx);
-  if (slot == 2 && !(a.wall_y && iy == a.ny - 1)) return;
-  const double hx = a.hx[ix], hy = a.hy[iy];
-  double o[4][3], nb[4][3], qc[4], fn[4];
-  const int oface = slot == 0 ? 0 : (slot == 1 ? 2 : 3);
-  const double* src = a.tb + (((e * 4 + oface) * N + k) * 4) * 3;
+  const bool wall = north || (slot == 1 && a.wall_y && iy == 0);
+  double m[8], o[8], qc[4], gn[4], gt[4];
+  double so = 0.0, sn = 0.0, st = 0.0;
+  if (active) {
+    const int oface = slot == 0 ? 0 : (north ? 3 : 2);
+    const double* src = a.tb + ((e * 4 + oface) * N + k) * 8;
 #pragma unroll
-  for (int v = 0; v < 4; ++v)
+    for (int v = 0; v < 8; ++v) o[v] = src[v];
+    so = slot == 0 ? a.sx[ix] : a.sy[iy];
+    st = slot == 0 ? a.sy[iy] : a.sx[ix];
+    if (!wall) {
+      const int jx = slot == 0 ? (ix + a.nx - 1) % a.nx : ix, jy = slot == 0 ? iy : (iy + a.ny - 1) % a.ny;
+      const double* nsrc = a.tb + (((jx + (long long)a.nx * jy) * 4 + (slot == 0 ? 1 : 3)) * N + k) * 8;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) o[v][c] = src[v * 3 + c];
-  if (slot == 2) {
-    wall_flux(o, false, hy, cbr2, a, qc, fn);
-  } else if (slot == 1 && a.wall_y && iy == 0) {
-    wall_flux(o, true, hy, cbr2, a, qc, fn);
-  } else {
-    long long nbe;
-    double hn;
-    int nface;
-    if (slot == 0) { const int jx = (ix + a.nx - 1) % a.nx; nbe = jx + (long long)a.nx * iy; nface = 1; hn = a.hx[jx]; }
-    else { const int jy = (iy + a.ny - 1) % a.ny; nbe = ix + (long long)a.nx * jy; nface = 3; hn = a.hy[jy]; }
-    const double* ns = a.tb + (((nbe * 4 + nface) * N + k) * 4) * 3;
+      for (int v = 0; v < 8; ++v) m[v] = nsrc[v];
+      sn = slot == 0 ? a.sx[jx] : a.sy[jy];
+    }
+    // the field whose derivative along the face is the tangential gradient: the
+    // common solution, at a wall the element's own trace
 #pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) nb[v][c] = ns[v * 3 + c];
-    common_flux(nb, o, slot == 0 ? 0 : 1, hn, slot == 0 ? hx : hy, cbr2, a, qc, fn);
+    for (int v = 0; v < 4; ++v) sc[threadIdx.x][v] = qc[v] = wall ? o[v] : 0.5 * (m[v] + o[v]);
   }
-  double* dst = a.fb + ((e * 3 + slot) * N + k) * 8;
+  __syncthreads();
+  if (!active) return;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const double* x = &sc[threadIdx.x - k][v];
+    double s = sD[k][0] * x[0];
+#pragma unroll
+    for (int l = 1; l < N; ++l) s = fma(sD[k][l], x[4 * l], s);
+    gt[v] = st * s;
+  }
+  double fi[4], fv[4];
+  if (wall) {
+    double f[4];
+    qc[1] = qc[2] = 0.0;
+    qc[3] = qc[0] * a.t_wall / (a.gam - 1.0);
+#pragma unroll
+    for (int v = 0; v < 4; ++v)  // the lifting points out of the wall
+      gn[v] = o[4 + v] + (north ? 1.0 : -1.0) * so * cbr2 * (qc[v] - o[v]);
+    euler_fluxes(qc, a.gam, f, fi);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const double rm = sn * cbr2 * (qc[v] - m[v]);   // lifting of the (-) element
+      const double rp = -so * cbr2 * (qc[v] - o[v]);  // lifting of the (+) element
+      gn[v] = 0.5 * ((m[4 + v] + rm) + (o[4 + v] + rp));
+    }
+    rusanov2<false>(m, o, slot, a.gam, fi);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) fi[v] *= 0.5;
+  }
+  visc_normal(qc, gn, gt, slot, a, fv);
+  double* dst = a.fb + (north ? inner * 8 + (tid - inner) * 8 : tid * 8);
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     dst[v] = qc[v];
-    dst[4 + v] = fn[v];
+    dst[4 + v] = fi[v] - fv[v];
   }
 }
 
@@ -430,8 +530,7 @@ __global__ void __launch_bounds__(256) k_ns_cell(const NsArgs a) {
   constexpr int N = P + 1, NP = N * N, E = NsSlots<P>::E;
   constexpr bool PERTURB = MODE == 1 || MODE == 2;
   __shared__ double sq[E][4 * NP], dxi[E][4 * NP], deta[E][4 * NP];
-  __shared__ double cq[E][4][N][4];    // q_com on the own faces [W,E,S,N]
-  __shared__ double tq[E][4][N][4];    // own face traces of q
+  __shared__ double dq[E][4][N][4];    // q_com minus the own trace on the own faces [W,E,S,N]
   __shared__ double fnum[E][4][N][4];  // common total flux on the own faces
   __shared__ double sD[N][N], sDt[N][N], sdgL[N], sdgR[N];
   if (a.done && *a.done) return;
@@ -451,79 +550,74 @@ __global__ void __launch_bounds__(256) k_ns_cell(const NsArgs a) {
     eps = a.eps2[0];
     ieps = a.eps2[1];
   }
-  int ix = 0, iy = 0;
-  double hx = 1.0, hy = 1.0;
+  double sx = 0.0, sy = 0.0;
   if (active) {
-    ix = (int)(e % a.nx);
-    iy = (int)(e / a.nx);
-    hx = a.hx[ix];
-    hy = a.hy[iy];
+    const int ix = (int)(e % a.nx), iy = (int)(e / a.nx);
+    sx = a.sx[ix];
+    sy = a.sy[iy];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const long long o = e * 4 * NP + v * NP + t;
       sq[el][v * NP + t] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
     }
-    // own traces of q and the common data of the four faces
+    // the common data of the four faces: W, S own; E, N the neighbours' W, S (or the wall's)
     for (int fp = t; fp < 4 * N; fp += NP) {
       const int face = fp / N, k = fp % N;
-      const double* tr = a.tb + (((e * 4 + face) * N + k) * 4) * 3;
-      long long fe;
-      int fs;
-      if (face == 0) { fe = e; fs = 0; }
-      else if (face == 2) { fe = e; fs = 1; }
-      else if (face == 1) { fe = (long long)((ix + 1) % a.nx) + (long long)a.nx * iy; fs = 0; }
-      else if (a.wall_y && iy == a.ny - 1) { fe = e; fs = 2; }
-      else { fe = (long long)ix + (long long)a.nx * ((iy + 1) % a.ny); fs = 1; }
-      const double* fd = a.fb + ((fe * 3 + fs) * N + k) * 8;
+      long long fe = e * 2 + (face >> 1);
+      if (face == 1) fe = ((ix + 1) % a.nx + (long long)a.nx * iy) * 2;
+      else if (face == 3 && a.wall_y && iy == a.ny - 1) fe = a.ne * 2 + ix;
+      else if (face == 3) fe = (ix + (long long)a.nx * ((iy + 1) % a.ny)) * 2 + 1;
+      const double* fd = a.fb + (fe * N + k) * 8;
+      const double* tr = a.tb + ((e * 4 + face) * N + k) * 8;
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        tq[el][face][k][v] = tr[v * 3];
-        cq[el][face][k][v] = fd[v];
+        dq[el][face][k][v] = fd[v] - tr[v];
         fnum[el][face][k][v] = fd[4 + v];
       }
     }
   }
   __syncthreads();
   const int i = t % N, j = t / N;
+  // FR-corrected gradient and total flux at the own point
   if (active) {
+    double q[4], gx[4], gy[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
+      q[v] = sq[el][v * NP + t];
       double d1 = 0.0, d2 = 0.0;
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         d1 = fma(sD[i][k], sq[el][v * NP + k + N * j], d1);
         d2 = fma(sD[j][k], sq[el][v * NP + i + N * k], d2);
       }
-      dxi[el][v * NP + t] = d1;
-      deta[el][v * NP + t] = d2;
+      d1 = fma(dq[el][0][j][v], sdgL[i], d1);
+      d1 = fma(dq[el][1][j][v], sdgR[i], d1);
+      d2 = fma(dq[el][2][i][v], sdgL[j], d2);
+      d2 = fma(dq[el][3][i][v], sdgR[j], d2);
+      gx[v] = sx * d1;
+      gy[v] = sy * d2;
     }
-  }
-  __syncthreads();
-  const double sx = 2.0 / hx, sy = 2.0 / hy;
-  // corrected gradient and total flux at the own point (overwrites dxi / deta)
-  if (active) {
-    double q[4], gxv[4], gyv[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      q[v] = sq[el][v * NP + t];
-      double dx = dxi[el][v * NP + t];
-      dx = fma(cq[el][0][j][v] - tq[el][0][j][v], sdgL[i], dx);
-      dx = fma(cq[el][1][j][v] - tq[el][1][j][v], sdgR[i], dx);
-      double dy = deta[el][v * NP + t];
-      dy = fma(cq[el][2][i][v] - tq[el][2][i][v], sdgL[j], dy);
-      dy = fma(cq[el][3][i][v] - tq[el][3][i][v], sdgR[j], dy);
-      gxv[v] = sx * dx;
-      gyv[v] = sy * dy;
-    }
-    double f[4], g[4], fv[4], gv[4];
+    double f[4], g[4];
     euler_fluxes(q, a.gam, f, g);
-    visc_flux(q, gxv, gyv, a.gam, a.mu, a.kappa, fv, gv);
-    // each thread reads and overwrites only its own point
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      dxi[el][v * NP + t] = f[v] - fv[v];
-      deta[el][v * NP + t] = g[v] - gv[v];
-    }
+    const double rinv = 1.0 / q[0];  // the one of euler_fluxes
+    const double u = q[1] * rinv, w = q[2] * rinv, en = q[3] * rinv;
+    const double ux = fma(-u, gx[0], gx[1]) * rinv, wx = fma(-w, gx[0], gx[2]) * rinv;
+    const double uy = fma(-u, gy[0], gy[1]) * rinv, wy = fma(-w, gy[0], gy[2]) * rinv;
+    const double Tx = (a.gam - 1.0) * fma(-w, wx, fma(-u, ux, fma(-en, gx[0], gx[3]) * rinv));
+    const double Ty = (a.gam - 1.0) * fma(-w, wy, fma(-u, uy, fma(-en, gy[0], gy[3]) * rinv));
+    const double txx = a.mu * fma(4.0 / 3.0, ux, (-2.0 / 3.0) * wy);
+    const double tyy = a.mu * fma(4.0 / 3.0, wy, (-2.0 / 3.0) * ux);
+    const double txy = a.mu * (uy + wx);
+    double* F = dxi[el] + t;
+    double* G = deta[el] + t;
+    F[0] = f[0];
+    F[NP] = f[1] - txx;
+    F[2 * NP] = f[2] - txy;
+    F[3 * NP] = f[3] - fma(a.kappa, Tx, fma(w, txy, u * txx));
+    G[0] = g[0];
+    G[NP] = g[1] - txy;
+    G[2 * NP] = g[2] - tyy;
+    G[3 * NP] = g[3] - fma(a.kappa, Ty, fma(w, tyy, u * txy));
   }
   __syncthreads();
   if (!active) return;
@@ -558,6 +652,8 @@ NsArgs make_args(fr_ctx* ctx) {
   a.fb = ctx->fb;
   a.hx = ctx->hx;
   a.hy = ctx->hy;
+  a.sx = ctx->sx;
+  a.sy = ctx->sy;
   a.ne = ctx->ne;
   a.nx = ctx->nx;
   a.ny = ctx->ny;
@@ -574,41 +670,54 @@ NsArgs make_args(fr_ctx* ctx) {
 }
 
 template <int P>
-int ns_launch(fr_ctx* ctx, int mode, const NsArgs& a, bool perturb_trace, cudaStream_t s, double wb,
-              double wf) {
-  constexpr int NP = (P + 1) * (P + 1), E = NsSlots<P>::E, NB = 4 * NP;
+int ns_launch(fr_ctx* ctx, int mode, const NsArgs& a, cudaStream_t s, double wb, double wf) {
+  constexpr int NP = (P + 1) * (P + 1), E = NsSlots<P>::E;
   const unsigned gt = (unsigned)((ctx->ne + E - 1) / E);
-  const int fam = mode == 3 ? FR_KF_FACTOR : (mode == 0 ? FR_KF_RESIDUAL : FR_KF_JV);
-  {
-    ProfScope ps_(ctx, fam, s, wb, wf);  // one timed record for the trace + residual pair
-    if (perturb_trace) k_ns_trace<P, true><<<gt, E * NP, 0, s>>>(a);
-    else k_ns_trace<P, false><<<gt, E * NP, 0, s>>>(a);
-    FRK_LAUNCHED(ctx);
-    count_launch();  // the scope counted the trace kernel
-    if (mode == 3) {
-      k_ns_res<P, 3><<<(unsigned)((ctx->ne * NB + E - 1) / E), E * NP, 0, s>>>(a);
-    } else {
-      const long long nf = ctx->ne * 3 * (P + 1);
-      k_ns_face<P><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(a);
-      FRK_LAUNCHED(ctx);
-      count_launch();
-      if (mode == 0) k_ns_cell<P, 0><<<gt, E * NP, 0, s>>>(a);
-      else if (mode == 1) k_ns_cell<P, 1><<<gt, E * NP, 0, s>>>(a);
-      else k_ns_cell<P, 2><<<gt, E * NP, 0, s>>>(a);
-    }
-  }
+  ProfScope ps_(ctx, mode == 0 ? FR_KF_RESIDUAL : FR_KF_JV, s, wb, wf);  // one timed record for the three kernels
+  if (mode == 0) k_ns_trace<P, false><<<gt, E * NP, 0, s>>>(a);
+  else k_ns_trace<P, true><<<gt, E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();  // the scope counted the trace kernel
+  const long long nf = (ctx->ne * 2 + (a.wall_y ? ctx->nx : 0)) * (P + 1);
+  k_ns_face<P><<<(unsigned)((nf + FaceThreads<P>::value - 1) / FaceThreads<P>::value), FaceThreads<P>::value, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();
+  if (mode == 0) k_ns_cell<P, 0><<<gt, E * NP, 0, s>>>(a);
+  else if (mode == 1) k_ns_cell<P, 1><<<gt, E * NP, 0, s>>>(a);
+  else k_ns_cell<P, 2><<<gt, E * NP, 0, s>>>(a);
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }
 
-int dispatch(fr_ctx* ctx, int mode, const NsArgs& a, bool perturb_trace, cudaStream_t s, double wb,
-             double wf) {
+int dispatch(fr_ctx* ctx, int mode, const NsArgs& a, cudaStream_t s, double wb, double wf) {
   switch (ctx->p) {
-    case 2: return ns_launch<2>(ctx, mode, a, perturb_trace, s, wb, wf);
-    case 3: return ns_launch<3>(ctx, mode, a, perturb_trace, s, wb, wf);
-    case 4: return ns_launch<4>(ctx, mode, a, perturb_trace, s, wb, wf);
+    case 2: return ns_launch<2>(ctx, mode, a, s, wb, wf);
+    case 3: return ns_launch<3>(ctx, mode, a, s, wb, wf);
+    case 4: return ns_launch<4>(ctx, mode, a, s, wb, wf);
     default: return set_error(ctx, FR_ERR_UNSUPPORTED, "degree %d not compiled", ctx->p);
   }
+}
+
+// traces of U and its gradient, R(U) into ctx->rloc and the block columns into
+// ctx->mst, all by the operations of k_ns_res
+template <int P>
+int ns_columns(fr_ctx* ctx, NsArgs a, double shift, cudaStream_t s) {
+  constexpr int NP = (P + 1) * (P + 1), E = NsSlots<P>::E, NB = 4 * NP;
+  const unsigned gt = (unsigned)((ctx->ne + E - 1) / E);
+  ProfScope ps_(ctx, FR_KF_FACTOR, s);  // one timed record for the three kernels
+  k_ns_fulltrace<P><<<gt, E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();
+  a.out = ctx->rloc;
+  k_ns_res<P, 0><<<gt, E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();
+  a.R0 = ctx->rloc;
+  a.out = ctx->mst;
+  a.shift = shift;
+  k_ns_res<P, 3><<<(unsigned)((ctx->ne * NB + E - 1) / E), E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  return FR_OK;
 }
 
 }  // namespace
@@ -630,21 +739,18 @@ int launch_ns_residual(fr_ctx* ctx, int mode, const double* U, const double* z, 
   const bool in_cycle = done != nullptr;
   const double wb = in_cycle ? 0.0 : (mode == 0 ? 16.0 : (mode == 1 ? 32.0 : 40.0)) * nd;
   const double wf = in_cycle ? 0.0 : ns_residual_flops_per_element(ctx->p) * (double)ctx->ne + (mode == 0 ? 0.0 : 6.0 * nd);
-  return dispatch(ctx, mode, a, mode != 0, s, wb, wf);
+  return dispatch(ctx, mode, a, s, wb, wf);
 }
 
 int launch_ns_factor(fr_ctx* ctx, const double* U, double shift, cudaStream_t s) {
-  // R0 of the element-local residuals = R(U) with the same (unperturbed) traces
   NsArgs a = make_args(ctx);
   a.U = U;
-  a.z = nullptr;
-  a.out = ctx->rloc;
-  a.shift = 0.0;
-  FRK_TRY(dispatch(ctx, 0, a, false, s, 0.0, 0.0));
-  a.R0 = ctx->rloc;
-  a.out = ctx->mst;
-  a.shift = shift;
-  FRK_TRY(dispatch(ctx, 3, a, false, s, 0.0, 0.0));
+  switch (ctx->p) {
+    case 2: FRK_TRY(ns_columns<2>(ctx, a, shift, s)); break;
+    case 3: FRK_TRY(ns_columns<3>(ctx, a, shift, s)); break;
+    case 4: FRK_TRY(ns_columns<4>(ctx, a, shift, s)); break;
+    default: return set_error(ctx, FR_ERR_UNSUPPORTED, "degree %d not compiled", ctx->p);
+  }
   return launch_block_invert(ctx, ctx->mst, 0.0, s);
 }
 

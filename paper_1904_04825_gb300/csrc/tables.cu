@@ -69,6 +69,12 @@ void build_tables(int p, Tables* t) {
     }
     D[i][i] = diag;
   }
+  // l_k'(+-1): the degree-(n-1) derivative interpolated at the element ends
+  for (int k = 0; k < n; ++k)
+    for (int i = 0; i < n; ++i) {
+      t->dlm[k] += t->lm[i] * D[i][k];
+      t->dlp[k] += t->lp[i] * D[i][k];
+    }
   // Radau corrections: g_L = (-1)^n/2 (P_n - P_{n-1}), g_R = (P_n + P_{n-1})/2
   const double sgn = (n % 2 == 0) ? 1.0 : -1.0;
   for (int i = 0; i < n; ++i) {
