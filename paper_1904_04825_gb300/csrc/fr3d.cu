@@ -9,19 +9,25 @@
 // the two other directions in increasing order.
 //
 // R(U), A z and b - A z take three kernels, like the 2D viscous path:
-//  k3_trace: per element, the (possibly perturbed) state and its own
-//    polynomial gradient traced to the 6 N^2 face points -> trace buffer
-//    [ne][6][N^2][5][4] = (q, q_x, q_y, q_z).
-//  k3_face:  per low face point of every element (each face once), the
-//    common solution, BR2 common gradient and common total normal flux
-//    (Rusanov inviscid minus viscous) from the two traces -> face buffer
-//    [ne][3][N^2][10] = (q_com, f_n).
+//  k3_trace: per element, the (possibly perturbed) state q and its normal
+//    derivative traced to the 6 N^2 face points -> trace buffer
+//    [ne][6][N^2][q 5, q_n 5].  The normal derivative comes straight from q
+//    (rows l_k'(+-1)); the tangential ones are derivatives along the face of
+//    the common solution, which k3_face takes once for both elements.
+//  k3_face:  per low face point of every element (each face once), the half
+//    jump of q (q_com minus either trace, up to sign), the BR2 common gradient
+//    and the common total normal flux (Rusanov inviscid minus viscous) -> face
+//    buffer [ne][3][N^2][half jump 5, f_n 5].
 //  k3_cell:  per element, the FR-corrected gradient, the total fluxes along
 //    x, y, z at the solution points and their corrected divergence with the
 //    six faces' common fluxes (low faces its own, high faces the neighbours'
 //    low faces), then the output of the mode.  Both elements of a face read
 //    the same stored flux, so conservation holds to round-off.
-// Element-Jacobi columns (k3_cell mode 3, degrees 1 to 3): slot = (element,
+// Bound: FP64 issue.  R + A z at 32^3, p = 3: 4.03 ms; 6.15 ms when k3_trace
+// differentiated the element and traced the whole gradient (twice the trace
+// buffer), k3_cell traced q again, and divisions and roots were IEEE.
+// Element-Jacobi columns (k3_cols, degrees 1 to 3) follow k3_fulltrace, which
+// traces q and its whole gradient [ne][6][N^2][5][4]: slot = (element,
 // column c), own state perturbed in DOF c by eps_c = beps (1 + |q_c|), own
 // traces recomputed in the kernel, neighbour traces frozen (trace buffer of
 // the unperturbed state); the slot forms its six faces' common data itself
@@ -39,16 +45,20 @@ struct F3Args {
   const double* R0;
   const double* b;
   double* out;
-  double* tb;          // traces [ne][6][N^2][5][4]
-  double* fb;          // low-face common data [ne][3][N^2][10]
+  double* tb;          // traces [ne][6][N^2][10], for the blocks and caches [ne][6][N^2][5][4]
+  double* fb;          // low-face data [ne][3][N^2][10]
   const double* hx;
   const double* hy;
   const double* hz;
+  const double* sx;    // 2 / hx, 2 / hy, 2 / hz
+  const double* sy;
+  const double* sz;
   const double* eps2;
   const int* done;
   long long ne;
   long long e0, nchunk;  // mode 3: the elements e0 .. e0 + nchunk - 1, columns staged from out[0]
   float* r0f;            // mode 3 in FP32: element-local R(U) of the chunk, [nchunk][NB]
+  double* r0d;           // mode 3 in FP64: the same
   const float* tbf;      // mode 3 in FP32: the trace buffer in FP32
   // A z with FP32 linear parts (jv_precision 1): caches at the linearisation
   // point U and the FP32 buffers of the product
@@ -59,8 +69,7 @@ struct F3Args {
   float* tbz;            // traces of z and of its gradient [ne][6][N^2][20]
   float* fbz;            // per unit eps: q_com differences and f_n differences [ne][3][N^2][10]
   double* lgc;           // BR2 common gradient of U at the low-face points [ne][3][N^2][15]
-  int write_gc;          // cache pass: k3_face writes lgc
-  int r0_pass;           // mode 3 in FP32: 1 = write r0f (one unperturbed slot per element)
+  int r0_pass;           // mode 3: 1 = write the element-local R(U) (one unperturbed slot per element)
   int nx, ny, nz;
   double gam, mu, kappa, shift, beps;
   Tables tab;
@@ -248,8 +257,9 @@ __device__ __forceinline__ void own_trace(const T* sq, const T* d0, const T* d1,
   }
 }
 
-template <int P, bool PERTURB>
-__global__ void __launch_bounds__(256) k3_trace(const F3Args a) {
+// q and its gradient of the unperturbed state at the face points
+template <int P>
+__global__ void __launch_bounds__(256) k3_fulltrace(const F3Args a) {
   constexpr int N = P + 1, N2 = N * N, NP = N2 * N, E = F3Slots<P>::E;
   __shared__ double sq[E][5 * NP], dd[3][E][5 * NP];
   __shared__ double sD[N][N], slm[N], slp[N];
@@ -258,16 +268,14 @@ __global__ void __launch_bounds__(256) k3_trace(const F3Args a) {
     slm[threadIdx.x] = a.tab.lm[threadIdx.x];
     slp[threadIdx.x] = a.tab.lp[threadIdx.x];
   }
-  if (a.done && *a.done) return;
   const int el = threadIdx.x / NP, t = threadIdx.x % NP;
   const long long e = (long long)blockIdx.x * E + el;
   const bool active = el < E && e < a.ne;
-  const double eps = PERTURB ? a.eps2[0] : 0.0;
   if (active) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const long long o = e * 5 * NP + v * NP + t;
-      sq[el][v * NP + t] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+      sq[el][v * NP + t] = a.U[o];
     }
   }
   __syncthreads();
@@ -276,7 +284,7 @@ __global__ void __launch_bounds__(256) k3_trace(const F3Args a) {
   if (!active) return;
   int ix, iy, iz;
   coords(e, a, &ix, &iy, &iz);
-  const double s[3] = {2.0 / a.hx[ix], 2.0 / a.hy[iy], 2.0 / a.hz[iz]};
+  const double s[3] = {a.sx[ix], a.sy[iy], a.sz[iz]};
   for (int fp = t; fp < 6 * N2; fp += NP) {
     const int face = fp / N2, f = fp % N2;
     double o[5][4];
@@ -289,12 +297,12 @@ __global__ void __launch_bounds__(256) k3_trace(const F3Args a) {
   }
 }
 
-// one thread per (element, direction d, point of its low face d)
+// Caches of the A z with FP32 linear parts: q_com, f_n and the BR2 common gradient
+// at U, one thread per (element, direction d, point of its low face d)
 template <int P>
-__global__ void __launch_bounds__(256) k3_face(const F3Args a) {
+__global__ void __launch_bounds__(256) k3_face_cache(const F3Args a) {
   constexpr int N = P + 1, N2 = N * N;
   constexpr double cbr2 = (P + 1) * (P + 2) / 2.0;
-  if (a.done && *a.done) return;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= a.ne * 3 * N2) return;
   const int f = (int)(tid % N2);
@@ -316,44 +324,40 @@ __global__ void __launch_bounds__(256) k3_face(const F3Args a) {
       pp[v][c] = own[v * 4 + c];
     }
   double gc[3][5];
-  common3(m, pp, d, hm, hp, cbr2, a, qc, fn, a.write_gc ? gc : nullptr);
+  common3(m, pp, d, hm, hp, cbr2, a, qc, fn, gc);
   double* dst = a.fb + ((e * 3 + d) * N2 + f) * 10;
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     dst[v] = qc[v];
     dst[5 + v] = fn[v];
   }
-  if (a.write_gc) {  // cache pass of the FP32-linear-parts A z: the common gradient at U
-    double* g = a.lgc + ((e * 3 + d) * N2 + f) * 15;
+  double* g = a.lgc + ((e * 3 + d) * N2 + f) * 15;
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+  for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int v = 0; v < 5; ++v) g[c * 5 + v] = gc[c][v];
-  }
+    for (int v = 0; v < 5; ++v) g[c * 5 + v] = gc[c][v];
 }
 
-// MODE 0: out = R(U); 1: out = A z; 2: out = b - A z (state U + eps z, face
-// data from the face buffer); 3: element-Jacobi column (see the file header);
-// 4: the caches of the FP32-linear-parts A z at U (corrected gradient and
-// total fluxes at the points to a.lg, a.lf; face data from the face buffer).
+// MODE 3: element-Jacobi column (see the file header); 4: the caches of the
+// FP32-linear-parts A z at U (corrected gradient and total fluxes at the
+// points to a.lg, a.lf; face data from the face buffer).
 // T: arithmetic type, double except for FP32 element-Jacobi columns (MODE 3,
-// T = float): then a first pass (a.r0_pass) writes the element-local R(U) of
-// each element of the chunk in FP32 to a.r0f, and the columns pass divides
-// R(U + eps_c e_c) - r0f by the step actually taken in FP32.
+// T = float).  A first pass of MODE 3 (a.r0_pass) writes the element-local
+// R(U) of each element of the chunk by the same operations to a.r0d (FP32:
+// a.r0f); the columns pass divides R(U + eps_c e_c) minus that by eps_c (FP32:
+// by the step actually taken).
 template <int P, int MODE, typename T = double>
-__global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
+__global__ void __launch_bounds__(256) k3_cols(const F3Args a) {
   using L = CellLayout<P, T>;
   constexpr int N = P + 1, N2 = N * N, NP = N2 * N, E = F3Slots<P>::E, NB = 5 * NP;
-  constexpr bool PERTURB = MODE == 1 || MODE == 2;
   constexpr bool JAC = MODE == 3;
   constexpr bool J32 = JAC && sizeof(T) == 4;
-  static_assert(sizeof(T) == 8 || JAC, "R(U) and A z run in FP64");
+  static_assert(JAC || (MODE == 4 && sizeof(T) == 8), "columns, or the FP64 caches");
   constexpr T cbr2 = T((P + 1) * (P + 2) / 2.0);
   extern __shared__ __align__(16) unsigned char smem3_raw[];
   T* smem3 = reinterpret_cast<T*>(smem3_raw);
   __shared__ T sD[N][N], sDt[N][N], slm[N], slp[N], sdgL[N], sdgR[N];
   __shared__ float sceps[E];  // FP32 columns: the step each slot took
-  if (a.done && *a.done) return;
   if (threadIdx.x < N * N) {
     sD[threadIdx.x / N][threadIdx.x % N] = (T)a.tab.D[threadIdx.x / N][threadIdx.x % N];
     sDt[threadIdx.x / N][threadIdx.x % N] = (T)a.tab.Dt[threadIdx.x / N][threadIdx.x % N];
@@ -372,17 +376,12 @@ __global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
   T* d2 = d1 + 5 * NP;
   T* dq = d2 + 5 * NP;          // [6][N2][5] q_com - q_face
   T* fn = dq + 30 * N2;         // [6][N2][5] common total normal flux
-  const bool r0_pass = J32 && a.r0_pass;
+  const bool r0_pass = JAC && a.r0_pass;
   const long long slot = (long long)blockIdx.x * E + el;
   const long long nslots = JAC ? (r0_pass ? a.nchunk : a.nchunk * NB) : a.ne;
   const bool active = el < E && slot < nslots;
   const long long e = JAC ? a.e0 + (r0_pass ? slot : slot / NB) : slot;
   const int col = JAC && !r0_pass ? (int)(slot % NB) : -1;
-  double eps = 0.0, ieps = 0.0;
-  if (PERTURB) {
-    eps = a.eps2[0];
-    ieps = a.eps2[1];
-  }
   int ix = 0, iy = 0, iz = 0;
   T s[3] = {T(1), T(1), T(1)}, hown[3] = {T(1), T(1), T(1)};
   double ceps = 0.0;  // FD step of the column (FP32: the step taken after rounding)
@@ -392,7 +391,7 @@ __global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
     hown[1] = (T)a.hy[iy];
     hown[2] = (T)a.hz[iz];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) s[c] = T(2) / hown[c];
+    for (int c = 0; c < 3; ++c) s[c] = J32 ? T(2) / hown[c] : (T)(c == 0 ? a.sx[ix] : (c == 1 ? a.sy[iy] : a.sz[iz]));
     if (JAC && !J32 && col >= 0) {
       const double uc = a.U[e * NB + col];
       ceps = a.beps * (1.0 + fabs(uc));
@@ -400,7 +399,7 @@ __global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const long long o = e * NB + v * NP + t;
-      double qv = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+      double qv = a.U[o];
       if (JAC && !J32 && v * NP + t == col) qv += ceps;
       T tq = (T)qv;
       if (J32 && v * NP + t == col) {
@@ -527,24 +526,341 @@ __global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
       dH = fma(sDt[k][l], H[i + N * j + N2 * l], dH);
     }
     const T R = -fma(s[0], dF, fma(s[1], dG, s[2] * dH));
-    const long long o = e * NB + v * NP + t;
-    if (MODE == 0) {
-      a.out[o] = (double)R;
-    } else if (MODE == 3) {
-      // column col of M = shift I - J_ee, staged column-major [col][row]
-      const int row = v * NP + t;
+    // column col of M = shift I - J_ee, staged column-major [col][row]
+    const int row = v * NP + t;
+    const long long ro = (e - a.e0) * NB + row;
+    if (r0_pass) {
+      if (J32) a.r0f[ro] = (float)R;
+      else a.r0d[ro] = (double)R;
+    } else {
       double* dst = a.out + ((e - a.e0) * NB + col) * NB + row;
-      if (r0_pass) {
-        a.r0f[(e - a.e0) * NB + row] = (float)R;
-      } else if (J32) {  // the difference quotient and the column in FP32
-        const float dq32 = ((float)R - a.r0f[(e - a.e0) * NB + row]) / ceps32;
+      if (J32) {  // the difference quotient and the column in FP32
+        const float dq32 = ((float)R - a.r0f[ro]) / ceps32;
         *dst = (double)((row == col ? (float)a.shift : 0.f) - dq32);
       } else {
-        *dst = (row == col ? a.shift : 0.0) - ((double)R - a.R0[o]) / ceps;
+        *dst = (row == col ? a.shift : 0.0) - ((double)R - a.r0d[ro]) / ceps;
       }
+    }
+  }
+}
+
+// ---- R(U), A z and b - A z in FP64 ----
+
+// q and its normal derivative at the face points; work items over the CTA's E
+// elements x 6 N^2 points
+template <int P, bool PERTURB>
+__global__ void __launch_bounds__(256) k3_trace(const F3Args a) {
+  constexpr int N = P + 1, N2 = N * N, NP = N2 * N, E = F3Slots<P>::E, NB = 5 * NP;
+  __shared__ double sq[E][NB];
+  __shared__ double sl[2][N], sd[2][N];  // l_k(-+1), l_k'(-+1)
+  if (a.done && *a.done) return;
+  if (threadIdx.x < N) {
+    sl[0][threadIdx.x] = a.tab.lm[threadIdx.x];
+    sl[1][threadIdx.x] = a.tab.lp[threadIdx.x];
+    sd[0][threadIdx.x] = a.tab.dlm[threadIdx.x];
+    sd[1][threadIdx.x] = a.tab.dlp[threadIdx.x];
+  }
+  const long long e0 = (long long)blockIdx.x * E;
+  const int ne = a.ne - e0 < E ? (int)(a.ne - e0) : E;
+  const double eps = PERTURB ? a.eps2[0] : 0.0;
+  for (int i = threadIdx.x; i < ne * NB; i += blockDim.x) {
+    const long long o = e0 * NB + i;
+    sq[0][i] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * 6 * N2; i += blockDim.x) {
+    const int el = i / (6 * N2), face = (i / N2) % 6, f = i % N2, d = face >> 1;
+    const long long e = e0 + el;
+    int ix, iy, iz, off, stride;
+    coords(e, a, &ix, &iy, &iz);
+    const double s = d == 0 ? a.sx[ix] : (d == 1 ? a.sy[iy] : a.sz[iz]);
+    line_of<N>(d, f, &off, &stride);
+    double* dst = a.tb + ((e * 6 + face) * N2 + f) * 10;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double* x = sq[el] + v * NP + off;
+      dst[v] = tsum3<N>(x, stride, sl[face & 1]);
+      dst[5 + v] = s * tsum3<N>(x, stride, sd[face & 1]);
+    }
+  }
+}
+
+// Viscous flux along direction d from the common state and its gradient g[c][v]
+// (c: direction), R = 1.
+__device__ __forceinline__ void visc3_normal(const double q[5], const double g[3][5], int d, const F3Args& a,
+                                             double fv[5]) {
+  const double ri = rcp_fast(q[0]);
+  const double vel[3] = {q[1] * ri, q[2] * ri, q[3] * ri};
+  const double e = q[4] * ri;
+  double gd[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) gd[v] = d == 0 ? g[0][v] : (d == 1 ? g[1][v] : g[2][v]);
+  double dvd[3], dd[3], vdc[3];  // d v_m / d x_d, d v_c / d x_c, d v_d / d x_c
+  const double vd = d == 0 ? vel[0] : (d == 1 ? vel[1] : vel[2]);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    dvd[m] = fma(-vel[m], gd[0], gd[1 + m]) * ri;
+    dd[m] = fma(-vel[m], g[m][0], g[m][1 + m]) * ri;
+    vdc[m] = fma(-vd, g[m][0], d == 0 ? g[m][1] : (d == 1 ? g[m][2] : g[m][3])) * ri;
+  }
+  const double dT = (a.gam - 1.0) *
+                    fma(-vel[2], dvd[2], fma(-vel[1], dvd[1], fma(-vel[0], dvd[0], fma(-e, gd[0], gd[4]) * ri)));
+  const double div = dd[0] + dd[1] + dd[2];
+  double w = a.kappa * dT;
+  fv[0] = 0.0;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    double t = dvd[m] + vdc[m];
+    if (m == d) t = fma(-2.0 / 3.0, div, t);
+    fv[1 + m] = a.mu * t;
+    w = fma(vel[m], fv[1 + m], w);
+  }
+  fv[4] = w;
+}
+
+// inviscid flux along d and |v_d| + c, with 1/rho and the pressure given
+__device__ __forceinline__ void flux3_of(const double q[5], int d, double ri, double p, double f[5]) {
+  const double md = d == 0 ? q[1] : (d == 1 ? q[2] : q[3]);
+  const double vd = md * ri;
+  f[0] = md;
+  f[1] = fma(q[1], vd, d == 0 ? p : 0.0);
+  f[2] = fma(q[2], vd, d == 1 ? p : 0.0);
+  f[3] = fma(q[3], vd, d == 2 ? p : 0.0);
+  f[4] = vd * (q[4] + p);
+}
+__device__ __forceinline__ double pressure3(const double q[5], double ri, double gam) {
+  return (gam - 1.0) * (q[4] - 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * ri);
+}
+
+// threads of k3_face: whole faces of N^2 points per CTA
+template <int P> struct Face3Threads { static constexpr int value = 256 / ((P + 1) * (P + 1)) * (P + 1) * (P + 1); };
+
+// one thread per (element, direction d, point of its low face d); the N^2
+// threads of a face exchange its common solution in shared memory for the
+// tangential derivatives
+template <int P>
+__global__ void __launch_bounds__(256) k3_face(const F3Args a) {
+  constexpr int N = P + 1, N2 = N * N, T = Face3Threads<P>::value;
+  constexpr double cbr2 = (P + 1) * (P + 2) / 2.0;
+  __shared__ double sD[N][N], sc[5][T];
+  if (a.done && *a.done) return;
+  if (threadIdx.x < N * N) sD[threadIdx.x / N][threadIdx.x % N] = a.tab.D[threadIdx.x / N][threadIdx.x % N];
+  const long long tid = (long long)blockIdx.x * T + threadIdx.x;
+  const bool active = tid < a.ne * 3 * N2;
+  const int f = threadIdx.x % N2;
+  const int d = (int)((tid / N2) % 3);
+  const long long e = tid / (3 * N2);
+  double m[10], o[10], qc[5];
+  double s[3] = {}, sm = 0.0;
+  if (active) {
+    int ix, iy, iz;
+    coords(e, a, &ix, &iy, &iz);
+    s[0] = a.sx[ix];
+    s[1] = a.sy[iy];
+    s[2] = a.sz[iz];
+    const int jx = d == 0 ? (ix + a.nx - 1) % a.nx : ix, jy = d == 1 ? (iy + a.ny - 1) % a.ny : iy,
+              jz = d == 2 ? (iz + a.nz - 1) % a.nz : iz;
+    sm = d == 0 ? a.sx[jx] : (d == 1 ? a.sy[jy] : a.sz[jz]);
+    const double2* own = reinterpret_cast<const double2*>(a.tb + ((e * 6 + 2 * d) * N2 + f) * 10);
+    const double2* nb = reinterpret_cast<const double2*>(a.tb + ((elem(jx, jy, jz, a) * 6 + 2 * d + 1) * N2 + f) * 10);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double2 x = own[v], y = nb[v];
+      o[2 * v] = x.x;
+      o[2 * v + 1] = x.y;
+      m[2 * v] = y.x;
+      m[2 * v + 1] = y.y;
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) sc[v][threadIdx.x] = qc[v] = 0.5 * (m[v] + o[v]);
+  }
+  __syncthreads();
+  if (!active) return;
+  const double sd = d == 0 ? s[0] : (d == 1 ? s[1] : s[2]);
+  const double st1 = d == 0 ? s[1] : s[0], st2 = d == 2 ? s[1] : s[2];  // the two other directions, in order
+  const double lift = 0.5 * cbr2 * (sm + sd);  // both BR2 liftings act on the jump
+  const int f1 = f % N, f2 = f / N;
+  double g[3][5], hj[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const double* x = &sc[v][threadIdx.x - f];
+    double t1 = sD[f1][0] * x[N * f2], t2 = sD[f2][0] * x[f1];
+#pragma unroll
+    for (int l = 1; l < N; ++l) {
+      t1 = fma(sD[f1][l], x[l + N * f2], t1);
+      t2 = fma(sD[f2][l], x[f1 + N * l], t2);
+    }
+    t1 *= st1;
+    t2 *= st2;
+    const double j = o[v] - m[v];
+    hj[v] = 0.5 * j;
+    const double gn = 0.5 * fma(lift, j, m[5 + v] + o[5 + v]);
+    g[0][v] = d == 0 ? gn : t1;
+    g[1][v] = d == 1 ? gn : (d == 0 ? t1 : t2);
+    g[2][v] = d == 2 ? gn : t2;
+  }
+  double fn[5], fv[5];
+  {
+    double fm[5], fp[5];
+    const double rm = rcp_fast(m[0]), rp = rcp_fast(o[0]);
+    const double pm = pressure3(m, rm, a.gam), pp = pressure3(o, rp, a.gam);
+    flux3_of(m, d, rm, pm, fm);
+    flux3_of(o, d, rp, pp, fp);
+    const double lam = max_nonneg(fabs(fm[0] * rm) + sqrt_fast(a.gam * pm * rm),
+                                  fabs(fp[0] * rp) + sqrt_fast(a.gam * pp * rp));
+#pragma unroll
+    for (int v = 0; v < 5; ++v) fn[v] = fma(-lam, o[v] - m[v], fm[v] + fp[v]);
+  }
+  visc3_normal(qc, g, d, a, fv);
+  double2* dst = reinterpret_cast<double2*>(a.fb + ((e * 3 + d) * N2 + f) * 10);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) fn[v] = fma(0.5, fn[v], -fv[v]);
+  dst[0] = make_double2(hj[0], hj[1]);
+  dst[1] = make_double2(hj[2], hj[3]);
+  dst[2] = make_double2(hj[4], fn[0]);
+  dst[3] = make_double2(fn[1], fn[2]);
+  dst[4] = make_double2(fn[3], fn[4]);
+}
+
+// MODE 0: out = R(U); 1: out = A z; 2: out = b - A z (state U + eps z)
+template <int P, int MODE>
+__global__ void __launch_bounds__(256) k3_cell(const F3Args a) {
+  using L = CellLayout<P>;
+  constexpr int N = P + 1, N2 = N * N, NP = N2 * N, E = F3Slots<P>::E, NB = 5 * NP;
+  constexpr bool PERTURB = MODE != 0;
+  extern __shared__ __align__(16) unsigned char smem3_raw[];
+  double* smem3 = reinterpret_cast<double*>(smem3_raw);
+  __shared__ double sD[N][N], sDt[N][N], sdgL[N], sdgR[N];
+  if (a.done && *a.done) return;
+  if (threadIdx.x < N * N) {
+    sD[threadIdx.x / N][threadIdx.x % N] = a.tab.D[threadIdx.x / N][threadIdx.x % N];
+    sDt[threadIdx.x / N][threadIdx.x % N] = a.tab.Dt[threadIdx.x / N][threadIdx.x % N];
+  }
+  if (threadIdx.x < N) {
+    sdgL[threadIdx.x] = a.tab.dgL[threadIdx.x];
+    sdgR[threadIdx.x] = a.tab.dgR[threadIdx.x];
+  }
+  const int el = threadIdx.x / NP, t = threadIdx.x % NP;
+  double* sq = smem3 + (size_t)(el < E ? el : 0) * L::PER;  // [5][NP]
+  double* d0 = sq + 5 * NP;          // total fluxes along x / y / z
+  double* d1 = d0 + 5 * NP;
+  double* d2 = d1 + 5 * NP;
+  double* dq = d2 + 5 * NP;          // [6][N2][5] stored half jumps
+  double* fn = dq + 30 * N2;         // [6][N2][5] common total normal flux
+  const long long e = (long long)blockIdx.x * E + el;
+  const bool active = el < E && e < a.ne;
+  double eps = 0.0, ieps = 0.0;
+  if (PERTURB) {
+    eps = a.eps2[0];
+    ieps = a.eps2[1];
+  }
+  double s[3] = {};
+  if (active) {
+    int ix, iy, iz;
+    coords(e, a, &ix, &iy, &iz);
+    s[0] = a.sx[ix];
+    s[1] = a.sy[iy];
+    s[2] = a.sz[iz];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const long long o = e * NB + v * NP + t;
+      sq[v * NP + t] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
+    }
+    for (int fp = t; fp < 6 * N2; fp += NP) {
+      const int face = fp / N2, f = fp % N2, d = face >> 1;
+      long long fe = e;
+      if (face & 1)
+        fe = elem(d == 0 ? (ix + 1) % a.nx : ix, d == 1 ? (iy + 1) % a.ny : iy, d == 2 ? (iz + 1) % a.nz : iz, a);
+      const double2* src = reinterpret_cast<const double2*>(a.fb + ((fe * 3 + d) * N2 + f) * 10);
+      const double2 x0 = src[0], x1 = src[1], x2 = src[2], x3 = src[3], x4 = src[4];
+      double* q5 = dq + fp * 5;
+      double* f5 = fn + fp * 5;
+      q5[0] = x0.x; q5[1] = x0.y; q5[2] = x1.x; q5[3] = x1.y; q5[4] = x2.x;
+      f5[0] = x2.y; f5[1] = x3.x; f5[2] = x3.y; f5[3] = x4.x; f5[4] = x4.y;
+    }
+  }
+  __syncthreads();
+  const int i = t % N, j = (t / N) % N, k = t / N2;
+  const int f0 = j + N * k, f1 = i + N * k, f2 = i + N * j;  // this point's face points per direction
+  // corrected gradient and total fluxes at the own point
+  if (active) {
+    double q[5], g[3][5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double* x = sq + v * NP;
+      q[v] = x[t];
+      double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) {
+        a0 = fma(sD[i][l], x[l + N * j + N2 * k], a0);
+        a1 = fma(sD[j][l], x[i + N * l + N2 * k], a1);
+        a2 = fma(sD[k][l], x[i + N * j + N2 * l], a2);
+      }
+      // the stored half jump is q_com - q on a high face, its negative on a low one
+      a0 = fma(-dq[(0 * N2 + f0) * 5 + v], sdgL[i], a0);
+      a0 = fma(dq[(1 * N2 + f0) * 5 + v], sdgR[i], a0);
+      a1 = fma(-dq[(2 * N2 + f1) * 5 + v], sdgL[j], a1);
+      a1 = fma(dq[(3 * N2 + f1) * 5 + v], sdgR[j], a1);
+      a2 = fma(-dq[(4 * N2 + f2) * 5 + v], sdgL[k], a2);
+      a2 = fma(dq[(5 * N2 + f2) * 5 + v], sdgR[k], a2);
+      g[0][v] = s[0] * a0;
+      g[1][v] = s[1] * a1;
+      g[2][v] = s[2] * a2;
+    }
+    const double ri = rcp_fast(q[0]), pr = pressure3(q, ri, a.gam);
+    const double vel[3] = {q[1] * ri, q[2] * ri, q[3] * ri}, en = q[4] * ri;
+    double dv[3][3], dT[3];  // dv[c][m] = d v_m / d x_c
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) dv[c][m] = fma(-vel[m], g[c][0], g[c][1 + m]) * ri;
+      dT[c] = (a.gam - 1.0) * fma(-vel[2], dv[c][2], fma(-vel[1], dv[c][1],
+                                  fma(-vel[0], dv[c][0], fma(-en, g[c][0], g[c][4]) * ri)));
+    }
+    const double div = dv[0][0] + dv[1][1] + dv[2][2];
+    double* dst[3] = {d0, d1, d2};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      double fi[5], w = a.kappa * dT[d];
+      flux3_of(q, d, ri, pr, fi);
+      dst[d][t] = fi[0];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        double tau = dv[d][m] + dv[m][d];
+        if (m == d) tau = fma(-2.0 / 3.0, div, tau);
+        tau *= a.mu;
+        w = fma(vel[m], tau, w);
+        dst[d][(1 + m) * NP + t] = fi[1 + m] - tau;
+      }
+      dst[d][4 * NP + t] = fi[4] - w;
+    }
+  }
+  __syncthreads();
+  if (!active) return;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const double* F = d0 + v * NP;
+    const double* G = d1 + v * NP;
+    const double* H = d2 + v * NP;
+    double dF = sdgL[i] * fn[(0 * N2 + f0) * 5 + v];
+    dF = fma(sdgR[i], fn[(1 * N2 + f0) * 5 + v], dF);
+    double dG = sdgL[j] * fn[(2 * N2 + f1) * 5 + v];
+    dG = fma(sdgR[j], fn[(3 * N2 + f1) * 5 + v], dG);
+    double dH = sdgL[k] * fn[(4 * N2 + f2) * 5 + v];
+    dH = fma(sdgR[k], fn[(5 * N2 + f2) * 5 + v], dH);
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+      dF = fma(sDt[i][l], F[l + N * j + N2 * k], dF);
+      dG = fma(sDt[j][l], G[i + N * l + N2 * k], dG);
+      dH = fma(sDt[k][l], H[i + N * j + N2 * l], dH);
+    }
+    const double R = -fma(s[0], dF, fma(s[1], dG, s[2] * dH));
+    const long long o = e * NB + v * NP + t;
+    if (MODE == 0) {
+      a.out[o] = R;
     } else {
       const double zo = a.z[o];
-      const double Az = eps > 0.0 ? fma(-((double)R - a.R0[o]), ieps, a.shift * zo) : a.shift * zo;
+      const double Az = eps > 0.0 ? fma(-(R - a.R0[o]), ieps, a.shift * zo) : a.shift * zo;
       a.out[o] = MODE == 2 ? a.b[o] - Az : Az;
     }
   }
@@ -873,10 +1189,14 @@ F3Args make_args3(fr_ctx* ctx) {
   a.hx = ctx->hx;
   a.hy = ctx->hy;
   a.hz = ctx->hz;
+  a.sx = ctx->sx;
+  a.sy = ctx->sy;
+  a.sz = ctx->sz;
   a.ne = ctx->ne;
   a.e0 = 0;
   a.nchunk = ctx->ne;
   a.r0f = nullptr;
+  a.r0d = nullptr;
   a.tbf = nullptr;
   a.r0_pass = 0;
   a.ltb = ctx->lin3_tb;
@@ -886,7 +1206,6 @@ F3Args make_args3(fr_ctx* ctx) {
   a.tbz = ctx->lin3_tbz;
   a.fbz = ctx->lin3_fbz;
   a.lgc = ctx->lin3_gc;
-  a.write_gc = 0;
   a.nx = ctx->nx;
   a.ny = ctx->ny;
   a.nz = ctx->nz;
@@ -900,20 +1219,19 @@ F3Args make_args3(fr_ctx* ctx) {
 }
 
 template <int P>
-int f3_launch(fr_ctx* ctx, int mode, const F3Args& a, bool perturb_trace, cudaStream_t s, double wb,
-              double wf) {
+int f3_launch(fr_ctx* ctx, int mode, const F3Args& a, cudaStream_t s, double wb, double wf) {
   using L = CellLayout<P>;
-  constexpr int NP = L::NP, N2 = L::N2, E = F3Slots<P>::E, NB = 5 * NP;
+  constexpr int NP = L::NP, N2 = L::N2, E = F3Slots<P>::E;
   static bool attr = false;  // dynamic shared memory above 48 KB, set once per process
   if (!attr) {
     FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
     FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
     FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
-    FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
     attr = true;
   }
   const unsigned gt = (unsigned)((ctx->ne + E - 1) / E);
-  const int fam = mode == 3 ? FR_KF_FACTOR : (mode == 0 ? FR_KF_RESIDUAL : FR_KF_JV);
+  const int fam = mode == 0 ? FR_KF_RESIDUAL : FR_KF_JV;
+  const long long nf = ctx->ne * 3 * N2;
   if ((mode == 1 || mode == 2) && ctx->opts.jv_precision == 1) {
     // A z with FP32 linear parts: FP32 traces of z, face differences, cell
     using LZ = CellLayout<P, float>;
@@ -928,7 +1246,6 @@ int f3_launch(fr_ctx* ctx, int mode, const F3Args& a, bool perturb_trace, cudaSt
     k3z_trace<P><<<gt, E * NP, 0, s>>>(a);
     FRK_LAUNCHED(ctx);
     count_launch();
-    const long long nf = ctx->ne * 3 * N2;
     k3z_face<P><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(a);
     FRK_LAUNCHED(ctx);
     count_launch();
@@ -937,36 +1254,28 @@ int f3_launch(fr_ctx* ctx, int mode, const F3Args& a, bool perturb_trace, cudaSt
     FRK_LAUNCHED(ctx);
     return FR_OK;
   }
-  {
-    ProfScope ps_(ctx, fam, s, wb, wf);  // one timed record for the three kernels
-    if (perturb_trace) k3_trace<P, true><<<gt, E * NP, 0, s>>>(a);
-    else k3_trace<P, false><<<gt, E * NP, 0, s>>>(a);
-    FRK_LAUNCHED(ctx);
-    count_launch();  // the scope counted the trace kernel
-    if (mode == 3) {
-      const long long g3 = (a.nchunk * NB + E - 1) / E;
-      k3_cell<P, 3><<<(unsigned)g3, E * NP, L::BYTES, s>>>(a);
-    } else {
-      const long long nf = ctx->ne * 3 * N2;
-      k3_face<P><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(a);
-      FRK_LAUNCHED(ctx);
-      count_launch();
-      if (mode == 0) k3_cell<P, 0><<<gt, E * NP, L::BYTES, s>>>(a);
-      else if (mode == 1) k3_cell<P, 1><<<gt, E * NP, L::BYTES, s>>>(a);
-      else k3_cell<P, 2><<<gt, E * NP, L::BYTES, s>>>(a);
-    }
-  }
+  ProfScope ps_(ctx, fam, s, wb, wf);  // one timed record for the three kernels
+  if (mode == 0) k3_trace<P, false><<<gt, E * NP, 0, s>>>(a);
+  else k3_trace<P, true><<<gt, E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();  // the scope counted the trace kernel
+  constexpr int FT = Face3Threads<P>::value;
+  k3_face<P><<<(unsigned)((nf + FT - 1) / FT), FT, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();
+  if (mode == 0) k3_cell<P, 0><<<gt, E * NP, L::BYTES, s>>>(a);
+  else if (mode == 1) k3_cell<P, 1><<<gt, E * NP, L::BYTES, s>>>(a);
+  else k3_cell<P, 2><<<gt, E * NP, L::BYTES, s>>>(a);
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }
 
-int f3_dispatch(fr_ctx* ctx, int mode, const F3Args& a, bool perturb_trace, cudaStream_t s, double wb,
-                double wf) {
+int f3_dispatch(fr_ctx* ctx, int mode, const F3Args& a, cudaStream_t s, double wb, double wf) {
   switch (ctx->p) {
-    case 1: return f3_launch<1>(ctx, mode, a, perturb_trace, s, wb, wf);
-    case 2: return f3_launch<2>(ctx, mode, a, perturb_trace, s, wb, wf);
-    case 3: return f3_launch<3>(ctx, mode, a, perturb_trace, s, wb, wf);
-    case 4: return f3_launch<4>(ctx, mode, a, perturb_trace, s, wb, wf);
+    case 1: return f3_launch<1>(ctx, mode, a, s, wb, wf);
+    case 2: return f3_launch<2>(ctx, mode, a, s, wb, wf);
+    case 3: return f3_launch<3>(ctx, mode, a, s, wb, wf);
+    case 4: return f3_launch<4>(ctx, mode, a, s, wb, wf);
     default: return set_error(ctx, FR_ERR_UNSUPPORTED, "3D degree %d not compiled", ctx->p);
   }
 }
@@ -1018,7 +1327,7 @@ int launch_f3_residual(fr_ctx* ctx, int mode, const double* U, const double* z, 
   const bool in_cycle = done != nullptr;
   const double wb = in_cycle ? 0.0 : (mode == 0 ? 16.0 : (mode == 1 ? 32.0 : 40.0)) * nd;
   const double wf = in_cycle ? 0.0 : ns3d_residual_flops_per_element(ctx->p) * (double)ctx->ne + (mode == 0 ? 0.0 : 6.0 * nd);
-  return f3_dispatch(ctx, mode, a, mode != 0, s, wb, wf);
+  return f3_dispatch(ctx, mode, a, s, wb, wf);
 }
 
 namespace {
@@ -1033,21 +1342,29 @@ template <int P, typename T>
 int f3_columns(fr_ctx* ctx, F3Args a, cudaStream_t s) {
   using L = CellLayout<P, T>;
   constexpr int NP = L::NP, E = F3Slots<P>::E, NB = 5 * NP;
-  FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 3, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
+  FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cols<P, 3, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
   // one element residual per column: the own six faces' common data, counted
   // like the residual with every face of the element
   const double per = ns3d_residual_flops_per_element(P) + 3.0 * L::N2 * 245.0;
-  if (sizeof(T) == 4) {
-    // FP32: the element-local R(U) of each element by the same arithmetic first
-    a.r0f = ctx->r0f;
-    a.r0_pass = 1;
-    { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * (double)a.nchunk);
-      k3_cell<P, 3, T><<<(unsigned)((a.nchunk + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
-    FRK_LAUNCHED(ctx);
-    a.r0_pass = 0;
-  }
+  // the element-local R(U) of each element by the same arithmetic first
+  a.r0f = ctx->r0f;
+  a.r0d = ctx->rloc;
+  a.r0_pass = 1;
+  { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * (double)a.nchunk);
+    k3_cols<P, 3, T><<<(unsigned)((a.nchunk + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
+  FRK_LAUNCHED(ctx);
+  a.r0_pass = 0;
   { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * NB * (double)a.nchunk);
-    k3_cell<P, 3, T><<<(unsigned)((a.nchunk * NB + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
+    k3_cols<P, 3, T><<<(unsigned)((a.nchunk * NB + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
+  FRK_LAUNCHED(ctx);
+  return FR_OK;
+}
+
+template <int P>
+int f3_fulltrace(fr_ctx* ctx, const F3Args& a, cudaStream_t s) {
+  constexpr int NP = CellLayout<P>::NP, E = F3Slots<P>::E;
+  { ProfScope ps_(ctx, FR_KF_FACTOR, s);
+    k3_fulltrace<P><<<(unsigned)((ctx->ne + E - 1) / E), E * NP, 0, s>>>(a); }
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }
@@ -1069,19 +1386,18 @@ int f3_linearize(fr_ctx* ctx, const double* U, cudaStream_t s) {
   a.U = U;
   a.tb = ctx->lin3_tb;
   a.fb = ctx->lin3_fb;
-  a.write_gc = 1;
-  FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cell<P, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
+  FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cols<P, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
   const unsigned gt = (unsigned)((ctx->ne + E - 1) / E);
   {
     ProfScope ps_(ctx, FR_KF_OTHER, s);
-    k3_trace<P, false><<<gt, E * NP, 0, s>>>(a);
+    k3_fulltrace<P><<<gt, E * NP, 0, s>>>(a);
     FRK_LAUNCHED(ctx);
     count_launch();
     const long long nf = ctx->ne * 3 * N2;
-    k3_face<P><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(a);
+    k3_face_cache<P><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(a);
     FRK_LAUNCHED(ctx);
     count_launch();
-    k3_cell<P, 4><<<gt, E * NP, L::BYTES, s>>>(a);
+    k3_cols<P, 4><<<gt, E * NP, L::BYTES, s>>>(a);
   }
   FRK_LAUNCHED(ctx);
   return FR_OK;
@@ -1102,16 +1418,16 @@ int launch_f3_linearize(fr_ctx* ctx, const double* U, cudaStream_t s) {
 int launch_f3_factor(fr_ctx* ctx, const double* U, double shift, cudaStream_t s) {
   if (ctx->p > 3 || !ctx->mst || ctx->blk_chunk < 1)
     return set_error(ctx, FR_ERR_UNSUPPORTED, "3D element blocks are built for degrees 1 to 3");
-  // R0 of the element-local residuals = R(U); it leaves the unperturbed
-  // traces in the trace buffer, which the columns read as the frozen
-  // neighbour traces
   F3Args a = make_args3(ctx);
   a.U = U;
-  a.out = ctx->rloc;
-  FRK_TRY(f3_dispatch(ctx, 0, a, false, s, 0.0, 0.0));
-  a.R0 = ctx->rloc;
   a.out = ctx->mst;
   a.shift = shift;
+  // the unperturbed traces, which the columns read as the frozen neighbour traces
+  switch (ctx->p) {
+    case 1: FRK_TRY(f3_fulltrace<1>(ctx, a, s)); break;
+    case 2: FRK_TRY(f3_fulltrace<2>(ctx, a, s)); break;
+    default: FRK_TRY(f3_fulltrace<3>(ctx, a, s)); break;
+  }
   if (ctx->opts.block_columns == 1) {
     if (!ctx->r0f || !ctx->tbf)
       return set_error(ctx, FR_ERR_UNSUPPORTED, "FP32 block columns need block_columns = 1 at creation");
