@@ -29,10 +29,10 @@ struct fr_mlp {
   float* G = nullptr;       // gradients (same layout)
   float* Mo = nullptr;      // Adam first moments
   float* Vo = nullptr;      // Adam second moments
-  float* Z[3] = {};         // pre-activations [M x n[l+1]]
-  float* A[2] = {};         // hidden activations [M x n[l+1]]
+  float* Z = nullptr;       // output of the last FP32 forward [M x n[3]]
+  float* A[2] = {};         // hidden activations [M x n[l+1]] (positive where the pre-activation is)
   float* D[3] = {};         // loss gradients w.r.t. Z
-  float* part = nullptr;    // split-M partial weight gradients
+  float* part = nullptr;    // row splits' partial weight and bias gradients
   __nv_bfloat16* X16 = nullptr;   // BF16 input / hidden activations for inference,
   __nv_bfloat16* H16[2] = {};     //   rows padded to kp[l] (16-byte rows, zero pad)
   __nv_bfloat16* W16[3] = {};     // BF16 weights [n[l+1]][kp[l]], zero-padded columns
@@ -53,8 +53,6 @@ struct fr_mlp {
 namespace frk {
 namespace {
 
-constexpr int kSplitRows = 4096;  // rows per partial in the weight-gradient reduction
-
 long long off_W(const fr_mlp* m, int l) {
   long long o = 0;
   for (int i = 0; i < l; ++i) o += (long long)m->n[i + 1] * m->n[i] + m->n[i + 1];
@@ -62,56 +60,180 @@ long long off_W(const fr_mlp* m, int l) {
 }
 long long off_b(const fr_mlp* m, int l) { return off_W(m, l) + (long long)m->n[l + 1] * m->n[l]; }
 
-// ---- FP32 tiled GEMM: C[i][j] = sum_k A(i,k) B(k,j) (+ bias[j]) (ReLU) ----
-// A(i,k) = A[i*sai + k*sak], B(k,j) = B[k*sbk + j*sbj], C row-major ldc.
-// 64x64 tile, 16-deep k slices, 256 threads x (4x4) outputs.
-template <bool RELU>
-__global__ void __launch_bounds__(256) k_sgemm(int M, int N, int K, const float* __restrict__ A,
-                                               long long sai, long long sak, const float* __restrict__ B,
-                                               long long sbk, long long sbj, float* __restrict__ C, int ldc,
-                                               const float* __restrict__ bias, float* __restrict__ Zout,
-                                               int kbeg, int kend) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
-  float acc[4][4] = {};
-  if (kend < 0) kend = K;
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    for (int t = threadIdx.x; t < 16 * 64; t += 256) {
-      const int kk = t / 64, r = t % 64;
-      const int i = i0 + r, k = k0 + kk, j = j0 + r;
-      As[kk][r] = (i < M && k < kend) ? A[i * sai + k * sak] : 0.f;
-      Bs[kk][r] = (j < N && k < kend) ? B[k * sbk + j * sbj] : 0.f;
+// ---- FP32 tiled GEMM: C(i, j) = sum over k in [kbeg, kend) of A(i, k) B(k, j) ----
+// A is [i][lda] (AK: k runs along memory) or [k][lda]; B is [j][ldb] (BK) or
+// [k][ldb].  64 x 64 tile per CTA, 16-deep slices double-buffered in shared
+// memory with the next slice's global loads in flight during the FMAs; 128
+// threads x (8 x 4) outputs, so a slice step costs 3 16-byte shared loads per 32
+// FMAs.  64 x 64 (not 128 x 64) because the batches are 256 to 73,728 rows of 100
+// to 300 columns: 8192 rows x 256 columns give 512 CTAs, 3.4 per SM.
+// Loads are 16 bytes wide where base, leading dimension and the k range allow
+// it (vec), else one value at a time.  One training step of 8192 samples (300-
+// 256-256-100), GEMMs and the rest: 5674 -> 366 us; the first version read
+// both operands with a stride of one row per lane, summed the bias gradients in
+// one thread per column and launched the row splits one after another.
+enum SgemmEpilogue {
+  EPI_RELU = 0,     // C = max(acc + bias, 0)
+  EPI_BIAS2 = 1,    // C = C2 = acc + bias
+  EPI_MASK = 2,     // C = acc where mask > 0, else 0 (mask laid out as C)
+  EPI_PARTIAL = 3   // C[split] = acc, then the sums of A over k behind it
+};
+struct SgemmArgs {
+  int M, N, K;
+  const float* A;
+  int lda;
+  const float* B;
+  int ldb;
+  float* C;
+  int ldc;
+  const float* bias;   // EPI_RELU, EPI_BIAS2
+  float* C2;           // EPI_BIAS2
+  const float* mask;   // EPI_MASK
+  int ksplit;          // k range of each blockIdx.z (K: one split)
+  int veca, vecb;      // 16-byte loads allowed
+};
+
+// four consecutive values along memory at p, `ok` of them in range
+__device__ __forceinline__ float4 load4(const float* p, int ok, int vec) {
+  if (vec && ok >= 4) return *reinterpret_cast<const float4*>(p);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (ok > 0) v.x = p[0];
+  if (ok > 1) v.y = p[1];
+  if (ok > 2) v.z = p[2];
+  if (ok > 3) v.w = p[3];
+  return v;
+}
+
+constexpr int kGT = 64, kGK = 16, kGP = kGT + 4;  // tile side, slice depth, shared pitch
+
+// this thread's 2 x 4 values of a 64 x 16 operand slice: KC (k along memory):
+// row tid / 2, k = 4 (tid % 2) and 8 more (the two halves land 16 banks apart);
+// else k = tid / 16 and 8 more, four rows at 4 (tid % 16)
+template <bool KC>
+__device__ __forceinline__ void slice_load(float4 v[2], const float* X, int ld, int x0, int nx, int k0, int kend,
+                                           int vec) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (KC) {
+      const int x = x0 + (tid >> 1), k = k0 + 4 * (tid & 1) + 8 * u;
+      v[u] = load4(X + (long long)x * ld + k, x < nx ? kend - k : 0, vec);
+    } else {
+      const int x = x0 + 4 * (tid & 15), k = k0 + (tid >> 4) + 8 * u;
+      v[u] = load4(X + (long long)k * ld + x, k < kend ? nx - x : 0, vec);
     }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[kk][ty + 16 * u];
-        b[u] = Bs[kk][tx + 16 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
-    }
-    __syncthreads();
   }
+}
+template <bool KC>
+__device__ __forceinline__ void slice_store(float (*S)[kGP], const float4 v[2]) {
+  const int tid = threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < 2; ++u) {
+    if (KC) {
+      const int x = tid >> 1, k = 4 * (tid & 1) + 8 * u;
+      S[k][x] = v[u].x;
+      S[k + 1][x] = v[u].y;
+      S[k + 2][x] = v[u].z;
+      S[k + 3][x] = v[u].w;
+    } else {
+      *reinterpret_cast<float4*>(&S[(tid >> 4) + 8 * u][4 * (tid & 15)]) = v[u];
+    }
+  }
+}
+
+template <bool AK, bool BK, int EPI>
+__global__ void __launch_bounds__(128) k_sgemm(const SgemmArgs a) {
+  __shared__ __align__(16) float As[2][kGK][kGP], Bs[2][kGK][kGP];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int i0 = blockIdx.y * kGT, j0 = blockIdx.x * kGT;
+  const int kbeg = blockIdx.z * a.ksplit, kend = min(a.K, kbeg + a.ksplit);
+  float acc[8][4] = {};
+  float asum = 0.f;  // EPI_PARTIAL: sum over k of A(i0 + tid, k), by the first tile of a row of tiles
+  float4 va[2], vb[2];
+  slice_load<AK>(va, a.A, a.lda, i0, a.M, kbeg, kend, a.veca);
+  slice_load<BK>(vb, a.B, a.ldb, j0, a.N, kbeg, kend, a.vecb);
+  slice_store<AK>(As[0], va);
+  slice_store<BK>(Bs[0], vb);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = kbeg; k0 < kend; k0 += kGK) {
+    const bool more = k0 + kGK < kend;
+    if (more) {
+      slice_load<AK>(va, a.A, a.lda, i0, a.M, k0 + kGK, kend, a.veca);
+      slice_load<BK>(vb, a.B, a.ldb, j0, a.N, k0 + kGK, kend, a.vecb);
+    }
+#pragma unroll
+    for (int kk = 0; kk < kGK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][8 * ty + 4]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b0.x, b0.y, b0.z, b0.w};
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+    }
+    if (EPI == EPI_PARTIAL && blockIdx.x == 0 && tid < kGT) {
+#pragma unroll
+      for (int kk = 0; kk < kGK; ++kk) asum += As[buf][kk][tid];
+    }
+    if (more) {  // the other buffer was last read before the previous barrier
+      slice_store<AK>(As[buf ^ 1], va);
+      slice_store<BK>(Bs[buf ^ 1], vb);
+      __syncthreads();
+      buf ^= 1;
+    }
+  }
+  const long long slot = (long long)blockIdx.z * ((long long)a.M * a.N + a.M);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = i0 + 8 * ty + u;
+    if (i >= a.M) break;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
-      if (i < M && j < N) {
-        float c = acc[u][v] + (bias ? bias[j] : 0.f);
-        if (Zout) Zout[(long long)i * ldc + j] = c;
-        if (RELU) c = fmaxf(c, 0.f);
-        C[(long long)i * ldc + j] = c;
+      const int j = j0 + 4 * tx + v;
+      if (j >= a.N) break;
+      const long long o = (long long)i * a.ldc + j;
+      float c = acc[u][v];
+      if (EPI == EPI_RELU) a.C[o] = fmaxf(c + a.bias[j], 0.f);
+      if (EPI == EPI_BIAS2) {
+        c += a.bias[j];
+        a.C[o] = c;
+        a.C2[o] = c;
       }
+      if (EPI == EPI_MASK) a.C[o] = a.mask[o] > 0.f ? c : 0.f;
+      if (EPI == EPI_PARTIAL) a.C[slot + o] = c;
     }
+  }
+  if (EPI == EPI_PARTIAL && blockIdx.x == 0 && tid < kGT && i0 + tid < a.M)
+    a.C[slot + (long long)a.M * a.N + i0 + tid] = asum;
+}
+
+int vec_ok(const float* p, int ld) { return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld % 4 == 0; }
+
+template <bool AK, bool BK, int EPI>
+void sgemm(SgemmArgs a, int splits, cudaStream_t s) {
+  a.veca = vec_ok(a.A, a.lda);
+  a.vecb = vec_ok(a.B, a.ldb);
+  const dim3 grid((a.N + kGT - 1) / kGT, (a.M + kGT - 1) / kGT, splits);
+  count_launch();
+  k_sgemm<AK, BK, EPI><<<grid, 128, 0, s>>>(a);
+}
+
+// Row splits of a weight gradient (n x k outputs summed over M rows): enough that
+// its 64 x 64 tiles give each SM about three CTAs, at least 64 rows each; grows
+// with M.
+int max_splits(int n, int k, int M) {
+  const int tiles = ((n + kGT - 1) / kGT) * ((k + kGT - 1) / kGT);
+  return std::max(1, std::min((3 * 152 + tiles - 1) / tiles, (M + 63) / 64));
+}
+// rows per split, a multiple of the slice depth, and the splits that makes (at
+// most max_splits)
+int split_rows(int n, int k, int M, int* splits) {
+  const int want = max_splits(n, k, M);
+  const int rows = ((M + want - 1) / want + kGK - 1) / kGK * kGK;
+  *splits = (M + rows - 1) / rows;
+  return rows;
 }
 
 // ---- BF16 tensor-core GEMM for inference: Y = act(X W^T + b) ----
@@ -360,40 +482,41 @@ __global__ void k_loss_grad(const float* __restrict__ y, const float* __restrict
   }
 }
 
-// d = d * (z > 0)
-__global__ void k_relu_back(float* __restrict__ d, const float* __restrict__ z, long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    if (!(z[i] > 0.f)) d[i] = 0.f;
-}
-
-// sum of the split-M partials (fixed order) into the weight gradient; bias
-// gradient = column sums of dZ (fixed order)
+// sum of the row splits' partials (fixed order) into a layer's weight and bias
+// gradients, which lie side by side as in the partials
 __global__ void k_sum_parts(const float* __restrict__ part, int nparts, long long n, float* __restrict__ out) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     float s = 0.f;
+#pragma unroll 8
     for (int p = 0; p < nparts; ++p) s += part[(long long)p * n + i];
     out[i] = s;
   }
 }
 
-__global__ void k_colsum(const float* __restrict__ d, int M, int N, float* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  float s = 0.f;
-  for (int i = 0; i < M; ++i) s += d[(long long)i * N + j];
-  out[j] = s;
-}
-
+// Adam on every parameter, and the BF16 copy of the weights for inference
+// (rows padded to kp; the padding stays zero)
+struct AdamLayers {
+  long long off[3];        // first weight of the layer
+  int rows[3], cols[3], kp[3];
+  __nv_bfloat16* W16[3];
+};
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, long long n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
+                       float c1, float c2, const AdamLayers al) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float x = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = x;
+    const int l = i >= al.off[2] ? 2 : (i >= al.off[1] ? 1 : 0);
+    const long long w = i - al.off[l];
+    if (w < (long long)al.rows[l] * al.cols[l]) {
+      const int r = (int)(w / al.cols[l]), c = (int)(w % al.cols[l]);
+      al.W16[l][(long long)r * al.kp[l] + c] = __float2bfloat16_rn(x);
+    }
   }
 }
 
@@ -479,7 +602,7 @@ void free_mlp(fr_mlp* m) {
   for (auto* p : m->W16) cudaFree(p);
   cudaFree(m->derr);
   cudaFreeHost(m->herr);
-  for (auto* p : m->Z) cudaFree(p);
+  cudaFree(m->Z);
   for (auto* p : m->A) cudaFree(p);
   for (auto* p : m->D) cudaFree(p);
   cudaFree(m->part); cudaFree(m->X16);
@@ -518,23 +641,27 @@ extern "C" int fr_mlp_create(int n_in, int n_hidden, int n_out, int max_batch, f
   if (e == cudaSuccess) e = cudaMalloc(&m->Vo, np * sizeof(float));
   for (int l = 0; l < 3; ++l) m->kp[l] = (m->n[l] + 7) / 8 * 8;
   for (int l = 0; l < 3 && e == cudaSuccess; ++l)
-    e = cudaMalloc(&m->W16[l], (size_t)m->n[l + 1] * m->kp[l] * sizeof(__nv_bfloat16));
+  {
+    const size_t wb = (size_t)m->n[l + 1] * m->kp[l] * sizeof(__nv_bfloat16);
+    e = cudaMalloc(&m->W16[l], wb);
+    if (e == cudaSuccess) e = cudaMemset(m->W16[l], 0, wb);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&m->derr, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->derr, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&m->herr, sizeof(int));
   if (e == cudaSuccess) *m->herr = 0;
-  for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
-    e = cudaMalloc(&m->Z[l], (size_t)max_batch * m->n[l + 1] * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&m->D[l], (size_t)max_batch * m->n[l + 1] * sizeof(float));
-  }
+  if (e == cudaSuccess) e = cudaMalloc(&m->Z, (size_t)max_batch * n_out * sizeof(float));
+  for (int l = 0; l < 3 && e == cudaSuccess; ++l)
+    e = cudaMalloc(&m->D[l], (size_t)max_batch * m->n[l + 1] * sizeof(float));
   for (int l = 0; l < 2 && e == cudaSuccess; ++l) {
     e = cudaMalloc(&m->A[l], (size_t)max_batch * m->n[l + 1] * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&m->H16[l], (size_t)max_batch * m->kp[l + 1] * sizeof(__nv_bfloat16));
   }
-  const int nparts = (max_batch + kSplitRows - 1) / kSplitRows;
-  long long maxw = 0;
-  for (int l = 0; l < 3; ++l) maxw = std::max(maxw, (long long)m->n[l + 1] * m->n[l]);
-  if (e == cudaSuccess) e = cudaMalloc(&m->part, (size_t)nparts * maxw * sizeof(float));
+  long long np_max = 0;
+  for (int l = 0; l < 3; ++l)
+    np_max = std::max(np_max, max_splits(m->n[l + 1], m->n[l], max_batch) *
+                                  ((long long)m->n[l + 1] * m->n[l] + m->n[l + 1]));
+  if (e == cudaSuccess) e = cudaMalloc(&m->part, (size_t)np_max * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&m->X16, (size_t)max_batch * m->kp[0] * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = cudaMalloc(&m->loss, sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(m->Mo, 0, np * sizeof(float));
@@ -597,17 +724,16 @@ extern "C" int fr_mlp_forward(fr_mlp* m, const float* X, int M, float* Y, int bf
   if (!bf16) {
     const float* in = X;
     for (int l = 0; l < 3; ++l) {
-      const int K = m->n[l], N = m->n[l + 1];
-      const dim3 grid((N + 63) / 64, (M + 63) / 64);
-      float* C = l < 2 ? m->A[l] : Y;
-      count_launch();
-      if (l < 2)
-        k_sgemm<true><<<grid, 256, 0, s>>>(M, N, K, in, K, 1, m->P + off_W(m, l), 1, K, C, N,
-                                           m->P + off_b(m, l), m->Z[l], 0, -1);
-      else
-        k_sgemm<false><<<grid, 256, 0, s>>>(M, N, K, in, K, 1, m->P + off_W(m, l), 1, K, C, N,
-                                            m->P + off_b(m, l), m->Z[l], 0, -1);
-      in = C;
+      SgemmArgs g{};
+      g.M = M; g.N = m->n[l + 1]; g.K = g.ksplit = m->n[l];
+      g.A = in; g.lda = m->n[l];
+      g.B = m->P + off_W(m, l); g.ldb = m->n[l];
+      g.bias = m->P + off_b(m, l);
+      g.C = l < 2 ? m->A[l] : Y; g.ldc = g.N;
+      g.C2 = m->Z;
+      if (l < 2) sgemm<true, true, EPI_RELU>(g, 1, s);
+      else sgemm<true, true, EPI_BIAS2>(g, 1, s);
+      in = g.C;
     }
   } else {
     static bool attr = false;  // dynamic shared memory above 48 KB, set once per process
@@ -678,34 +804,31 @@ extern "C" int fr_mlp_backward(fr_mlp* m, const float* X, const float* T, int M,
   MLP_CUDA(m, cudaGetDevice(&dev));
   Reduce red{g_mlp_red[dev].partials, g_mlp_red[dev].counter};
   const long long nout = (long long)M * m->n[3];
-  // output: Y = Z[2] (forward_train stored it)
+  // Z holds the forward pass's output
   count_launch();
-  k_loss_grad<<<grid_for(nout) > 1024 ? 1024 : grid_for(nout), 256, 0, s>>>(m->Z[2], T, m->D[2], nout, m->loss, red);
-  const int nparts = (M + kSplitRows - 1) / kSplitRows;
+  k_loss_grad<<<grid_for(nout) > 1024 ? 1024 : grid_for(nout), 256, 0, s>>>(m->Z, T, m->D[2], nout, m->loss, red);
   for (int l = 2; l >= 0; --l) {
     const int K = m->n[l], N = m->n[l + 1];
-    const float* in = l == 0 ? X : m->A[l - 1];
-    // dW[N x K] = sum over rows of D[l]^T (rows) x in (rows): split by rows
-    for (int p = 0; p < nparts; ++p) {
-      const int r0 = p * kSplitRows, r1 = std::min(M, r0 + kSplitRows);
-      const dim3 grid((K + 63) / 64, (N + 63) / 64);
-      count_launch();
-      // C[i=n][j=k] = sum_r D[r][n] in[r][k]; A(i,kr) = D[kr*N + i], B(kr,j) = in[kr*K + j]
-      k_sgemm<false><<<grid, 256, 0, s>>>(N, K, r1, m->D[l], 1, N, in, K, 1,
-                                          m->part + (long long)p * N * K, K, nullptr, nullptr, r0, r1);
-    }
+    // dW[N x K] = D[l]^T in and db[N] = column sums of D[l], over row splits
+    int splits = 0;
+    SgemmArgs g{};
+    g.M = N; g.N = K; g.K = M;
+    g.ksplit = split_rows(N, K, M, &splits);
+    g.A = m->D[l]; g.lda = N;
+    g.B = l == 0 ? X : m->A[l - 1]; g.ldb = K;
+    g.C = m->part; g.ldc = K;
+    sgemm<false, false, EPI_PARTIAL>(g, splits, s);
+    const long long np = (long long)N * K + N;
     count_launch();
-    k_sum_parts<<<grid_for((long long)N * K), 256, 0, s>>>(m->part, nparts, (long long)N * K, m->G + off_W(m, l));
-    count_launch();
-    k_colsum<<<(N + 127) / 128, 128, 0, s>>>(m->D[l], M, N, m->G + off_b(m, l));
-    if (l > 0) {
-      // D[l-1] = (D[l] W_l) * relu'(Z[l-1]);  D[l] [M x N], W_l [N x K]
-      const dim3 grid((K + 63) / 64, (M + 63) / 64);
-      count_launch();
-      k_sgemm<false><<<grid, 256, 0, s>>>(M, K, N, m->D[l], N, 1, m->P + off_W(m, l), K, 1, m->D[l - 1], K,
-                                          nullptr, nullptr, 0, -1);
-      count_launch();
-      k_relu_back<<<grid_for((long long)M * K), 256, 0, s>>>(m->D[l - 1], m->Z[l - 1], (long long)M * K);
+    k_sum_parts<<<grid_for(np), 256, 0, s>>>(m->part, splits, np, m->G + off_W(m, l));
+    if (l > 0) {  // D[l-1] = D[l] W_l where the activation is positive
+      SgemmArgs d{};
+      d.M = M; d.N = K; d.K = d.ksplit = N;
+      d.A = m->D[l]; d.lda = N;
+      d.B = m->P + off_W(m, l); d.ldb = K;
+      d.C = m->D[l - 1]; d.ldc = K;
+      d.mask = m->A[l - 1];
+      sgemm<true, false, EPI_MASK>(d, 1, s);
     }
   }
   MLP_CUDA(m, cudaGetLastError());
@@ -722,8 +845,16 @@ extern "C" int fr_mlp_adam(fr_mlp* m, float lr, float beta1, float beta2, float 
   m->step += 1;
   const float c1 = 1.f - std::pow(beta1, (float)m->step);
   const float c2 = 1.f - std::pow(beta2, (float)m->step);
+  AdamLayers al;
+  for (int l = 0; l < 3; ++l) {
+    al.off[l] = off_W(m, l);
+    al.rows[l] = m->n[l + 1];
+    al.cols[l] = m->n[l];
+    al.kp[l] = m->kp[l];
+    al.W16[l] = m->W16[l];
+  }
   count_launch();
-  k_adam<<<grid_for(m->nparam), 256, 0, s>>>(m->P, m->G, m->Mo, m->Vo, m->nparam, lr, beta1, beta2, eps, c1, c2);
+  k_adam<<<grid_for(m->nparam), 256, 0, s>>>(m->P, m->G, m->Mo, m->Vo, m->nparam, lr, beta1, beta2, eps, c1, c2, al);
   MLP_CUDA(m, cudaGetLastError());
-  return refresh_bf16(m, s);
+  return FR_OK;
 }

@@ -63,3 +63,48 @@ def test_density_outside_the_normal_range_stays_visible(fr, bad):
     assert not np.isfinite(R[0]).all()
     far = 4 + 4 * n
     assert np.array_equal(R[far], R0[far])
+
+
+@pytest.mark.parametrize("n_in,n_h,n_out", [(20, 64, 7), (21, 33, 5), (108, 256, 36), (3, 1, 2)])
+@pytest.mark.parametrize("M", [1, 63, 65, 130, 1472])
+def test_training_step_at_tile_edges(fr, n_in, n_h, n_out, M):
+    """FP32 forward, gradients and one Adam step where 64-wide tiles, 16-deep slices, row splits and the
+    16-byte loads end: against the oracle network in FP64.  A sum of K products of unit scale carries
+    at most K u (u = 2^-24) relative to the sum of their magnitudes, K <= 1472: 1472 u = 9e-5, and the
+    errors of a random sum grow like sqrt(K): bound 1e-5 relative in the 2-norm (the repository's)."""
+    import torch
+    rng = np.random.default_rng(M + n_in)
+    sizes = (n_in, n_h, n_h, n_out)
+    params = [(rng.standard_normal((b, a)) * np.sqrt(2.0 / a), 0.1 * rng.standard_normal(b))
+              for a, b in zip(sizes[:-1], sizes[1:])]
+    params = [(W.astype(np.float32).astype(np.float64), b.astype(np.float32).astype(np.float64)) for W, b in params]
+    X = rng.standard_normal((M, n_in)).astype(np.float32)
+    T = rng.standard_normal((M, n_out)).astype(np.float32)
+    # room for other batches: the partial buffer is sized by the model, not by this call
+    net = fr.MLP(n_in, n_h, n_out, max(M, 1500))
+    net.set_params(fr.flat_params(params))
+    Y = torch.empty((M, n_out), dtype=torch.float32, device="cuda")
+    Xd, Td = _t(X), _t(T)
+    net.forward(Xd, Y)
+    loss = net.backward(Xd, Td)
+    g = net.get_grads().astype(np.float64)
+    A, Z = [X.astype(np.float64)], []
+    for W, b in params:
+        Z.append(A[-1] @ W.T + b)
+        A.append(np.maximum(Z[-1], 0.0))
+    d = (Z[2] - T) / Z[2].size
+    want = [None] * 3
+    for k in (2, 1, 0):
+        want[k] = np.concatenate([(d.T @ A[k]).reshape(-1), d.sum(0)])
+        d = (d @ params[k][0]) * (Z[k - 1] > 0) if k else d
+    want = np.concatenate(want)
+    assert np.linalg.norm(Y.cpu().numpy() - Z[2]) <= 1e-5 * np.linalg.norm(Z[2])
+    assert abs(loss - 0.5 * np.mean((Z[2] - T) ** 2)) <= 1e-5 * abs(loss)
+    assert np.linalg.norm(g - want) <= 1e-5 * np.linalg.norm(want)
+    # Adam refreshes the BF16 weights: inference follows the FP32 forward to BF16 rounding
+    net.adam(1e-3)
+    Yb = torch.empty_like(Y)
+    net.forward(Xd, Y)
+    net.forward(Xd, Yb, bf16=True)
+    Y, Yb = Y.cpu().numpy(), Yb.cpu().numpy()
+    assert np.linalg.norm(Yb - Y) <= 3e-2 * np.linalg.norm(Y) + 1e-6
