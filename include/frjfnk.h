@@ -524,7 +524,9 @@ long long fr_kernel_launches(void);
 
 /* Start timing every launch of the families whose bit (1 << FR_KF_*) is set
  * in family_mask with CUDA events on the launching stream.  Creates the
- * events (host-side setup, no device allocation). */
+ * events (host-side setup, no device allocation).  While families are timed,
+ * a small 2D Euler solve that otherwise runs as one launch runs as the
+ * separate ones (same results). */
 int fr_profile_begin(fr_ctx* ctx, unsigned family_mask);
 
 /* Stop timing; synchronises the recorded events and writes, per family

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "device.cuh"
+#include "cycle.h"
 #include "internal.cuh"
 
 namespace frk {
@@ -81,6 +82,8 @@ void free_ctx(fr_ctx* c) {
   }
   cudaFreeHost(c->h_stat);
   cudaFreeHost(c->h_scal);
+  cudaFreeHost(c->h_cyc);
+  cudaFree(c->cyc_bar);
   delete c;
 }
 
@@ -150,7 +153,8 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->z, n));
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
-  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kMaxVec));
+  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
+  FRK_TRY(dalloc(c, &c->cyc_bar, 32));
   FRK_TRY(dalloc(c, &c->red.counter, 1));
   c->gd.ldh = m + 1;
   FRK_TRY(dalloc(c, &c->gd.H, (size_t)(m + 1) * m));
@@ -170,6 +174,7 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_CUDA(c, cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_stat), (4 + kMaxVec) * sizeof(int)));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double)));
+  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_cyc), sizeof(CycleStatus)));
   for (cudaEvent_t& e : c->chunk_ev) FRK_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   FRK_CUDA(c, cudaDeviceSynchronize());
   return FR_OK;
@@ -236,7 +241,8 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->z, n));
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
-  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kMaxVec));
+  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
+  FRK_TRY(dalloc(c, &c->cyc_bar, 32));
   FRK_TRY(dalloc(c, &c->red.counter, 1));
   c->gd.ldh = m + 1;
   FRK_TRY(dalloc(c, &c->gd.H, (size_t)(m + 1) * m));
@@ -256,6 +262,7 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_CUDA(c, cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_stat), (4 + kMaxVec) * sizeof(int)));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double)));
+  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_cyc), sizeof(CycleStatus)));
   for (cudaEvent_t& e : c->chunk_ev) FRK_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   FRK_CUDA(c, cudaDeviceSynchronize());
   return FR_OK;

@@ -140,26 +140,47 @@ __device__ __forceinline__ bool last_block(unsigned* counter, int nblk = -1) {
   return am_last;
 }
 
-// In the last block: out[i] = sum over blocks b (fixed order) of partials[b][i],
-// i < nvec, over the nblk blocks of the reduction (nblk < 0: the whole grid).
-// Each warp sums one value with its lanes striding over the blocks through
-// four independent accumulators.  Resets the counter.
+// Sum of the nblk partials of one value in a fixed order, by one warp (result in
+// lane 0): lane l takes partials l, l + 32, ... into four accumulators in turn,
+// those of its last incomplete round of four into the first.  Sixteen loads are
+// in flight at a time: one round of L2 latency per 512 partials, not per 128.
+__device__ __forceinline__ double sum_partials(const double* p, int nblk) {
+  const int lane = threadIdx.x & 31;
+  const int full = nblk - 96 > lane ? (nblk - 97 - lane) / 128 + 1 : 0;  // rounds of four
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  for (int r0 = 0; lane + 128 * r0 < nblk; r0 += 4) {
+    double v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int b = lane + 128 * r0 + 32 * u;
+      v[u] = b < nblk ? __ldcg(p + b) : 0.0;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (r0 + r < full) {
+        s0 += v[4 * r];
+        s1 += v[4 * r + 1];
+        s2 += v[4 * r + 2];
+        s3 += v[4 * r + 3];
+      } else {
+#pragma unroll
+        for (int u = 4 * r; u < 4 * r + 4; ++u)
+          if (lane + 128 * r0 + 32 * u < nblk) s0 += v[u];
+      }
+    }
+  }
+  return warp_sum((s0 + s1) + (s2 + s3));
+}
+
+// In the last block: out[i] = sum over blocks b (fixed order) of the partials of
+// value i, i < nvec, over the nblk blocks of the reduction (nblk < 0: the whole
+// grid), one warp per value.  Resets the counter.
 __device__ __forceinline__ void finish_sums(const Reduce& red, int nvec, double* out, int nblk = -1) {
   __threadfence();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int G = nblk < 0 ? (int)gridDim.x : nblk;
   for (int i = wid; i < nvec; i += nw) {
-    const double* p = red.partials + i;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int b = lane;
-    for (; b + 96 < G; b += 128) {
-      s0 += __ldcg(p + (size_t)b * kMaxVec);
-      s1 += __ldcg(p + (size_t)(b + 32) * kMaxVec);
-      s2 += __ldcg(p + (size_t)(b + 64) * kMaxVec);
-      s3 += __ldcg(p + (size_t)(b + 96) * kMaxVec);
-    }
-    for (; b < G; b += 32) s0 += __ldcg(p + (size_t)b * kMaxVec);
-    double s = warp_sum((s0 + s1) + (s2 + s3));
+    const double s = sum_partials(red.value(i), G);
     if (lane == 0) out[i] = s;
   }
   if (threadIdx.x == 0) *red.counter = 0u;

@@ -1177,7 +1177,7 @@ __global__ void __launch_bounds__(256) k3_dissipation(const F3Args a, Reduce red
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double bs = block_sum(acc[c], sh);
-    if (threadIdx.x == 0) red.partials[(size_t)blockIdx.x * kMaxVec + c] = bs;
+    if (threadIdx.x == 0) red.value(c)[blockIdx.x] = bs;
   }
   if (last_block(red.counter)) finish_sums(red, 3, out);
 }

@@ -39,8 +39,10 @@ struct Tables {
 // completion counter (the last block to finish sums the partials in a fixed
 // order and resets the counter).
 struct Reduce {
-  double* partials;   // [kRedBlocks][kMaxVec]
+  double* partials;   // [value][kRedBlocks]
   unsigned* counter;
+  // the blocks' partials of one value, side by side
+  __host__ __device__ double* value(int i) const { return partials + (size_t)i * kRedBlocks; }
 };
 
 // GMRES cycle state kept on the device so a whole cycle is launched without
@@ -105,6 +107,8 @@ struct Prof {
 struct fr_mlp;
 
 namespace frk {
+struct CycleStatus;
+
 // Training-pair capture of ROW stage solves (features and scaled targets).
 struct StageCapture {
   float* X = nullptr;       // [max][3 nb]
@@ -175,6 +179,8 @@ struct fr_ctx {
   int tile_variant = 0;      // element-tile shape of the Euler residual kernel (autotuned)
   frk::Reduce red{};
   frk::GmresDev gd{};
+  unsigned* cyc_bar = nullptr;             // one-launch solves: barrier counter
+  frk::CycleStatus* h_cyc = nullptr;       // pinned: how the last one ended
   int* h_stat = nullptr;     // pinned host mirror: done, k
   double* h_scal = nullptr;  // pinned host mirror of a few doubles
   frk::Prof prof;

@@ -9,7 +9,8 @@
 // cycle return at once.  The host reads the cycle status once per restart.
 #include <cmath>
 
-#include "device.cuh"
+#include "cycle.h"
+#include "krylov_body.cuh"
 
 namespace frk {
 namespace {
@@ -20,28 +21,11 @@ unsigned vgrid(const fr_ctx* ctx, long long n) {
   return (unsigned)(g < 1 ? 1 : g);
 }
 
-// this thread's share of ||x||^2: one FMA chain in row order, eight loads in
-// flight (with one, 16.8 M rows ran at a tenth of HBM's rate)
-__device__ __forceinline__ double sumsq_rows(const double* __restrict__ x, long long n) {
-  const long long S = (long long)gridDim.x * blockDim.x;
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double ss = 0.0;
-  for (; i + 7 * S < n; i += 8 * S) {
-    double v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = x[i + u * S];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) ss = fma(v[u], v[u], ss);
-  }
-  for (; i < n; i += S) ss = fma(x[i], x[i], ss);
-  return ss;
-}
-
 __global__ void k_sumsq(const double* __restrict__ x, long long n, double* out, Reduce red,
                         EpsArgs ea) {
   __shared__ double sh[32];
-  const double bs = block_sum(sumsq_rows(x, n), sh);
-  if (threadIdx.x == 0) red.partials[(size_t)blockIdx.x * kMaxVec] = bs;
+  const double bs = block_sum(sumsq_rows(x, n, blockIdx.x, gridDim.x), sh);
+  if (threadIdx.x == 0) red.value(0)[blockIdx.x] = bs;
   if (last_block(red.counter)) {
     finish_sums(red, 1, out);
     if (threadIdx.x == 0) write_eps(ea, *out);
@@ -53,11 +37,11 @@ __global__ void k_sumsq(const double* __restrict__ x, long long n, double* out, 
 __global__ void k_sumsq2(const double* __restrict__ x, const double* __restrict__ y, long long n, double* out,
                          Reduce red, EpsArgs ea) {
   __shared__ double sh[32];
-  const double bx = block_sum(sumsq_rows(x, n), sh);
-  const double by = block_sum(sumsq_rows(y, n), sh);
+  const double bx = block_sum(sumsq_rows(x, n, blockIdx.x, gridDim.x), sh);
+  const double by = block_sum(sumsq_rows(y, n, blockIdx.x, gridDim.x), sh);
   if (threadIdx.x == 0) {
-    red.partials[(size_t)blockIdx.x * kMaxVec] = bx;
-    red.partials[(size_t)blockIdx.x * kMaxVec + 1] = by;
+    red.value(0)[blockIdx.x] = bx;
+    red.value(1)[blockIdx.x] = by;
   }
   if (last_block(red.counter)) {
     finish_sums(red, 2, out);
@@ -85,112 +69,9 @@ __global__ void k_lincomb(double* out, long long len, const Lincomb lc, double* 
   }
   if (sumsq) {
     const double bs = block_sum(ss, sh);
-    if (threadIdx.x == 0) red.partials[(size_t)blockIdx.x * kMaxVec] = bs;
+    if (threadIdx.x == 0) red.value(0)[blockIdx.x] = bs;
     if (last_block(red.counter)) finish_sums(red, 1, sumsq);
   }
-}
-
-// One sweep over the rows accumulating NC dot products against w; the
-// basis pointers are resolved outside the row loop so every row costs
-// exactly NC fused multiply-adds on the FP64 pipe.  UR rows are in flight per
-// thread (NC x UR independent accumulation chains hide the FMA latency).
-template <int NC>
-__device__ __forceinline__ void dots_chunk(const double* const* ptr, const double* __restrict__ w,
-                                           long long n, double* acc, int bid, int nblk) {
-  constexpr int UR = NC >= 8 ? 1 : (NC >= 4 ? 2 : 4);
-  double a[NC][UR];
-#pragma unroll
-  for (int i = 0; i < NC; ++i)
-#pragma unroll
-    for (int u = 0; u < UR; ++u) a[i][u] = 0.0;
-  const long long S = (long long)nblk * blockDim.x;
-  for (long long r0 = (long long)bid * blockDim.x + threadIdx.x; r0 < n; r0 += UR * S) {
-    double wr[UR];
-#pragma unroll
-    for (int u = 0; u < UR; ++u) wr[u] = (r0 + u * S < n) ? w[r0 + u * S] : 0.0;
-#pragma unroll
-    for (int i = 0; i < NC; ++i)
-#pragma unroll
-      for (int u = 0; u < UR; ++u)
-        if (r0 + u * S < n) a[i][u] = fma(ptr[i][r0 + u * S], wr[u], a[i][u]);
-  }
-#pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    double s = a[i][0];
-#pragma unroll
-    for (int u = 1; u < UR; ++u) s += a[i][u];
-    acc[i] = s;
-  }
-}
-
-// out[i] = <V_i, w> for i < nvec, and out[nvec] = <w, w> when with_self,
-// in chunks of up to 8 values per sweep.  Skipped when the cycle is done or
-// when `gate` points at a zero flag.
-__device__ __forceinline__ void dots_body(const double* __restrict__ V, long long ldv, int nvec,
-                                          const double* __restrict__ w, long long n, double* out,
-                                          int with_self, const Reduce& red, const int* done,
-                                          const int* gate, int bid, int nblk) {
-  __shared__ double sred[8][kThreads / 32];
-  if ((done && *done) || (gate && !*gate)) return;
-  const int total = nvec + (with_self ? 1 : 0);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int c0 = 0; c0 < total; c0 += 8) {
-    const int nc = min(8, total - c0);
-    const double* ptr[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int idx = c0 + i;
-      ptr[i] = idx < nvec ? V + (size_t)idx * ldv : w;
-    }
-    double acc[8];
-    switch (nc) {
-      case 1: dots_chunk<1>(ptr, w, n, acc, bid, nblk); break;
-      case 2: dots_chunk<2>(ptr, w, n, acc, bid, nblk); break;
-      case 3: dots_chunk<3>(ptr, w, n, acc, bid, nblk); break;
-      case 4: dots_chunk<4>(ptr, w, n, acc, bid, nblk); break;
-      case 5: dots_chunk<5>(ptr, w, n, acc, bid, nblk); break;
-      case 6: dots_chunk<6>(ptr, w, n, acc, bid, nblk); break;
-      case 7: dots_chunk<7>(ptr, w, n, acc, bid, nblk); break;
-      default: dots_chunk<8>(ptr, w, n, acc, bid, nblk); break;
-    }
-    // Warp sums of the (up to) 8 values by recursive halving: each exchange
-    // sends half of the values still held to the partner lane and keeps the
-    // other half, so lane l ends with the warp sum of value
-    // 4 b4 + 2 b3 + b2 (b = bits of l) after 9 additions instead of 8 x 5.
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (i >= nc) acc[i] = 0.0;
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const double send = b4 ? acc[q] : acc[q + 4];
-      const double keep = b4 ? acc[q + 4] : acc[q];
-      acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const double send = b3 ? acc[q] : acc[q + 2];
-      const double keep = b3 ? acc[q + 2] : acc[q];
-      acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    {
-      const double send = b2 ? acc[0] : acc[1];
-      const double keep = b2 ? acc[1] : acc[0];
-      acc[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
-    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-    const int vi = (b4 ? 4 : 0) + (b3 ? 2 : 0) + (b2 ? 1 : 0);
-    if ((lane & 3) == 0 && vi < nc) sred[vi][wid] = acc[0];
-    __syncthreads();
-    if ((int)threadIdx.x < nc) {
-      double t = 0.0;
-      for (int q = 0; q < nw; ++q) t += sred[threadIdx.x][q];
-      red.partials[(size_t)bid * kMaxVec + c0 + threadIdx.x] = t;
-    }
-    __syncthreads();
-  }
-  if (last_block(red.counter, nblk)) finish_sums(red, total, out, nblk);
 }
 
 __global__ void __launch_bounds__(256) k_dots(const double* __restrict__ V, long long ldv, int nvec,
@@ -198,68 +79,6 @@ __global__ void __launch_bounds__(256) k_dots(const double* __restrict__ V, long
                                               int with_self, Reduce red, const int* done,
                                               const int* gate) {
   dots_body(V, ldv, nvec, w, n, out, with_self, red, done, gate, blockIdx.x, gridDim.x);
-}
-
-// w -= sum_i h_i V_i as one FMA chain per row (exactly nvec FP64 FMAs); optional sum of
-// squares of the new w.  With `self2` (the first Gram-Schmidt pass) the last
-// block also decides whether iteration j needs the second pass: it does when
-// ||w_new|| < eta ||w_old|| (the test of Daniel, Gragg, Kaufman and Stewart;
-// one classical pass leaves an orthogonality error of about
-// u ||w_old|| / ||w_new||, so eta = 1/64 keeps it below ~64 u), recorded in
-// rflag[j]; otherwise h2 is cleared.
-struct Reorth {
-  const double* self2;  // ||w||^2 before the first pass, or nullptr
-  double eta2;          // second pass when ||w_new||^2 < eta2 ||w_old||^2
-  int* rflag;           // &rflag[j]
-  double* h2;
-};
-
-__device__ __forceinline__ void update_body(double* __restrict__ w, const double* __restrict__ V,
-                                            long long ldv, int nvec, const double* h,
-                                            long long n, double* sumsq, const Reduce& red,
-                                            const int* done, const int* gate, const Reorth& ro,
-                                            int bid, int nblk) {
-  __shared__ double sh[32];
-  __shared__ double hs[kMaxVec];
-  if ((done && *done) || (gate && !*gate)) return;
-  if (threadIdx.x < nvec) hs[threadIdx.x] = -h[threadIdx.x];
-  __syncthreads();
-  // four rows per thread in flight: four independent FMA chains of length nvec
-  constexpr int UR = 4;
-  double ss[UR] = {0.0, 0.0, 0.0, 0.0};
-  const long long S = (long long)nblk * blockDim.x;
-  for (long long r0 = (long long)bid * blockDim.x + threadIdx.x; r0 < n; r0 += UR * S) {
-    double v[UR];
-#pragma unroll
-    for (int u = 0; u < UR; ++u) v[u] = (r0 + u * S < n) ? w[r0 + u * S] : 0.0;
-    for (int i = 0; i < nvec; ++i) {
-      const double hi = hs[i];
-      const double* Vi = V + i * ldv;
-#pragma unroll
-      for (int u = 0; u < UR; ++u)
-        if (r0 + u * S < n) v[u] = fma(hi, Vi[r0 + u * S], v[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < UR; ++u) {
-      if (r0 + u * S < n) {
-        w[r0 + u * S] = v[u];
-        if (sumsq) ss[u] = fma(v[u], v[u], ss[u]);
-      }
-    }
-  }
-  if (sumsq) {
-    const double bs = block_sum((ss[0] + ss[1]) + (ss[2] + ss[3]), sh);
-    if (threadIdx.x == 0) red.partials[(size_t)bid * kMaxVec] = bs;
-    if (last_block(red.counter, nblk)) {
-      finish_sums(red, 1, sumsq, nblk);
-      if (ro.self2 && threadIdx.x == 0) {
-        const int need = (*sumsq < ro.eta2 * *ro.self2) ? 1 : 0;
-        *ro.rflag = need;
-        if (!need)
-          for (int q = 0; q < nvec; ++q) ro.h2[q] = 0.0;
-      }
-    }
-  }
 }
 
 __global__ void __launch_bounds__(256) k_update(double* __restrict__ w, const double* __restrict__ V,
@@ -290,74 +109,15 @@ __global__ void k_cycle_init(GmresDev gd, const double* nr2, const double* nb2, 
   gd.invh[0] = beta > 0.0 ? 1.0 / beta : 0.0;
 }
 
-// Hessenberg column j, Givens rotations, residual estimate, convergence.
-// One warp: the lanes bring the column's Gram-Schmidt coefficients and the
-// earlier rotations into shared memory together (one round of independent
-// loads instead of a chain of dependent ones), lane 0 applies the rotations
-// in order, and the lanes write the column back.
-__device__ __forceinline__ void givens_body(const GmresDev& gd, int j, const double* nw2) {
-  __shared__ double hs[kMaxVec + 1], cs_s[kMaxVec], sn_s[kMaxVec];
-  if (*gd.done) return;
-  const int lane = threadIdx.x & 31;
-  for (int i = lane; i <= j; i += 32) hs[i] = gd.h1[i] + gd.h2[i];
-  for (int i = lane; i < j; i += 32) {
-    cs_s[i] = gd.cs[i];
-    sn_s[i] = gd.sn[i];
-  }
-  __syncwarp();
-  if (lane == 0) {
-    const double hn = sqrt(*nw2);
-    hs[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-      const double t = cs_s[i] * hs[i] + sn_s[i] * hs[i + 1];
-      hs[i + 1] = -sn_s[i] * hs[i] + cs_s[i] * hs[i + 1];
-      hs[i] = t;
-    }
-    const double den = hypot(hs[j], hs[j + 1]);
-    const double c = den > 0.0 ? hs[j] / den : 1.0;
-    const double s = den > 0.0 ? hs[j + 1] / den : 0.0;
-    gd.cs[j] = c;
-    gd.sn[j] = s;
-    hs[j] = den;
-    hs[j + 1] = 0.0;
-    gd.g[j + 1] = -s * gd.g[j];
-    gd.g[j] = c * gd.g[j];
-    *gd.k = j + 1;
-    const double res = fabs(gd.g[j + 1]);
-    *gd.res = res;
-    gd.invh[j + 1] = hn > 0.0 ? 1.0 / hn : 0.0;
-    if (res <= *gd.target || hn == 0.0 || !(res == res)) *gd.done = 1;
-  }
-  __syncwarp();
-  double* Hj = gd.H + (size_t)j * gd.ldh;
-  for (int i = lane; i <= j + 1; i += 32) Hj[i] = hs[i];
-}
-
 __global__ void k_givens(GmresDev gd, int j, const double* nw2) {
   givens_body(gd, j, nw2);
 }
 
-// y = H(0:k,0:k)^{-1} g(0:k); one warp loads the triangle, lane 0 solves
 __global__ void k_backsub(GmresDev gd) {
-  __shared__ double Hs[kMaxVec][kMaxVec];
-  __shared__ double ys[kMaxVec];
+  __shared__ double Hs[kTriangle], ys[kMaxVec];
   const int k = *gd.k;
-  const int lane = threadIdx.x & 31;
-  for (int idx = lane; idx < k * k; idx += 32) {
-    const int l = idx / k, i = idx % k;   // column l, row i
-    if (i <= l) Hs[l][i] = gd.H[(size_t)l * gd.ldh + i];
-  }
-  for (int i = lane; i < k; i += 32) ys[i] = gd.g[i];
-  __syncwarp();
-  if (lane == 0) {
-    for (int i = k - 1; i >= 0; --i) {
-      double s = ys[i];
-      for (int l = i + 1; l < k; ++l) s -= Hs[l][i] * ys[l];
-      ys[i] = s / Hs[i][i];
-    }
-  }
-  __syncwarp();
-  for (int i = lane; i < k; i += 32) gd.y[i] = ys[i];
+  backsub(gd, k, Hs, ys);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) gd.y[i] = ys[i];
 }
 
 // cycle status for the host: [k, |g_k|, rtol ||b||, ||b||]; marks the
@@ -517,7 +277,7 @@ int gmres_cycle_prologue(fr_ctx* ctx, const double* U, const double* R0, double 
 
 int gmres_cycle_epilogue(fr_ctx* ctx, double* x, double* status, int* fin, cudaStream_t s) {
   GmresDev& gd = ctx->gd;
-  { ProfScope ps_(ctx, FR_KF_OTHER, s); k_backsub<<<1, 32, 0, s>>>(gd); }
+  { ProfScope ps_(ctx, FR_KF_OTHER, s); k_backsub<<<1, 256, 0, s>>>(gd); }
   FRK_LAUNCHED(ctx);
   FRK_TRY(launch_solution_update(ctx, x, s));
   { ProfScope ps_(ctx, FR_KF_OTHER, s); k_status<<<1, 32, 0, s>>>(gd, ctx->scal + S_NB2, status, fin, ctx->kerr); }
@@ -549,9 +309,101 @@ int gmres_cycle_enqueue(fr_ctx* ctx, const double* U, const double* R0, double s
   return gmres_cycle_epilogue(ctx, x, status, fin, s);
 }
 
+// Solves of 2D Euler contexts with element blocks and up to kCycleMaxDof unknowns
+// run as one launch; per-family timing and the apply's wait test need the
+// separate launches.  The line lies where the launches stop costing more than the
+// barriers: a ROW3 step at p = 3 takes 10.7 ms against 11.9 ms by launches at
+// 102,400 unknowns, 29.8 against 29.5 ms (BF16) and 38.8 against 38.3 ms (FP64
+// blocks) at 262,144, and 170 against 131 ms at 1,638,400, where the staged apply
+// and four CTAs per SM win; the 14,400-unknown ROW2 step takes 2.9 against 5.2 ms.
+constexpr long long kCycleMaxDof = 200000;
+
+bool cycle_supported(const fr_ctx* ctx) {
+  return !ctx->dim3 && !ctx->viscous && ctx->opts.jv_precision == 0 && ctx->opts.precond && ctx->p >= 2 && ctx->p <= 4 &&
+         ctx->ndof <= kCycleMaxDof && ctx->prof.mask == 0 && !ctx->test_skip_copy && cycle_grid(ctx) > 0;
+}
+
+// one CTA per SM while a barrier costs more than the phases between, two above
+// (14,400 unknowns: 2.9 against 3.5 ms; 102,400: 11.0 against 10.7 ms)
+int cycle_grid(const fr_ctx* ctx) {
+  int occ = 0;
+  switch (ctx->opts.block_precision) {
+    case 1: occ = resident_cycle_f32(ctx->opts.riemann); break;
+    case 2: occ = resident_cycle_bf16(ctx->opts.riemann); break;
+    default: occ = resident_cycle_f64(ctx->opts.riemann); break;
+  }
+  const int want = ctx->ndof <= 60000 ? 1 : 2;
+  return (occ < want ? occ : want) * ctx->num_sms;
+}
+
+int launch_cycle(int prec, const CycleArgs& a, int nblocks, int riemann, cudaStream_t s) {
+  switch (prec) {
+    case 1: return launch_cycle_f32(a, nblocks, riemann, s);
+    case 2: return launch_cycle_bf16(a, nblocks, riemann, s);
+    default: return launch_cycle_f64(a, nblocks, riemann, s);
+  }
+}
+
+int fill_cycle_args(fr_ctx* ctx, const double* U, const double* R0, double shift, double rtol, int m, int max_restarts,
+                    CycleArgs* a) {
+  *a = CycleArgs{};
+  a->res = residual_args(ctx, U, R0, shift);
+  a->p = ctx->p;
+  a->small_tile = residual_small_tile(ctx);
+  a->Minv = ctx->blocks;
+  a->V = ctx->V;
+  a->z = ctx->z;
+  a->n = ctx->ndof;
+  a->ne = ctx->ne;
+  a->red = ctx->red;
+  a->gd = ctx->gd;
+  a->eta2 = ctx->opts.reorth_eta * ctx->opts.reorth_eta;
+  a->rtol = rtol;
+  a->m = m;
+  a->max_restarts = max_restarts;
+  a->vgrid = (int)vgrid(ctx, ctx->ndof);
+  a->agrid = (int)apply_grid_of(ctx);
+  a->bar = ctx->cyc_bar;
+  a->err = ctx->kerr;
+  a->status = ctx->h_cyc;
+  return a->agrid > 0 ? FR_OK : FR_ERR_UNSUPPORTED;
+}
+
+namespace {
+int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x, int m,
+                     double rtol, int max_restarts, bool x_is_zero, fr_gmres_info* info, cudaStream_t s) {
+  CycleArgs a;
+  FRK_TRY(fill_cycle_args(ctx, U, R0, shift, rtol, m, max_restarts, &a));
+  a.b = b;
+  a.x = x;
+  a.x_zero = x_is_zero;
+  if (launch_cycle(ctx->opts.block_precision, a, cycle_grid(ctx), ctx->opts.riemann, s) !=
+      FR_OK)
+    return set_error(ctx, FR_ERR_CUDA, "launch of the solve failed: %s", cudaGetErrorString(cudaGetLastError()));
+  FRK_CUDA(ctx, cudaStreamSynchronize(s));
+  const CycleStatus& st = *ctx->h_cyc;
+  if (st.state == kCycleTimeout) return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
+  if (st.state == kCycleNonFinite) {
+    if (info) *info = fr_gmres_info{};
+    return set_error(ctx, FR_ERR_NONFINITE, "GMRES residual is not finite");
+  }
+  fr_gmres_info loc{};
+  loc.iters = st.iters;
+  loc.restarts = st.restarts;
+  loc.converged = st.state == kCycleConverged;
+  loc.relres = st.relres;
+  if (info) *info = loc;
+  if (!loc.converged)
+    return set_error(ctx, FR_ERR_NOT_CONVERGED, "GMRES stopped after %d iterations at relres %.3e", loc.iters, loc.relres);
+  return FR_OK;
+}
+}  // namespace
+
 int gmres_impl(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b,
                double* x, int m, double rtol, int max_restarts, bool x_is_zero,
                fr_gmres_info* info, cudaStream_t s) {
+  if (cycle_supported(ctx))
+    return gmres_one_launch(ctx, U, R0, shift, b, x, m, rtol, max_restarts, x_is_zero, info, s);
   const long long n = ctx->ndof;
   double* sc = ctx->scal;
   GmresDev& gd = ctx->gd;
@@ -624,7 +476,7 @@ int gmres_impl(fr_ctx* ctx, const double* U, const double* R0, double shift, con
         if (ctx->h_stat[2 + prev]) break;
       }
     }
-    { ProfScope ps_(ctx, FR_KF_OTHER, s); k_backsub<<<1, 32, 0, s>>>(gd); }
+    { ProfScope ps_(ctx, FR_KF_OTHER, s); k_backsub<<<1, 256, 0, s>>>(gd); }
     FRK_LAUNCHED(ctx);
     FRK_TRY(launch_solution_update(ctx, x, s));
     FRK_CUDA(ctx, cudaMemcpyAsync(ctx->h_stat, gd.k, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -475,7 +475,7 @@ __global__ void k_loss_grad(const float* __restrict__ y, const float* __restrict
     s += 0.5 * (double)e * (double)e;
   }
   const double bs = block_sum(s, sh);
-  if (threadIdx.x == 0) red.partials[(size_t)blockIdx.x * kMaxVec] = bs;
+  if (threadIdx.x == 0) red.value(0)[blockIdx.x] = bs;
   if (last_block(red.counter)) {
     finish_sums(red, 1, loss);
     if (threadIdx.x == 0) *loss /= (double)n;

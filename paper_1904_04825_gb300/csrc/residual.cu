@@ -17,274 +17,16 @@
 // A z with its two norms take 2241 us together; with IEEE divisions, roots and
 // fmax in the fluxes, two divisions per thread for the metric and one load in
 // flight in the norms they took 2718 us.
-#include "device.cuh"
+#include "residual_body.cuh"
 
 namespace frk {
 namespace {
 
-struct ResArgs {
-  const double* U;
-  const double* z;
-  const double* R0;
-  const double* b;
-  double* out;
-  const double* sx;    // 2 / hx per element column
-  const double* sy;    // 2 / hy per element row
-  const double* eps2;  // (eps, 1/eps) of the FD product
-  const int* done;
-  long long ne;
-  int nx, ny;
-  double gam;
-  double shift;
-  double eps_rel;
-  double eps_fixed;
-  double* lin_fg;  // mode 3 writes / mixed A z reads: F(U), G(U) [ne][8][NP]
-  double* lin_fx;  // per element's west face point: q-, q+, f^num (4 each) [ne][N][12]
-  double* lin_fy;  // per element's south face point, same layout
-  int riemann;     // common flux: 0 Rusanov, 1 Roe
-  Tables tab;
-};
-
-// sum_k c[k] * x[k*stride], fixed order, explicit FMAs
-template <int N>
-__device__ __forceinline__ double trace_sum(const double* __restrict__ x, int stride,
-                                            const double* c) {
-  double s = c[0] * x[0];
-#pragma unroll
-  for (int k = 1; k < N; ++k) s = fma(c[k], x[k * stride], s);
-  return s;
-}
-
-// neighbour trace from global memory, optionally perturbed by eps * z
-template <int N, bool PERTURB>
-__device__ __forceinline__ double trace_global(const double* __restrict__ U,
-                                               const double* __restrict__ z, long long off,
-                                               int stride, const double* c, double eps) {
-  if (!PERTURB) return trace_sum<N>(U + off, stride, c);
-  double s = c[0] * fma(eps, z[off], U[off]);
-#pragma unroll
-  for (int k = 1; k < N; ++k) s = fma(c[k], fma(eps, z[off + k * stride], U[off + k * stride]), s);
-  return s;
-}
-
-// Element tile handled by one CTA (TX x TY elements, one thread per point);
-// two shapes per degree, picked at run time by the autotuner.
-template <int P, int V> struct Tile;
-template <> struct Tile<2, 0> { static constexpr int TX = 5, TY = 5; };
-template <> struct Tile<2, 1> { static constexpr int TX = 7, TY = 4; };
-template <> struct Tile<3, 0> { static constexpr int TX = 4, TY = 4; };
-template <> struct Tile<3, 1> { static constexpr int TX = 8, TY = 2; };
-template <> struct Tile<4, 0> { static constexpr int TX = 3, TY = 3; };
-template <> struct Tile<4, 1> { static constexpr int TX = 5, TY = 2; };
-template <> struct Tile<5, 0> { static constexpr int TX = 2, TY = 3; };
-template <> struct Tile<5, 1> { static constexpr int TX = 3, TY = 2; };
-template <> struct Tile<6, 0> { static constexpr int TX = 2, TY = 2; };
-template <> struct Tile<6, 1> { static constexpr int TX = 5, TY = 1; };
-// Shape 2: small meshes, whose shape-0 tiles would leave most SMs idle (see use_small_tile).
-template <> struct Tile<2, 2> { static constexpr int TX = 2, TY = 2; };
-template <> struct Tile<3, 2> { static constexpr int TX = 2, TY = 2; };
-template <> struct Tile<4, 2> { static constexpr int TX = 2, TY = 1; };
-template <> struct Tile<5, 2> { static constexpr int TX = 2, TY = 1; };
-template <> struct Tile<6, 2> { static constexpr int TX = 1, TY = 1; };
-
 template <int P, int MODE, int TV, int RM>
-__device__ __forceinline__ void residual_body(const ResArgs& a, double* __restrict__ out, int bid) {
-  constexpr int N = P + 1, NP = N * N;
-  constexpr int TX = Tile<P, TV>::TX, TY = Tile<P, TV>::TY, NE = TX * TY;
-  constexpr int NXF = (TX + 1) * TY * N;  // points on the tile's x-faces (normal +x)
-  constexpr int NYF = (TY + 1) * TX * N;  // points on the tile's y-faces (normal +y)
-  constexpr bool PERTURB = MODE == 1 || MODE == 2;  // MODE 3: R's fluxes at U into the caches
-  // MODE 3 feeds the FP32-linear-parts product, which repeats its fluxes with
-  // the correctly rounded operations; the others take the fast ones, whose
-  // common flux comes out doubled (sdgL, sdgR carry the 1/2)
-  constexpr bool FAST = MODE != 3;
-  __shared__ double sq[NE][4][NP];
-  __shared__ double sF[NE][4][NP];
-  __shared__ double sG[NE][4][NP];
-  __shared__ double str[NE][4][4][N];       // own traces [face W,E,S,N][var][k]
-  __shared__ double shx[2][TY][4][N];       // outside traces on the tile's west / east faces
-  __shared__ double shy[2][TX][4][N];       // outside traces on the tile's south / north faces
-  __shared__ double sfx[TY][TX + 1][4][N];  // common flux f_n on x-face xf of tile row ly
-  __shared__ double sfy[TX][TY + 1][4][N];  // common flux g_n on y-face yf of tile column lx
-  __shared__ double sDt[N][N], slm[N], slp[N], sdgL[N], sdgR[N];
-  constexpr int NOWN = NE * 4 * N;           // own-trace work items
-  constexpr int NHALO = 2 * (TX + TY) * N;   // outside-trace work items
-
+__global__ void __launch_bounds__(TV == 2 ? 128 : 256, 4) k_residual(const __grid_constant__ ResArgs a) {
+  __shared__ ResSmem<P, TV> sm;
   if (a.done && *a.done) return;
-  if (threadIdx.x < N * N) sDt[threadIdx.x / N][threadIdx.x % N] = a.tab.Dt[threadIdx.x / N][threadIdx.x % N];
-  if (threadIdx.x < N) {
-    slm[threadIdx.x] = a.tab.lm[threadIdx.x];
-    slp[threadIdx.x] = a.tab.lp[threadIdx.x];
-    sdgL[threadIdx.x] = 0.5 * a.tab.dgL[threadIdx.x];
-    sdgR[threadIdx.x] = 0.5 * a.tab.dgR[threadIdx.x];
-  }
-
-  const int tiles_x = (a.nx + TX - 1) / TX;
-  const int ix0 = (int)(bid % tiles_x) * TX, iy0 = (int)(bid / tiles_x) * TY;
-  const int ax = min(TX, a.nx - ix0), ay = min(TY, a.ny - iy0);  // active tile extent
-  const int el = threadIdx.x / NP, t = threadIdx.x % NP;
-  const int lx = el % TX, ly = el / TX;
-  const bool active = el < NE && lx < ax && ly < ay;
-  const long long e = (long long)(ix0 + lx) + (long long)a.nx * (iy0 + ly);
-
-  double eps = 0.0, ieps = 0.0;
-  if (PERTURB) {
-    eps = a.eps2[0];
-    ieps = a.eps2[1];
-  }
-  // ---- 1: state (perturbed for A z) and pointwise fluxes ----
-  if (active) {
-    const long long base = e * 4 * NP + t;
-    double q[4], f[4], g[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const long long o = base + v * NP;
-      q[v] = PERTURB ? fma(eps, a.z[o], a.U[o]) : a.U[o];
-      sq[el][v][t] = q[v];
-    }
-    euler_fluxes<FAST>(q, a.gam, f, g);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      sF[el][v][t] = f[v];
-      sG[el][v][t] = g[v];
-      if (MODE == 3) {
-        a.lin_fg[(e * 8 + v) * NP + t] = f[v];
-        a.lin_fg[(e * 8 + 4 + v) * NP + t] = g[v];
-      }
-    }
-  }
-  __syncthreads();
-  // ---- 2a: own solution traces on the four faces of every tile element,
-  //      then (separate work items, starting on a warp boundary when NOWN is
-  //      a multiple of 32, so the FP64 work does not diverge) the outside
-  //      neighbours' traces on the tile's boundary faces, from global memory ----
-  for (int idx = threadIdx.x; idx < NOWN + NHALO; idx += blockDim.x) {
-    if (idx < NOWN) {
-      const int e2 = idx / (4 * N), face = (idx / N) % 4, k = idx % N;
-      if ((e2 % TX) >= ax || (e2 / TX) >= ay) continue;
-      const int off = face < 2 ? N * k : k;
-      const int stride = face < 2 ? 1 : N;
-      const double* c = (face == 0 || face == 2) ? slm : slp;
-#pragma unroll
-      for (int v = 0; v < 4; ++v) str[e2][face][v][k] = trace_sum<N>(&sq[e2][v][off], stride, c);
-    } else {
-      const int h = idx - NOWN, seg = h / N, k = h % N;
-      long long nb;
-      int off, stride;
-      const double* c;
-      double* dst;
-      if (seg < 2 * TY) {  // west (side 0) / east (side 1) boundary of tile row fy
-        const int side = seg / TY, fy = seg % TY;
-        if (fy >= ay) continue;
-        const int gx = side == 0 ? (ix0 + a.nx - 1) % a.nx : (ix0 + ax) % a.nx;
-        nb = (long long)gx + (long long)a.nx * (iy0 + fy);
-        off = N * k;
-        stride = 1;
-        c = side == 0 ? slp : slm;  // the west neighbour's east trace, the east one's west trace
-        dst = &shx[side][fy][0][k];
-      } else {             // south (side 0) / north (side 1) boundary of tile column fx
-        const int s2 = seg - 2 * TY, side = s2 / TX, fx = s2 % TX;
-        if (fx >= ax) continue;
-        const int gy = side == 0 ? (iy0 + a.ny - 1) % a.ny : (iy0 + ay) % a.ny;
-        nb = (long long)(ix0 + fx) + (long long)a.nx * gy;
-        off = k;
-        stride = N;
-        c = side == 0 ? slp : slm;
-        dst = &shy[side][fx][0][k];
-      }
-#pragma unroll
-      for (int v = 0; v < 4; ++v)
-        dst[v * N] = trace_global<N, PERTURB>(a.U, a.z, nb * 4 * NP + v * NP + off, stride, c, eps);
-    }
-  }
-  __syncthreads();
-  // ---- 2b: one Rusanov flux per face point, both traces from shared memory ----
-  for (int idx = threadIdx.x; idx < NXF + NYF; idx += blockDim.x) {
-    double qm[4], qp[4], fc[4];
-    if (idx < NXF) {
-      const int k = idx % N, rr = idx / N, xf = rr % (TX + 1), fy = rr / (TX + 1);
-      if (fy >= ay || xf > ax) continue;
-      const int gy = iy0 + fy;
-      const double* pm = xf >= 1 ? &str[xf - 1 + TX * fy][1][0][k] : &shx[0][fy][0][k];
-      const double* pp = xf < ax ? &str[xf + TX * fy][0][0][k] : &shx[1][fy][0][k];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        qm[v] = pm[v * N];
-        qp[v] = pp[v * N];
-      }
-      if (FAST) riemann_flux2(RM, qm, qp, 0, a.gam, fc);
-      else riemann_flux(RM, qm, qp, 0, a.gam, fc);
-#pragma unroll
-      for (int v = 0; v < 4; ++v) sfx[fy][xf][v][k] = fc[v];
-      if (MODE == 3 && xf < ax) {  // the west face of tile element xf
-        double* c = a.lin_fx + (((long long)(ix0 + xf) + (long long)a.nx * gy) * N + k) * 12;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          c[v] = qm[v];
-          c[4 + v] = qp[v];
-          c[8 + v] = fc[v];
-        }
-      }
-    } else {
-      const int i2 = idx - NXF;
-      const int k = i2 % N, rr = i2 / N, yf = rr % (TY + 1), fx = rr / (TY + 1);
-      if (fx >= ax || yf > ay) continue;
-      const int gx = ix0 + fx;
-      const double* pm = yf >= 1 ? &str[fx + TX * (yf - 1)][3][0][k] : &shy[0][fx][0][k];
-      const double* pp = yf < ay ? &str[fx + TX * yf][2][0][k] : &shy[1][fx][0][k];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        qm[v] = pm[v * N];
-        qp[v] = pp[v * N];
-      }
-      if (FAST) riemann_flux2(RM, qm, qp, 1, a.gam, fc);
-      else riemann_flux(RM, qm, qp, 1, a.gam, fc);
-#pragma unroll
-      for (int v = 0; v < 4; ++v) sfy[fx][yf][v][k] = fc[v];
-      if (MODE == 3 && yf < ay) {  // the south face of tile element yf
-        double* c = a.lin_fy + ((long long)gx + (long long)a.nx * (iy0 + yf)) * N * 12 + k * 12;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          c[v] = qm[v];
-          c[4 + v] = qp[v];
-          c[8 + v] = fc[v];
-        }
-      }
-    }
-  }
-  __syncthreads();
-
-  // ---- 3: corrected divergence and the output ----
-  if (MODE == 3 || !active) return;
-  const int i = t % N, j = t / N;
-  // with unscaled fluxes, -(1/|J|)(dF~/dxi + dG~/deta) = -(2/hx) df~ - (2/hy) dg~
-  const double sx = a.sx[ix0 + lx], sy = a.sy[iy0 + ly];
-  const long long base = e * 4 * NP + t;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    double dF = sdgL[i] * sfx[ly][lx][v][j];
-    dF = fma(sdgR[i], sfx[ly][lx + 1][v][j], dF);
-#pragma unroll
-    for (int k = 0; k < N; ++k) dF = fma(sDt[i][k], sF[el][v][k + N * j], dF);
-    double dG = sdgL[j] * sfy[lx][ly][v][i];
-    dG = fma(sdgR[j], sfy[lx][ly + 1][v][i], dG);
-#pragma unroll
-    for (int k = 0; k < N; ++k) dG = fma(sDt[j][k], sG[el][v][i + N * k], dG);
-    const double R = -fma(sx, dF, sy * dG);
-    const long long o = base + v * NP;
-    if (MODE == 0) {
-      out[o] = R;
-    } else {
-      const double zo = a.z[o];
-      const double Az = eps > 0.0 ? fma(-(R - a.R0[o]), ieps, a.shift * zo) : a.shift * zo;
-      out[o] = MODE == 2 ? a.b[o] - Az : Az;
-    }
-  }
-}
-
-template <int P, int MODE, int TV, int RM>
-__global__ void __launch_bounds__(256, 4) k_residual(const ResArgs a) {
-  residual_body<P, MODE, TV, RM>(a, a.out, blockIdx.x);
+  residual_body<P, MODE, TV, RM>(a, a.z, a.b, a.eps2, a.out, blockIdx.x, sm);
 }
 
 // A z of Arnoldi iteration j of every instance (of one degree) in one grid:
@@ -296,7 +38,9 @@ __global__ void __launch_bounds__(256, 4) kb_residual(const ResArgs* __restrict_
   const int k = batch_instance(start, ninst, blockIdx.x);
   const ResArgs& a = tab[k];
   const long long ndof = a.ne * 4 * (P + 1) * (P + 1);
-  residual_body<P, 1, 0, RM>(a, a.out + (size_t)(j + 1) * ndof, blockIdx.x - start[k]);
+  __shared__ ResSmem<P, 0> sm;
+  if (*a.done) return;
+  residual_body<P, 1, 0, RM>(a, a.z, nullptr, a.eps2, a.out + (size_t)(j + 1) * ndof, blockIdx.x - start[k], sm);
 }
 
 // A z with FP32 linear parts (jv_precision 1).  R(U+eps z) - R(U) is the
@@ -530,20 +274,35 @@ int launch_p(fr_ctx* ctx, int mode, const ResArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-int launch_residual(fr_ctx* ctx, int mode, const double* U, const double* z, const double* R0,
-                    const double* b, double* out, double shift, const double* eps2,
-                    const int* done, cudaStream_t s) {
-  if (ctx->dim3) return launch_f3_residual(ctx, mode, U, z, R0, b, out, shift, eps2, done, s);
-  if (ctx->viscous) return launch_ns_residual(ctx, mode, U, z, R0, b, out, shift, eps2, done, s);
-  ResArgs a;
-  a.U = U; a.z = z; a.R0 = R0; a.b = b; a.out = out;
-  a.sx = ctx->sx; a.sy = ctx->sy; a.eps2 = eps2; a.done = done;
+ResArgs residual_args(fr_ctx* ctx, const double* U, const double* R0, double shift) {
+  ResArgs a{};
+  a.U = U; a.R0 = R0;
+  a.sx = ctx->sx; a.sy = ctx->sy;
   a.ne = ctx->ne; a.nx = ctx->nx; a.ny = ctx->ny;
   a.gam = ctx->opts.gamma; a.shift = shift;
   a.eps_rel = ctx->opts.eps_rel; a.eps_fixed = ctx->opts.eps_fixed;
   a.lin_fg = ctx->lin_fg; a.lin_fx = ctx->lin_fx; a.lin_fy = ctx->lin_fy;
   a.riemann = ctx->opts.riemann;
   a.tab = ctx->tab;
+  return a;
+}
+
+bool residual_small_tile(const fr_ctx* ctx) {
+  switch (ctx->p) {
+    case 2: return use_small_tile<2>(ctx, 1);
+    case 3: return use_small_tile<3>(ctx, 1);
+    case 4: return use_small_tile<4>(ctx, 1);
+    default: return false;
+  }
+}
+
+int launch_residual(fr_ctx* ctx, int mode, const double* U, const double* z, const double* R0,
+                    const double* b, double* out, double shift, const double* eps2,
+                    const int* done, cudaStream_t s) {
+  if (ctx->dim3) return launch_f3_residual(ctx, mode, U, z, R0, b, out, shift, eps2, done, s);
+  if (ctx->viscous) return launch_ns_residual(ctx, mode, U, z, R0, b, out, shift, eps2, done, s);
+  ResArgs a = residual_args(ctx, U, R0, shift);
+  a.z = z; a.b = b; a.out = out; a.eps2 = eps2; a.done = done;
   switch (ctx->p) {
     case 2: return launch_p<2>(ctx, mode, a, s);
     case 3: return launch_p<3>(ctx, mode, a, s);
@@ -572,15 +331,9 @@ unsigned residual_grid_of(const fr_ctx* ctx) {
 // context's preconditioned vector, output base = the Krylov basis
 int fill_batch_residual(fr_ctx* ctx, const double* U, const double* R0, double shift, void* out) {
   if (ctx->dim3 || ctx->viscous || ctx->opts.jv_precision != 0 || ctx->p < 2 || ctx->p > 4) return FR_ERR_UNSUPPORTED;
-  ResArgs a{};
-  a.U = U; a.z = ctx->z; a.R0 = R0; a.b = nullptr; a.out = ctx->V;
-  a.sx = ctx->sx; a.sy = ctx->sy; a.eps2 = ctx->scal + S_EPS; a.done = ctx->gd.done;
-  a.ne = ctx->ne; a.nx = ctx->nx; a.ny = ctx->ny;
-  a.gam = ctx->opts.gamma; a.shift = shift;
-  a.eps_rel = ctx->opts.eps_rel; a.eps_fixed = ctx->opts.eps_fixed;
-  a.lin_fg = ctx->lin_fg; a.lin_fx = ctx->lin_fx; a.lin_fy = ctx->lin_fy;
-  a.riemann = ctx->opts.riemann;
-  a.tab = ctx->tab;
+  ResArgs a = residual_args(ctx, U, R0, shift);
+  a.z = ctx->z; a.out = ctx->V;
+  a.eps2 = ctx->scal + S_EPS; a.done = ctx->gd.done;
   *reinterpret_cast<ResArgs*>(out) = a;
   return FR_OK;
 }

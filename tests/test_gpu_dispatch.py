@@ -108,3 +108,86 @@ def test_training_step_at_tile_edges(fr, n_in, n_h, n_out, M):
     net.forward(Xd, Yb, bf16=True)
     Y, Yb = Y.cpu().numpy(), Yb.cpu().numpy()
     assert np.linalg.norm(Yb - Y) <= 3e-2 * np.linalg.norm(Y) + 1e-6
+
+
+@pytest.mark.parametrize("p,prec,riemann", [(2, 0, 0), (3, 0, 1), (4, 0, 0), (2, 2, 1), (3, 1, 0), (3, 2, 0), (4, 1, 1)])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (5, 7), (40, 11), (61, 50)])
+def test_one_launch_solve_equals_the_launches(fr, p, prec, riemann, nx, ny):
+    """Small 2D Euler solves run as one launch; with a family being timed they run as the separate
+    launches.  Both sum in the same order: the same iterations and the same bits, from a zero guess,
+    from a nonzero one, over restarts, with both Gram-Schmidt passes forced, and for a zero
+    right-hand side."""
+    import torch
+    xe, ye = S.stretched_mesh(nx, ny, seed=p)
+    X, Y = S.point_coords(xe, ye, p)
+    U = _t(S.smooth_random_state(X, Y, seed=nx, amp=0.05))
+    for eta in (1.0 / 64.0, 1.0):
+        ctx = fr.Context(xe, ye, p, fr.default_opts(riemann=riemann, block_precision=prec, reorth_eta=eta))
+        R0 = ctx.empty()
+        fr.fr_residual(ctx, U, R0)
+        fr.ejacobi_factor(ctx, U, R0, 4.0)
+        b, x1 = _t(S.random_vector(U.shape, 1)), _t(S.random_vector(U.shape, 2))
+        for rhs, x0, m, rtol, restarts in ((b, torch.zeros_like(b), 30, 1e-8, 20), (b, 0.01 * x1, 30, 1e-7, 20),
+                                           (b, torch.zeros_like(b), 3, 1e-9, 4), (b, torch.zeros_like(b), 1, 1e-3, 0),
+                                           (torch.zeros_like(b), x1, 5, 1e-8, 2), (b, torch.zeros_like(b), 4, 2.0, 2)):
+            res = []
+            for timed in (False, True):
+                x = x0.clone()
+                if timed:
+                    fr.fr_profile_begin(ctx, ["dots"])
+                info = fr.gmres_solve(ctx, U, R0, 4.0, rhs, x, m=m, rtol=rtol, max_restarts=restarts)
+                if timed:
+                    fr.fr_profile_end(ctx)
+                res.append((x.cpu().numpy(), info))
+            assert res[0][1] == res[1][1]
+            assert np.array_equal(res[0][0], res[1][0])
+        ctx.close()
+
+
+def test_one_launch_solve_reports_non_finite_values(fr):
+    import torch
+    xe, ye = S.uniform_mesh(8)
+    X, Y = S.point_coords(xe, ye, 3)
+    U = _t(S.Vortex().state(X, Y))
+    ctx = fr.Context(xe, ye, 3)
+    R0 = ctx.empty()
+    fr.fr_residual(ctx, U, R0)
+    fr.ejacobi_factor(ctx, U, R0, 4.0)
+    b = _t(S.random_vector(U.shape, 1))
+    for bad in (np.nan, np.inf):
+        c = b.clone()
+        c.view(-1)[17] = bad
+        with pytest.raises(fr.FrError) as e:
+            fr.gmres_solve(ctx, U, R0, 4.0, c, torch.zeros_like(b))
+        assert e.value.code == fr.FR_ERR_NONFINITE
+    x = torch.zeros_like(b)   # the context still solves
+    assert fr.gmres_solve(ctx, U, R0, 4.0, b, x, rtol=1e-8).converged
+
+
+def test_solves_on_several_streams_and_threads(fr):
+    """Contexts on streams and threads of their own, their grids competing for the device."""
+    import threading
+    import torch
+    cs = []
+    for k in range(6):
+        n, p = 20 + 7 * k, 2 + k % 3
+        xe, ye = S.uniform_mesh(n)
+        X, Y = S.point_coords(xe, ye, p)
+        U = _t(S.Vortex(x0=0.2 * k).state(X, Y))
+        cs.append((fr.Context(xe, ye, p), U, U.clone(), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for ctx, U, V, s in cs:
+        fr.step_row(ctx, 3, 0.05, V)
+    torch.cuda.synchronize()
+
+    def work(ctx, U, s):
+        fr.step_row(ctx, 3, 0.05, U, stream=s.cuda_stream)
+
+    ts = [threading.Thread(target=work, args=(c, U, s)) for c, U, _, s in cs]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    for ctx, U, V, s in cs:
+        assert torch.equal(U, V)
