@@ -15,6 +15,7 @@
 
 #include "apply_body.cuh"
 #include "gj_cluster.cuh"
+#include "gj_fx.cuh"
 #include "gj_tc.cuh"
 
 namespace frk {
@@ -40,7 +41,9 @@ template <int P, typename T>
 struct FactorLayout {
   static constexpr int N = P + 1, NP = N * N, NB = 4 * NP, LD = NB + 1;
   static constexpr int THREADS = NB <= 64 ? 128 : 256;
-  // shared memory: doubles first, then the block (type T), its pivot column and pivots
+  static constexpr bool TC = gjtc::Use<T, NB>::value;       // inversion on the tensor cores
+  static constexpr bool FX = std::is_same<T, double>::value;  // ... with integer updates
+  // doubles of the state
   static constexpr int OFF_Q = 0;                       // 4 x NP state
   static constexpr int OFF_F = OFF_Q + 4 * NP;          // 4 x NP  (hy/2) f
   static constexpr int OFF_G = OFF_F + 4 * NP;          // 4 x NP  (hx/2) g
@@ -48,11 +51,19 @@ struct FactorLayout {
   static constexpr int OFF_NT = OFF_TR + 16 * N;        // neighbour traces [4][4][N]
   static constexpr int OFF_FN = OFF_NT + 16 * N;        // base common fluxes [4][4][N] (scaled)
   static constexpr int DOUBLES = OFF_FN + 16 * N;
-  static constexpr bool TC = gjtc::Use<T, NB>::value;  // inversion on the tensor cores
-  // block, pivot column and pivots, then (TC) the tensor-core scratch, 128-byte aligned
-  static constexpr size_t GJ_END = DOUBLES * sizeof(double) + (size_t)(NB * LD + NB) * sizeof(T) + NB * sizeof(int);
-  static constexpr size_t OFF_TC = (GJ_END + 127) / 128 * 128;
-  static constexpr size_t BYTES = TC ? OFF_TC + gjtc::Shape<NB>::BYTES : GJ_END + 64;
+  static constexpr size_t STATE = DOUBLES * sizeof(double);
+  static constexpr size_t up(size_t x) { return (x + 127) / 128 * 128; }
+  // FP64: the block, the pivots, then the state and, once the columns are formed,
+  // the inversion's scratch in its place (at p = 3 four CTAs fit an SM, three
+  // without); FP32: state, block, pivot column and pivots, tensor-core scratch
+  static constexpr size_t FXS = gjfx::Shape<NB, THREADS>::BYTES;
+  static constexpr size_t OFF_M = FX ? 0 : STATE;
+  static constexpr size_t OFF_PIV = OFF_M + (size_t)(NB * LD + (FX ? 0 : NB)) * sizeof(T);
+  static constexpr size_t OFF_STATE = FX ? up(OFF_PIV + NB * sizeof(int)) : 0;
+  static constexpr size_t OFF_SCRATCH = FX ? OFF_STATE : up(OFF_PIV + NB * sizeof(int));
+  static constexpr size_t BYTES = TC   ? OFF_SCRATCH + gjtc::Shape<NB>::BYTES
+                                  : FX ? OFF_STATE + (STATE > FXS ? STATE : FXS)
+                                       : OFF_PIV + NB * sizeof(int) + 64;
 };
 
 constexpr size_t kSmemMax = 227 * 1024;  // opt-in shared memory per CTA
@@ -65,8 +76,8 @@ __device__ __forceinline__ double tsum(const double* x, int stride, const double
   return s;
 }
 
-// In-place Gauss-Jordan inversion with partial (row) pivoting of the NB x NB
-// matrix M (row stride LD) in shared memory, by the whole CTA; col holds the
+// (FP32 blocks of more than 128 rows) In-place Gauss-Jordan inversion with partial (row)
+// pivoting of the NB x NB matrix M (row stride LD) in shared memory, by the whole CTA; col holds the
 // pivot column, piv the row exchanges (undone on the columns at the end).
 template <typename T, int NB, int LD>
 __device__ void gauss_jordan(T* M, T* col, int* piv) {
@@ -130,16 +141,17 @@ template <int P, typename T, typename S>
 __global__ void __launch_bounds__(FactorLayout<P, T>::THREADS) k_factor(const FactorArgs a) {
   using L = FactorLayout<P, T>;
   constexpr int N = L::N, NP = L::NP, NB = L::NB, LD = L::LD;
-  extern __shared__ double smem[];
+  extern __shared__ __align__(128) unsigned char smem_f[];
+  double* smem = reinterpret_cast<double*>(smem_f + L::OFF_STATE);
   double* q = smem + L::OFF_Q;
   double* F = smem + L::OFF_F;
   double* G = smem + L::OFF_G;
   double* tr = smem + L::OFF_TR;
   double* nt = smem + L::OFF_NT;
   double* fn = smem + L::OFF_FN;
-  T* M = reinterpret_cast<T*>(smem + L::DOUBLES);
-  T* col = M + NB * LD;
-  int* piv = reinterpret_cast<int*>(col + NB);
+  T* M = reinterpret_cast<T*>(smem_f + L::OFF_M);
+  T* col = M + NB * LD;  // FP32 only
+  int* piv = reinterpret_cast<int*>(smem_f + L::OFF_PIV);
 
   const long long e = blockIdx.x;
   const int ix = (int)(e % a.nx), iy = (int)(e / a.nx);
@@ -273,11 +285,19 @@ __global__ void __launch_bounds__(FactorLayout<P, T>::THREADS) k_factor(const Fa
   __syncthreads();
   S* out = reinterpret_cast<S*>(a.blocks) + e * (long long)NB * NB;
   if constexpr (L::TC) {
-    unsigned char* tcs = reinterpret_cast<unsigned char*>(smem) + L::OFF_TC;
+    unsigned char* tcs = smem_f + L::OFF_SCRATCH;
     const bool ok = gjtc::invert<NB, LD>(M, col, piv, tcs);
     if (!ok && threadIdx.x == 0) atomicExch(a.err, 1);
     // ---- store column-major: inverse(i, k) = M[pr[i]][ipr[k]] ----
     const int* ipr = reinterpret_cast<const int*>(tcs + gjtc::Shape<NB>::OFF_IPR);
+    for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
+      const int kk = idx / NB, ii = idx % NB;
+      out[idx] = StoreT<S>::to(M[piv[ii] * LD + ipr[kk]]);
+    }
+  } else if constexpr (L::FX) {
+    unsigned char* fxs = smem_f + L::OFF_SCRATCH;
+    gjfx::invert<NB, LD, L::THREADS>(M, piv, fxs);
+    const int* ipr = reinterpret_cast<const int*>(fxs + gjfx::Shape<NB, L::THREADS>::OFF_IPR);
     for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
       const int kk = idx / NB, ii = idx % NB;
       out[idx] = StoreT<S>::to(M[piv[ii] * LD + ipr[kk]]);
@@ -297,14 +317,18 @@ __global__ void __launch_bounds__(FactorLayout<P, T>::THREADS) k_factor(const Fa
 template <int NB, typename T>
 struct InvertLayout {
   static constexpr int LD = NB + 1;
+  static constexpr int THREADS = NB <= 64 ? 128 : 256;
   static constexpr bool TC = gjtc::Use<T, NB>::value;
+  static constexpr bool FX = std::is_same<T, double>::value;
   static constexpr size_t GJ_END = (size_t)(NB * LD + NB) * sizeof(T) + NB * sizeof(int);
   static constexpr size_t OFF_TC = (GJ_END + 127) / 128 * 128;
-  static constexpr size_t BYTES = TC ? OFF_TC + gjtc::Shape<NB>::BYTES : GJ_END + 64;
+  static constexpr size_t BYTES = TC   ? OFF_TC + gjtc::Shape<NB>::BYTES
+                                  : FX ? OFF_TC + gjfx::Shape<NB, THREADS>::BYTES
+                                       : GJ_END + 64;
 };
 
 template <int NB, typename T, typename S>
-__global__ void __launch_bounds__(256) k_invert(const double* __restrict__ mst, void* blocks, long long e0,
+__global__ void __launch_bounds__(InvertLayout<NB, T>::THREADS) k_invert(const double* __restrict__ mst, void* blocks, long long e0,
                                                 double dshift, int* err) {
   using L = InvertLayout<NB, T>;
   constexpr int LD = L::LD;
@@ -325,6 +349,14 @@ __global__ void __launch_bounds__(256) k_invert(const double* __restrict__ mst, 
     const bool ok = gjtc::invert<NB, LD>(M, col, piv, tcs);
     if (!ok && threadIdx.x == 0) atomicExch(err, 1);
     const int* ipr = reinterpret_cast<const int*>(tcs + gjtc::Shape<NB>::OFF_IPR);
+    for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
+      const int kk = idx / NB, ii = idx % NB;
+      out[idx] = StoreT<S>::to(M[piv[ii] * LD + ipr[kk]]);
+    }
+  } else if constexpr (L::FX) {
+    unsigned char* fxs = reinterpret_cast<unsigned char*>(smem_inv) + L::OFF_TC;
+    gjfx::invert<NB, LD, L::THREADS>(M, piv, fxs);
+    const int* ipr = reinterpret_cast<const int*>(fxs + gjfx::Shape<NB, L::THREADS>::OFF_IPR);
     for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
       const int kk = idx / NB, ii = idx % NB;
       out[idx] = StoreT<S>::to(M[piv[ii] * LD + ipr[kk]]);
@@ -824,7 +856,7 @@ int invert_nbts(fr_ctx* ctx, const double* mst, double dshift, long long e0, lon
   FRK_CUDA(ctx, cudaFuncSetAttribute(k_invert<NB, T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)bytes));
   { ProfScope ps_(ctx, FR_KF_INVERT, s, 0.0, 2.0 * NB * NB * (double)NB * (double)n);
-    k_invert<NB, T, S><<<(unsigned)n, NB <= 64 ? 128 : 256, bytes, s>>>(mst, ctx->blocks, e0, dshift, ctx->kerr); }
+    k_invert<NB, T, S><<<(unsigned)n, InvertLayout<NB, T>::THREADS, bytes, s>>>(mst, ctx->blocks, e0, dshift, ctx->kerr); }
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }

@@ -191,3 +191,43 @@ def test_solves_on_several_streams_and_threads(fr):
     torch.cuda.synchronize()
     for ctx, U, V, s in cs:
         assert torch.equal(U, V)
+
+
+@pytest.mark.parametrize("p,nx,ny", [(2, 3, 2), (3, 2, 5), (4, 3, 3), (5, 2, 2)])
+@pytest.mark.parametrize("scale", [1.0, 30.0])
+def test_fp64_block_inverse_against_the_oracle_solve(fr, p, nx, ny, scale):
+    """The FP64 element blocks' inverse (panels in FP64, updates in 57-bit integers) in states whose
+    variables, and so the blocks' rows and columns, differ by orders of magnitude: M^-1 r against the
+    oracle's solve with its own finite-difference blocks, at the tolerance of FP64 blocks (1e-6: the
+    difference quotients of step 1e-7; each side's columns carry 1e-16 / 1e-7 of the flux scale)."""
+    from oracle.fr2d import Mesh
+    from oracle.jfnk import ElementJacobi, Problem, element_blocks
+    xe, ye = S.stretched_mesh(nx, ny, seed=p)
+    X, Y = S.point_coords(xe, ye, p)
+    U = S.smooth_random_state(X, Y, seed=nx, amp=0.05, base=(1.0, 0.7, -0.4, 2.0 * scale))
+    ctx = fr.Context(xe, ye, p)
+    fr.ejacobi_factor(ctx, _t(U), None, 30.0)
+    r = S.random_vector(U.shape, 3)
+    r[:, 3] *= scale
+    z = ctx.empty()
+    fr.ejacobi_apply(ctx, _t(r), z)
+    want = ElementJacobi(element_blocks(Problem(Mesh(xe, ye), p), U, 30.0))(r)
+    got = z.cpu().numpy()
+    for v in range(4):
+        assert np.linalg.norm(got[:, v] - want[:, v]) < 1e-6 * np.linalg.norm(want[:, v])
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_fp64_block_inverse_keeps_non_finite_values_visible(fr, bad):
+    """A non-finite state in one element makes that element's preconditioned vector non-finite."""
+    xe, ye = S.uniform_mesh(6)
+    X, Y = S.point_coords(xe, ye, 3)
+    U = S.Vortex().state(X, Y)
+    U[7, 3, 2] = bad
+    ctx = fr.Context(xe, ye, 3)
+    fr.ejacobi_factor(ctx, _t(U), None, 30.0)
+    z = ctx.empty()
+    fr.ejacobi_apply(ctx, _t(S.random_vector(U.shape, 3)), z)
+    z = z.cpu().numpy()
+    assert not np.isfinite(z[7]).all()
+    assert np.isfinite(z[21]).all()
