@@ -19,7 +19,7 @@
 #include <new>
 
 #include "device.cuh"
-#include "umma_ws.cuh"
+#include "mlp_fused.cuh"
 
 struct fr_mlp {
   int n[4] = {0, 0, 0, 0};  // layer widths: in, hidden, hidden, out
@@ -743,6 +743,26 @@ extern "C" int fr_mlp_forward(fr_mlp* m, const float* X, int M, float* Y, int bf
       MLP_CUDA(m, cudaFuncSetAttribute(k_umma_gemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)umma::SMEM));
       attr = true;
+    }
+    // the whole network in one kernel where the call's widths and rows allow it (mlp_fused.cuh)
+    if (m->ws && mlpf::takes(m->n, X, Y, M)) {
+      MLP_CUDA(m, cudaFuncSetAttribute(mlpf::k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlpf::BYTES));
+      int sms = 0, dev = 0;
+      MLP_CUDA(m, cudaGetDevice(&dev));
+      MLP_CUDA(m, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      mlpf::Layers L;
+      for (int l = 0; l < 4; ++l) L.n[l] = m->n[l];
+      for (int l = 0; l < 3; ++l) {
+        L.kp[l] = m->kp[l];
+        L.bias[l] = m->P + off_b(m, l);
+      }
+      const int tiles = (M + umws::BM - 1) / umws::BM;
+      count_launch();
+      mlpf::k_mlp_fused<<<std::min(tiles, sms), mlpf::THREADS, mlpf::BYTES, s>>>(m->wmap[0], m->wmap[1], m->wmap[2], L, X, M,
+                                                                               Y, m->derr);
+      MLP_CUDA(m, cudaGetLastError());
+      MLP_CUDA(m, cudaMemcpyAsync(m->herr, m->derr, sizeof(int), cudaMemcpyDeviceToHost, s));
+      return FR_OK;
     }
     count_launch();
     k_f2bf_pad<<<grid_for((long long)M * m->kp[0]), 256, 0, s>>>(X, m->X16, M, m->n[0], m->kp[0]);

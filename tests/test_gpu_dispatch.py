@@ -231,3 +231,30 @@ def test_fp64_block_inverse_keeps_non_finite_values_visible(fr, bad):
     z = z.cpu().numpy()
     assert not np.isfinite(z[7]).all()
     assert np.isfinite(z[21]).all()
+
+
+@pytest.mark.parametrize("n_in,n_h,n_out", [(300, 256, 100), (320, 256, 128), (108, 64, 36), (20, 33, 7), (12, 130, 120), (4, 1, 1)])
+def test_network_inference_in_one_kernel_equals_the_layer_kernels(fr, n_in, n_h, n_out):
+    """BF16 inference in one kernel against the layer kernels, which rows of X at an odd address and an
+    output over its own input take: the same K steps, bias, rounding, so the same bits, also with
+    infinities and NaN, for row counts around the 128-row tile and the number of SMs."""
+    import torch
+    rng = np.random.default_rng(n_in)
+    most = 128 * 310 + 5
+    net = fr.MLP(n_in, n_h, n_out, most)
+    net.set_params(rng.standard_normal(net.nparam).astype(np.float32) * 0.1)
+    X = rng.standard_normal((most, n_in)).astype(np.float32)
+    X[3, 1], X[200, 0], X[201, 2] = np.inf, np.nan, -np.inf
+    base = _t(np.concatenate([np.zeros(1, np.float32), X.reshape(-1)]))
+    odd = base[1:].reshape(most, n_in)  # 4 bytes past a 16-byte boundary
+    even = odd.clone()
+    for M in (1, 127, 128, 129, 128 * 152, 128 * 153 + 1, most):
+        Y = torch.full((M + 1, n_out), 7.0, dtype=torch.float32, device="cuda")
+        want = torch.full((M + 1, n_out), 7.0, dtype=torch.float32, device="cuda")
+        net.forward(even[:M], Y[:M], bf16=True)
+        net.forward(odd[:M], want[:M], bf16=True)
+        assert torch.equal(Y.view(torch.int32), want.view(torch.int32)), M
+    if n_out <= n_in:  # in place: every row of X is read before Y is written
+        inplace = even.clone()
+        net.forward(inplace, inplace.view(-1)[:most * n_out].view(most, n_out), bf16=True)
+        assert torch.equal(inplace.view(-1)[:most * n_out].view(torch.int32), want[:most].view(-1).view(torch.int32))
