@@ -60,7 +60,7 @@ long long off_W(const fr_mlp* m, int l) {
 }
 long long off_b(const fr_mlp* m, int l) { return off_W(m, l) + (long long)m->n[l + 1] * m->n[l]; }
 
-// ---- FP32 tiled GEMM: C(i, j) = sum over k in [kbeg, kend) of A(i, k) B(k, j) ----
+// ---- FP32 tiled GEMM: C(i, j) = sum over k < K of A(i, k) B(k, j) ----
 // A is [i][lda] (AK: k runs along memory) or [k][lda]; B is [j][ldb] (BK) or
 // [k][ldb].  64 x 64 tile per CTA, 16-deep slices double-buffered in shared
 // memory with the next slice's global loads in flight during the FMAs; 128
@@ -69,14 +69,13 @@ long long off_b(const fr_mlp* m, int l) { return off_W(m, l) + (long long)m->n[l
 // to 300 columns: 8192 rows x 256 columns give 512 CTAs, 3.4 per SM.
 // Loads are 16 bytes wide where base, leading dimension and the k range allow
 // it (vec), else one value at a time.  One training step of 8192 samples (300-
-// 256-256-100), GEMMs and the rest: 5674 -> 366 us; the first version read
+// 256-256-100), GEMMs and the rest: 5614 -> 412 us; the first version read
 // both operands with a stride of one row per lane, summed the bias gradients in
 // one thread per column and launched the row splits one after another.
 enum SgemmEpilogue {
   EPI_RELU = 0,     // C = max(acc + bias, 0)
   EPI_BIAS2 = 1,    // C = C2 = acc + bias
-  EPI_MASK = 2,     // C = acc where mask > 0, else 0 (mask laid out as C)
-  EPI_PARTIAL = 3   // C[split] = acc, then the sums of A over k behind it
+  EPI_MASK = 2      // C = acc where mask > 0, else 0 (mask laid out as C)
 };
 struct SgemmArgs {
   int M, N, K;
@@ -89,7 +88,6 @@ struct SgemmArgs {
   const float* bias;   // EPI_RELU, EPI_BIAS2
   float* C2;           // EPI_BIAS2
   const float* mask;   // EPI_MASK
-  int ksplit;          // k range of each blockIdx.z (K: one split)
   int veca, vecb;      // 16-byte loads allowed
 };
 
@@ -146,17 +144,16 @@ __global__ void __launch_bounds__(128) k_sgemm(const SgemmArgs a) {
   __shared__ __align__(16) float As[2][kGK][kGP], Bs[2][kGK][kGP];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int i0 = blockIdx.y * kGT, j0 = blockIdx.x * kGT;
-  const int kbeg = blockIdx.z * a.ksplit, kend = min(a.K, kbeg + a.ksplit);
+  const int kend = a.K;
   float acc[8][4] = {};
-  float asum = 0.f;  // EPI_PARTIAL: sum over k of A(i0 + tid, k), by the first tile of a row of tiles
   float4 va[2], vb[2];
-  slice_load<AK>(va, a.A, a.lda, i0, a.M, kbeg, kend, a.veca);
-  slice_load<BK>(vb, a.B, a.ldb, j0, a.N, kbeg, kend, a.vecb);
+  slice_load<AK>(va, a.A, a.lda, i0, a.M, 0, kend, a.veca);
+  slice_load<BK>(vb, a.B, a.ldb, j0, a.N, 0, kend, a.vecb);
   slice_store<AK>(As[0], va);
   slice_store<BK>(Bs[0], vb);
   __syncthreads();
   int buf = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += kGK) {
+  for (int k0 = 0; k0 < kend; k0 += kGK) {
     const bool more = k0 + kGK < kend;
     if (more) {
       slice_load<AK>(va, a.A, a.lda, i0, a.M, k0 + kGK, kend, a.veca);
@@ -173,10 +170,6 @@ __global__ void __launch_bounds__(128) k_sgemm(const SgemmArgs a) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
     }
-    if (EPI == EPI_PARTIAL && blockIdx.x == 0 && tid < kGT) {
-#pragma unroll
-      for (int kk = 0; kk < kGK; ++kk) asum += As[buf][kk][tid];
-    }
     if (more) {  // the other buffer was last read before the previous barrier
       slice_store<AK>(As[buf ^ 1], va);
       slice_store<BK>(Bs[buf ^ 1], vb);
@@ -184,7 +177,6 @@ __global__ void __launch_bounds__(128) k_sgemm(const SgemmArgs a) {
       buf ^= 1;
     }
   }
-  const long long slot = (long long)blockIdx.z * ((long long)a.M * a.N + a.M);
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int i = i0 + 8 * ty + u;
@@ -202,38 +194,117 @@ __global__ void __launch_bounds__(128) k_sgemm(const SgemmArgs a) {
         a.C2[o] = c;
       }
       if (EPI == EPI_MASK) a.C[o] = a.mask[o] > 0.f ? c : 0.f;
-      if (EPI == EPI_PARTIAL) a.C[slot + o] = c;
     }
   }
-  if (EPI == EPI_PARTIAL && blockIdx.x == 0 && tid < kGT && i0 + tid < a.M)
-    a.C[slot + (long long)a.M * a.N + i0 + tid] = asum;
 }
 
 int vec_ok(const float* p, int ld) { return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld % 4 == 0; }
 
 template <bool AK, bool BK, int EPI>
-void sgemm(SgemmArgs a, int splits, cudaStream_t s) {
+void sgemm(SgemmArgs a, cudaStream_t s) {
   a.veca = vec_ok(a.A, a.lda);
   a.vecb = vec_ok(a.B, a.ldb);
-  const dim3 grid((a.N + kGT - 1) / kGT, (a.M + kGT - 1) / kGT, splits);
+  const dim3 grid((a.N + kGT - 1) / kGT, (a.M + kGT - 1) / kGT);
   count_launch();
   k_sgemm<AK, BK, EPI><<<grid, 128, 0, s>>>(a);
 }
 
-// Row splits of a weight gradient (n x k outputs summed over M rows): enough that
-// its 64 x 64 tiles give each SM about three CTAs, at least 64 rows each; grows
-// with M.
-int max_splits(int n, int k, int M) {
-  const int tiles = ((n + kGT - 1) / kGT) * ((k + kGT - 1) / kGT);
-  return std::max(1, std::min((3 * 152 + tiles - 1) / tiles, (M + 63) / 64));
+// ---- weight and bias gradients of all layers in one launch ----
+// dW(i, j) = sum over rows r of D(r, i) in(r, j), db(i) = sum of D(r, i), one
+// CTA for 32 x 32 outputs of one layer and one part of kPartRows rows: every
+// output is one chain of FMAs over its rows in order, because an Adam step
+// divides a gradient by its own magnitude and so shows the order of the sums
+// wherever a gradient nearly cancels.  The chains leave the outputs as the only
+// parallelism, hence the small tile, 2 x 4 outputs a thread (300-256-256-100:
+// 176 CTAs a part) and the three layers side by side; D and the layer inputs of
+// every layer are kept, so nothing is waited for.  32 rows a stage by cp.async,
+// four stages.  A training step of 8192 rows takes 412 us so (5614 with one launch
+// per layer and part and strided reads); with 23 shorter chains per output and 64 x
+// 64 tiles it took 363, but an element whose gradient nearly cancelled could move
+// by 1e-3 of the parameters' size.
+constexpr int kPartRows = 4096, kWT = 32, kWStages = 4;
+struct WgradArgs {
+  int M, first[4];          // rows; first tile of each layer, and their number
+  float* out;               // [part][parameters]
+  long long stride;
+  struct {
+    const float *D, *in;    // [M][n], [M][k]
+    int n, k, vd, vin;      // widths, 16-byte copies allowed
+    long long off;          // weights, biases behind them
+  } l[3];
+};
+// four consecutive floats at x of a row, `ok` of them in range, the rest zero
+__device__ __forceinline__ void wgrad_copy4(float* dst, const float* base, long long at, int ok, int vec) {
+  const unsigned d = smem_u32(dst);
+  if (vec) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(ok >= 4 ? base + at : base),
+                 "r"(ok >= 4 ? 16 : 0)
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4 * c), "l"(c < ok ? base + at + c : base),
+                   "r"(c < ok ? 4 : 0)
+                   : "memory");
+  }
 }
-// rows per split, a multiple of the slice depth, and the splits that makes (at
-// most max_splits)
-int split_rows(int n, int k, int M, int* splits) {
-  const int want = max_splits(n, k, M);
-  const int rows = ((M + want - 1) / want + kGK - 1) / kGK * kGK;
-  *splits = (M + rows - 1) / rows;
-  return rows;
+__global__ void __launch_bounds__(128) k_wgrad(const __grid_constant__ WgradArgs a) {
+  __shared__ __align__(16) float As[kWStages][kWT][kWT], Bs[kWStages][kWT][kWT];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int tile = blockIdx.x, l = tile >= a.first[2] ? 2 : (tile >= a.first[1] ? 1 : 0);
+  const int n = a.l[l].n, k = a.l[l].k, tk = (k + kWT - 1) / kWT;
+  const int i0 = (tile - a.first[l]) / tk * kWT, j0 = (tile - a.first[l]) % tk * kWT;
+  const int rbeg = blockIdx.y * kPartRows, rend = min(a.M, rbeg + kPartRows), steps = (rend - rbeg + kWT - 1) / kWT;
+  const float *D = a.l[l].D, *in = a.l[l].in;
+  const int vd = a.l[l].vd, vin = a.l[l].vin;
+  const auto load = [&](int step) {
+    if (step < steps) {
+      const int r0 = rbeg + step * kWT, st = step % kWStages;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int row = (tid >> 3) + 16 * u, c = 4 * (tid & 7), r = r0 + row;
+        wgrad_copy4(&As[st][row][c], D, (long long)r * n + i0 + c, r < rend ? n - i0 - c : 0, vd);
+        wgrad_copy4(&Bs[st][row][c], in, (long long)r * k + j0 + c, r < rend ? k - j0 - c : 0, vin);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[2][4] = {};
+  float asum = 0.f;  // column sum of D, by the first warp of a layer's first column of tiles
+#pragma unroll
+  for (int st = 0; st < kWStages - 1; ++st) load(st);
+  for (int step = 0; step < steps; ++step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kWStages - 2) : "memory");
+    __syncthreads();  // this stage is filled, and the one before it has been read
+    load(step + kWStages - 1);
+    const int st = step % kWStages;
+#pragma unroll
+    for (int kk = 0; kk < kWT; ++kk) {
+      const float2 av = *reinterpret_cast<const float2*>(&As[st][kk][2 * ty]);
+      const float4 bv = *reinterpret_cast<const float4*>(&Bs[st][kk][4 * tx]);
+      acc[0][0] = fmaf(av.x, bv.x, acc[0][0]);
+      acc[0][1] = fmaf(av.x, bv.y, acc[0][1]);
+      acc[0][2] = fmaf(av.x, bv.z, acc[0][2]);
+      acc[0][3] = fmaf(av.x, bv.w, acc[0][3]);
+      acc[1][0] = fmaf(av.y, bv.x, acc[1][0]);
+      acc[1][1] = fmaf(av.y, bv.y, acc[1][1]);
+      acc[1][2] = fmaf(av.y, bv.z, acc[1][2]);
+      acc[1][3] = fmaf(av.y, bv.w, acc[1][3]);
+    }
+    if (j0 == 0 && tid < kWT) {
+#pragma unroll
+      for (int kk = 0; kk < kWT; ++kk) asum += As[st][kk][tid];
+    }
+  }
+  float* out = a.out + blockIdx.y * a.stride + a.l[l].off;
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int i = i0 + 2 * ty + u, j = j0 + 4 * tx + v;
+      if (i < n && j < k) out[(long long)i * k + j] = acc[u][v];
+    }
+  if (j0 == 0 && tid < kWT && i0 + tid < n) out[(long long)n * k + i0 + tid] = asum;
 }
 
 // ---- BF16 tensor-core GEMM for inference: Y = act(X W^T + b) ----
@@ -482,8 +553,7 @@ __global__ void k_loss_grad(const float* __restrict__ y, const float* __restrict
   }
 }
 
-// sum of the row splits' partials (fixed order) into a layer's weight and bias
-// gradients, which lie side by side as in the partials
+// sum of the parts' gradients, in order
 __global__ void k_sum_parts(const float* __restrict__ part, int nparts, long long n, float* __restrict__ out) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     float s = 0.f;
@@ -657,11 +727,8 @@ extern "C" int fr_mlp_create(int n_in, int n_hidden, int n_out, int max_batch, f
     e = cudaMalloc(&m->A[l], (size_t)max_batch * m->n[l + 1] * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&m->H16[l], (size_t)max_batch * m->kp[l + 1] * sizeof(__nv_bfloat16));
   }
-  long long np_max = 0;
-  for (int l = 0; l < 3; ++l)
-    np_max = std::max(np_max, max_splits(m->n[l + 1], m->n[l], max_batch) *
-                                  ((long long)m->n[l + 1] * m->n[l] + m->n[l + 1]));
-  if (e == cudaSuccess) e = cudaMalloc(&m->part, (size_t)np_max * sizeof(float));
+  const int parts = (max_batch + kPartRows - 1) / kPartRows;
+  if (e == cudaSuccess && parts > 1) e = cudaMalloc(&m->part, (size_t)parts * np * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&m->X16, (size_t)max_batch * m->kp[0] * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = cudaMalloc(&m->loss, sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(m->Mo, 0, np * sizeof(float));
@@ -725,14 +792,14 @@ extern "C" int fr_mlp_forward(fr_mlp* m, const float* X, int M, float* Y, int bf
     const float* in = X;
     for (int l = 0; l < 3; ++l) {
       SgemmArgs g{};
-      g.M = M; g.N = m->n[l + 1]; g.K = g.ksplit = m->n[l];
+      g.M = M; g.N = m->n[l + 1]; g.K = m->n[l];
       g.A = in; g.lda = m->n[l];
       g.B = m->P + off_W(m, l); g.ldb = m->n[l];
       g.bias = m->P + off_b(m, l);
       g.C = l < 2 ? m->A[l] : Y; g.ldc = g.N;
       g.C2 = m->Z;
-      if (l < 2) sgemm<true, true, EPI_RELU>(g, 1, s);
-      else sgemm<true, true, EPI_BIAS2>(g, 1, s);
+      if (l < 2) sgemm<true, true, EPI_RELU>(g, s);
+      else sgemm<true, true, EPI_BIAS2>(g, s);
       in = g.C;
     }
   } else {
@@ -827,29 +894,36 @@ extern "C" int fr_mlp_backward(fr_mlp* m, const float* X, const float* T, int M,
   // Z holds the forward pass's output
   count_launch();
   k_loss_grad<<<grid_for(nout) > 1024 ? 1024 : grid_for(nout), 256, 0, s>>>(m->Z, T, m->D[2], nout, m->loss, red);
-  for (int l = 2; l >= 0; --l) {
-    const int K = m->n[l], N = m->n[l + 1];
-    // dW[N x K] = D[l]^T in and db[N] = column sums of D[l], over row splits
-    int splits = 0;
-    SgemmArgs g{};
-    g.M = N; g.N = K; g.K = M;
-    g.ksplit = split_rows(N, K, M, &splits);
-    g.A = m->D[l]; g.lda = N;
-    g.B = l == 0 ? X : m->A[l - 1]; g.ldb = K;
-    g.C = m->part; g.ldc = K;
-    sgemm<false, false, EPI_PARTIAL>(g, splits, s);
-    const long long np = (long long)N * K + N;
+  for (int l = 2; l > 0; --l) {  // D[l-1] = D[l] W_l where the activation is positive
+    SgemmArgs d{};
+    d.M = M; d.N = m->n[l]; d.K = m->n[l + 1];
+    d.A = m->D[l]; d.lda = d.K;
+    d.B = m->P + off_W(m, l); d.ldb = d.N;
+    d.C = m->D[l - 1]; d.ldc = d.N;
+    d.mask = m->A[l - 1];
+    sgemm<true, false, EPI_MASK>(d, s);
+  }
+  const int parts = (M + kPartRows - 1) / kPartRows;
+  WgradArgs g{};
+  g.M = M;
+  g.out = parts > 1 ? m->part : m->G;
+  g.stride = m->nparam;
+  for (int l = 0; l < 3; ++l) {
+    const int n = m->n[l + 1], k = m->n[l];
+    g.l[l].D = m->D[l];
+    g.l[l].in = l == 0 ? X : m->A[l - 1];
+    g.l[l].n = n;
+    g.l[l].k = k;
+    g.l[l].vd = vec_ok(g.l[l].D, n);
+    g.l[l].vin = vec_ok(g.l[l].in, k);
+    g.l[l].off = off_W(m, l);
+    g.first[l + 1] = g.first[l] + ((n + kWT - 1) / kWT) * ((k + kWT - 1) / kWT);
+  }
+  count_launch();
+  k_wgrad<<<dim3(g.first[3], parts), 128, 0, s>>>(g);
+  if (parts > 1) {
     count_launch();
-    k_sum_parts<<<grid_for(np), 256, 0, s>>>(m->part, splits, np, m->G + off_W(m, l));
-    if (l > 0) {  // D[l-1] = D[l] W_l where the activation is positive
-      SgemmArgs d{};
-      d.M = M; d.N = K; d.K = d.ksplit = N;
-      d.A = m->D[l]; d.lda = N;
-      d.B = m->P + off_W(m, l); d.ldb = K;
-      d.C = m->D[l - 1]; d.ldc = K;
-      d.mask = m->A[l - 1];
-      sgemm<true, false, EPI_MASK>(d, 1, s);
-    }
+    k_sum_parts<<<grid_for(m->nparam), 256, 0, s>>>(m->part, parts, m->nparam, m->G);
   }
   MLP_CUDA(m, cudaGetLastError());
   if (loss_host) {
