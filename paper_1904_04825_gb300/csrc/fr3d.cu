@@ -58,7 +58,6 @@ struct F3Args {
   long long ne;
   long long e0, nchunk;  // mode 3: the elements e0 .. e0 + nchunk - 1, columns staged from out[0]
   float* r0f;            // mode 3 in FP32: element-local R(U) of the chunk, [nchunk][NB]
-  double* r0d;           // mode 3 in FP64: the same
   const float* tbf;      // mode 3 in FP32: the trace buffer in FP32
   // A z with FP32 linear parts (jv_precision 1): caches at the linearisation
   // point U and the FP32 buffers of the product
@@ -69,7 +68,7 @@ struct F3Args {
   float* tbz;            // traces of z and of its gradient [ne][6][N^2][20]
   float* fbz;            // per unit eps: q_com differences and f_n differences [ne][3][N^2][10]
   double* lgc;           // BR2 common gradient of U at the low-face points [ne][3][N^2][15]
-  int r0_pass;           // mode 3: 1 = write the element-local R(U) (one unperturbed slot per element)
+  int r0_pass;           // mode 3 in FP32: 1 = write r0f (one unperturbed slot per element)
   int nx, ny, nz;
   double gam, mu, kappa, shift, beps;
   Tables tab;
@@ -297,8 +296,8 @@ __global__ void __launch_bounds__(256) k3_fulltrace(const F3Args a) {
   }
 }
 
-// Caches of the A z with FP32 linear parts: q_com, f_n and the BR2 common gradient
-// at U, one thread per (element, direction d, point of its low face d)
+// q_com, f_n and (lgc: for the caches of the A z with FP32 linear parts) the BR2
+// common gradient at U, one thread per (element, direction d, point of its low face d)
 template <int P>
 __global__ void __launch_bounds__(256) k3_face_cache(const F3Args a) {
   constexpr int N = P + 1, N2 = N * N;
@@ -331,6 +330,7 @@ __global__ void __launch_bounds__(256) k3_face_cache(const F3Args a) {
     dst[v] = qc[v];
     dst[5 + v] = fn[v];
   }
+  if (!a.lgc) return;
   double* g = a.lgc + ((e * 3 + d) * N2 + f) * 15;
 #pragma unroll
   for (int c = 0; c < 3; ++c)
@@ -340,19 +340,22 @@ __global__ void __launch_bounds__(256) k3_face_cache(const F3Args a) {
 
 // MODE 3: element-Jacobi column (see the file header); 4: the caches of the
 // FP32-linear-parts A z at U (corrected gradient and total fluxes at the
-// points to a.lg, a.lf; face data from the face buffer).
+// points to a.lg, a.lf; face data from the face buffer); 0: the R(U) that FP64
+// columns subtract, from the face buffer.
 // T: arithmetic type, double except for FP32 element-Jacobi columns (MODE 3,
-// T = float).  A first pass of MODE 3 (a.r0_pass) writes the element-local
-// R(U) of each element of the chunk by the same operations to a.r0d (FP32:
-// a.r0f); the columns pass divides R(U + eps_c e_c) minus that by eps_c (FP32:
-// by the step actually taken).
+// T = float): then a first pass (a.r0_pass) writes the element-local R(U) of
+// each element of the chunk in FP32 to a.r0f, and the columns pass divides
+// R(U + eps_c e_c) - r0f by the step actually taken in FP32.  FP64 columns
+// divide by eps_c ~ 1e-8, which makes the last bits of the R(U) they subtract
+// 1e-8 of a column: that R(U) keeps its order of operations (three kernels,
+// 1/NB of the columns' work) rather than the faster operator's.
 template <int P, int MODE, typename T = double>
 __global__ void __launch_bounds__(256) k3_cols(const F3Args a) {
   using L = CellLayout<P, T>;
   constexpr int N = P + 1, N2 = N * N, NP = N2 * N, E = F3Slots<P>::E, NB = 5 * NP;
   constexpr bool JAC = MODE == 3;
   constexpr bool J32 = JAC && sizeof(T) == 4;
-  static_assert(JAC || (MODE == 4 && sizeof(T) == 8), "columns, or the FP64 caches");
+  static_assert(JAC || ((MODE == 4 || MODE == 0) && sizeof(T) == 8), "columns, or R(U) and the caches in FP64");
   constexpr T cbr2 = T((P + 1) * (P + 2) / 2.0);
   extern __shared__ __align__(16) unsigned char smem3_raw[];
   T* smem3 = reinterpret_cast<T*>(smem3_raw);
@@ -376,7 +379,7 @@ __global__ void __launch_bounds__(256) k3_cols(const F3Args a) {
   T* d2 = d1 + 5 * NP;
   T* dq = d2 + 5 * NP;          // [6][N2][5] q_com - q_face
   T* fn = dq + 30 * N2;         // [6][N2][5] common total normal flux
-  const bool r0_pass = JAC && a.r0_pass;
+  const bool r0_pass = J32 && a.r0_pass;
   const long long slot = (long long)blockIdx.x * E + el;
   const long long nslots = JAC ? (r0_pass ? a.nchunk : a.nchunk * NB) : a.ne;
   const bool active = el < E && slot < nslots;
@@ -526,19 +529,20 @@ __global__ void __launch_bounds__(256) k3_cols(const F3Args a) {
       dH = fma(sDt[k][l], H[i + N * j + N2 * l], dH);
     }
     const T R = -fma(s[0], dF, fma(s[1], dG, s[2] * dH));
-    // column col of M = shift I - J_ee, staged column-major [col][row]
-    const int row = v * NP + t;
-    const long long ro = (e - a.e0) * NB + row;
-    if (r0_pass) {
-      if (J32) a.r0f[ro] = (float)R;
-      else a.r0d[ro] = (double)R;
+    const long long o = e * NB + v * NP + t;
+    if (MODE == 0) {
+      a.out[o] = (double)R;
     } else {
+      // column col of M = shift I - J_ee, staged column-major [col][row]
+      const int row = v * NP + t;
       double* dst = a.out + ((e - a.e0) * NB + col) * NB + row;
-      if (J32) {  // the difference quotient and the column in FP32
-        const float dq32 = ((float)R - a.r0f[ro]) / ceps32;
+      if (r0_pass) {
+        a.r0f[(e - a.e0) * NB + row] = (float)R;
+      } else if (J32) {  // the difference quotient and the column in FP32
+        const float dq32 = ((float)R - a.r0f[(e - a.e0) * NB + row]) / ceps32;
         *dst = (double)((row == col ? (float)a.shift : 0.f) - dq32);
       } else {
-        *dst = (row == col ? a.shift : 0.0) - ((double)R - a.r0d[ro]) / ceps;
+        *dst = (row == col ? a.shift : 0.0) - ((double)R - a.R0[o]) / ceps;
       }
     }
   }
@@ -1196,7 +1200,6 @@ F3Args make_args3(fr_ctx* ctx) {
   a.e0 = 0;
   a.nchunk = ctx->ne;
   a.r0f = nullptr;
-  a.r0d = nullptr;
   a.tbf = nullptr;
   a.r0_pass = 0;
   a.ltb = ctx->lin3_tb;
@@ -1346,25 +1349,39 @@ int f3_columns(fr_ctx* ctx, F3Args a, cudaStream_t s) {
   // one element residual per column: the own six faces' common data, counted
   // like the residual with every face of the element
   const double per = ns3d_residual_flops_per_element(P) + 3.0 * L::N2 * 245.0;
-  // the element-local R(U) of each element by the same arithmetic first
-  a.r0f = ctx->r0f;
-  a.r0d = ctx->rloc;
-  a.r0_pass = 1;
-  { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * (double)a.nchunk);
-    k3_cols<P, 3, T><<<(unsigned)((a.nchunk + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
-  FRK_LAUNCHED(ctx);
-  a.r0_pass = 0;
+  if constexpr (sizeof(T) == 4) {  // the element-local R(U) of each element by the same arithmetic first
+    a.r0f = ctx->r0f;
+    a.r0_pass = 1;
+    { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * (double)a.nchunk);
+      k3_cols<P, 3, T><<<(unsigned)((a.nchunk + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
+    FRK_LAUNCHED(ctx);
+    a.r0_pass = 0;
+  }
   { ProfScope ps_(ctx, FR_KF_FACTOR, s, 0.0, per * NB * (double)a.nchunk);
     k3_cols<P, 3, T><<<(unsigned)((a.nchunk * NB + E - 1) / E), E * NP, L::BYTES, s>>>(a); }
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }
 
+// the unperturbed traces, which the columns read as the frozen neighbour traces, and for
+// FP64 columns R(U) into ctx->rloc
 template <int P>
-int f3_fulltrace(fr_ctx* ctx, const F3Args& a, cudaStream_t s) {
-  constexpr int NP = CellLayout<P>::NP, E = F3Slots<P>::E;
-  { ProfScope ps_(ctx, FR_KF_FACTOR, s);
-    k3_fulltrace<P><<<(unsigned)((ctx->ne + E - 1) / E), E * NP, 0, s>>>(a); }
+int f3_base(fr_ctx* ctx, F3Args a, cudaStream_t s) {
+  using L = CellLayout<P>;
+  constexpr int NP = L::NP, E = F3Slots<P>::E;
+  const unsigned gt = (unsigned)((ctx->ne + E - 1) / E);
+  ProfScope ps_(ctx, FR_KF_FACTOR, s);
+  k3_fulltrace<P><<<gt, E * NP, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  if (ctx->opts.block_columns == 1) return FR_OK;
+  a.lgc = nullptr;
+  a.out = ctx->rloc;
+  FRK_CUDA(ctx, cudaFuncSetAttribute(k3_cols<P, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES));
+  count_launch();
+  k3_face_cache<P><<<(unsigned)((ctx->ne * 3 * L::N2 + 255) / 256), 256, 0, s>>>(a);
+  FRK_LAUNCHED(ctx);
+  count_launch();
+  k3_cols<P, 0><<<gt, E * NP, L::BYTES, s>>>(a);
   FRK_LAUNCHED(ctx);
   return FR_OK;
 }
@@ -1422,12 +1439,12 @@ int launch_f3_factor(fr_ctx* ctx, const double* U, double shift, cudaStream_t s)
   a.U = U;
   a.out = ctx->mst;
   a.shift = shift;
-  // the unperturbed traces, which the columns read as the frozen neighbour traces
   switch (ctx->p) {
-    case 1: FRK_TRY(f3_fulltrace<1>(ctx, a, s)); break;
-    case 2: FRK_TRY(f3_fulltrace<2>(ctx, a, s)); break;
-    default: FRK_TRY(f3_fulltrace<3>(ctx, a, s)); break;
+    case 1: FRK_TRY(f3_base<1>(ctx, a, s)); break;
+    case 2: FRK_TRY(f3_base<2>(ctx, a, s)); break;
+    default: FRK_TRY(f3_base<3>(ctx, a, s)); break;
   }
+  a.R0 = ctx->rloc;
   if (ctx->opts.block_columns == 1) {
     if (!ctx->r0f || !ctx->tbf)
       return set_error(ctx, FR_ERR_UNSUPPORTED, "FP32 block columns need block_columns = 1 at creation");
