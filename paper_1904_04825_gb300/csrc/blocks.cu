@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(FactorLayout<P, T>::THREADS) k_factor(const Fa
   S* out = reinterpret_cast<S*>(a.blocks) + e * (long long)NB * NB;
   if constexpr (L::TC) {
     unsigned char* tcs = smem_f + L::OFF_SCRATCH;
-    const bool ok = gjtc::invert<NB, LD>(M, col, piv, tcs);
+    const bool ok = gjtc::invert<NB, LD>(M, piv, tcs);
     if (!ok && threadIdx.x == 0) atomicExch(a.err, 1);
     // ---- store column-major: inverse(i, k) = M[pr[i]][ipr[k]] ----
     const int* ipr = reinterpret_cast<const int*>(tcs + gjtc::Shape<NB>::OFF_IPR);
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(InvertLayout<NB, T>::THREADS) k_invert(const d
   S* out = reinterpret_cast<S*>(blocks) + e * (long long)NB * NB;
   if constexpr (L::TC) {
     unsigned char* tcs = reinterpret_cast<unsigned char*>(smem_inv) + L::OFF_TC;
-    const bool ok = gjtc::invert<NB, LD>(M, col, piv, tcs);
+    const bool ok = gjtc::invert<NB, LD>(M, piv, tcs);
     if (!ok && threadIdx.x == 0) atomicExch(err, 1);
     const int* ipr = reinterpret_cast<const int*>(tcs + gjtc::Shape<NB>::OFF_IPR);
     for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {

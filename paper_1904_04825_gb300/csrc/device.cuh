@@ -311,6 +311,13 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+// one lane of a converged warp, always the same one; what it issues under a warp-uniform
+// branch keeps its operands in uniform registers
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
 constexpr unsigned kWaitPolls = 1u << 22;  // bounded waits: far above any copy's latency
 
 }  // namespace frk

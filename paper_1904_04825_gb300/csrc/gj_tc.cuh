@@ -6,7 +6,14 @@
 //  * panel factorisation: for each column c of the panel, the pivot row r is
 //    the unused row of largest |M[r][c]| (rows are not swapped: pr[c] = r is
 //    recorded instead), and the elimination is applied to the panel's
-//    columns only (all rows);
+//    columns only (all rows).
+//    One warp does it with the panel in registers (lane l holds rows l + 32 q):
+//    the largest of the column by redux.sync, the pivot row passed on through
+//    shared memory, no CTA barrier.  The chain of NB pivots bounds the
+//    inversion, and other CTAs of the SM fill the gaps; with the panel in
+//    shared memory and three CTA barriers a pivot, 4096 blocks of 64 rows took
+//    592 us, now 239, and columns, inversion and one apply of 2350 blocks of
+//    100 rows 1.93 ms, now 1.06;
 //  * the b pivots of a panel act on every other column x as x <- x + U x_P,
 //    with x_P the pivot rows' entries of x before the panel and
 //    U = (panel columns after the panel) - (unit vectors of the pivot rows):
@@ -45,17 +52,14 @@ struct Shape {
   static constexpr unsigned B_BYTES = N * BW * 4;
   static constexpr unsigned OPS = 2 * A_BYTES + 2 * B_BYTES;
   static constexpr unsigned TMEM_COLS = N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
-  // scratch after the operands: barrier (8), tensor-memory slot (4), pivot
-  // row (4), inverse permutation (4 NB), panel pivot rows (4 BW), scaled
-  // pivot row (4 BW), used-row flags (NB)
-  static constexpr unsigned OFF_BAR = OPS;
+  // scratch after the operands: pivot row (4 BW), barrier (8), tensor-memory
+  // slot (4), panel pivot rows (4 BW), inverse permutation (4 NB)
+  static constexpr unsigned OFF_SROW = OPS;
+  static constexpr unsigned OFF_BAR = OFF_SROW + 4 * BW;
   static constexpr unsigned OFF_SLOT = OFF_BAR + 8;
-  static constexpr unsigned OFF_PROW = OFF_SLOT + 4;
-  static constexpr unsigned OFF_IPR = OFF_PROW + 4;
-  static constexpr unsigned OFF_ROWS = OFF_IPR + 4 * NB;
-  static constexpr unsigned OFF_SROW = OFF_ROWS + 4 * BW;
-  static constexpr unsigned OFF_USED = OFF_SROW + 4 * BW;
-  static constexpr unsigned BYTES = (OFF_USED + NB + 127) / 128 * 128;
+  static constexpr unsigned OFF_ROWS = OFF_SLOT + 8;
+  static constexpr unsigned OFF_IPR = OFF_ROWS + 4 * BW;
+  static constexpr unsigned BYTES = (OFF_IPR + 4 * NB + 127) / 128 * 128;
 };
 
 // blocks whose inversion runs on the tensor cores (one MMA covers <= 128 rows)
@@ -106,11 +110,11 @@ __device__ __forceinline__ void mma_tf32(unsigned tmem, unsigned long long ad, u
 // Invert the NB x NB FP32 matrix M (row stride LD, shared memory) in place
 // into the permuted form described above; pr receives the pivot rows and
 // scratch (Shape<NB>::BYTES, 128-byte aligned) holds the operands and
-// bookkeeping, with ipr at scratch + OFF_IPR.  col: NB floats.  Whole CTA,
+// bookkeeping, with ipr at scratch + OFF_IPR.  Whole CTA,
 // blockDim.x a multiple of 128.  Returns false (on every thread) if a
 // tensor-core wait gave up; the tensor memory is freed in every case.
 template <int NB, int LD>
-__device__ bool invert(float* M, float* col, int* pr, unsigned char* scratch) {
+__device__ bool invert(float* M, int* pr, unsigned char* scratch) {
   using Sh = Shape<NB>;
   static_assert(NB <= MROWS, "one MMA covers at most 128 rows");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x;
@@ -120,14 +124,12 @@ __device__ bool invert(float* M, float* col, int* pr, unsigned char* scratch) {
   unsigned char* Blo = Bhi + Sh::B_BYTES;
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(scratch + Sh::OFF_BAR);
   unsigned* tslot = reinterpret_cast<unsigned*>(scratch + Sh::OFF_SLOT);
-  int* s_prow = reinterpret_cast<int*>(scratch + Sh::OFF_PROW);
   int* ipr = reinterpret_cast<int*>(scratch + Sh::OFF_IPR);
   int* rows = reinterpret_cast<int*>(scratch + Sh::OFF_ROWS);
   float* srow = reinterpret_cast<float*>(scratch + Sh::OFF_SROW);
-  unsigned char* used = scratch + Sh::OFF_USED;
+  constexpr int R = (NB + 31) / 32;  // rows a lane
 
   for (int i = tid; i < (int)(Sh::OPS / 16); i += nthr) reinterpret_cast<uint4*>(scratch)[i] = make_uint4(0, 0, 0, 0);
-  for (int i = tid; i < NB; i += nthr) used[i] = 0;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(Sh::TMEM_COLS)
@@ -146,59 +148,96 @@ __device__ bool invert(float* M, float* col, int* pr, unsigned char* scratch) {
 
   bool ok = true;
   int step = 0;
+  unsigned used = 0;  // warp 0: this lane's rows that have been pivots
   for (int c0 = 0; c0 < NB; c0 += BW, ++step) {
     const int kb = min(BW, NB - c0);
-    // ---- panel factorisation: kb pivots on the panel's columns ----
-    for (int k = 0; k < kb; ++k) {
-      const int c = c0 + k;
-      for (int i = tid; i < NB; i += nthr) col[i] = M[i * LD + c];
-      __syncthreads();
-      if (warp == 0) {
-        float best = -1.f;  // |pivot| (NaN ranks above everything)
-        int bi = NB;
-        for (int r = lane; r < NB; r += 32) {
-          if (used[r]) continue;
-          float v = fabsf(col[r]);
-          if (v != v) v = __int_as_float(0x7f800000);
-          if (v > best) { best = v; bi = r; }
-        }
+    if (warp == 0) {
+      // ---- panel factorisation: kb pivots on the panel's columns, lane l holds rows l + 32 q ----
+      float p[R][BW];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float ob = __shfl_down_sync(0xffffffffu, best, o);
-          const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        bi = __shfl_sync(0xffffffffu, bi, 0);
-        const float ip = 1.f / col[bi];
-        if (lane < kb) srow[lane] = (lane == k ? 1.f : M[bi * LD + c0 + lane]) * ip;
-        if (lane == 0) {
-          *s_prow = bi;
-          used[bi] = 1;
-          pr[c] = bi;
-          ipr[bi] = c;
-          rows[k] = bi;
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int t = 0; t < BW; ++t) p[q][t] = lane + 32 * q < NB && t < kb ? M[(lane + 32 * q) * LD + c0 + t] : 0.f;
+      unsigned piv = 0;  // this lane's rows chosen in this panel: 5 bits a row, 1 + the pivot's number
+#pragma unroll
+      for (int k = 0; k < BW; ++k) {
+        if (k < kb) {
+          // largest |M[r][c]| of the unused rows, the first of equals; NaN ranks with the infinities
+          unsigned best = 0;  // 0: a used row or none
+          int bi = NB;
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            const float v = fabsf(p[q][k]);
+            const unsigned key = (v != v ? 0x7f800000u : __float_as_uint(v)) + 1u;
+            if (!(used >> q & 1u) && key > best) {
+              best = key;
+              bi = lane + 32 * q;
+            }
+          }
+          const unsigned most = __reduce_max_sync(0xffffffffu, best);
+          bi = (int)__reduce_min_sync(0xffffffffu, best == most ? (unsigned)bi : (unsigned)NB);
+          const int bq = bi >> 5;
+          if (lane == (bi & 31)) {
+            used |= 1u << bq;
+            piv |= (unsigned)(k + 1) << (5 * bq);
+            pr[c0 + k] = bi;
+            ipr[bi] = c0 + k;
+            rows[k] = bi;
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              if (q == bq) {
+#pragma unroll
+                for (int t = 0; t < BW; t += 4)
+                  *reinterpret_cast<float4*>(srow + t) = make_float4(p[q][t], p[q][t + 1], p[q][t + 2], p[q][t + 3]);
+              }
+          }
+          __syncwarp();
+          float sr[BW];
+#pragma unroll
+          for (int t = 0; t < BW; t += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(srow + t);
+            sr[t] = v.x; sr[t + 1] = v.y; sr[t + 2] = v.z; sr[t + 3] = v.w;
+          }
+          __syncwarp();  // before the next pivot's row is written
+          const float ip = 1.f / sr[k];
+#pragma unroll
+          for (int t = 0; t < BW; ++t) sr[t] = (t == k ? 1.f : sr[t]) * ip;
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            const bool own = lane + 32 * q == bi;
+            const float f = p[q][k];
+#pragma unroll
+            for (int t = 0; t < BW; ++t) {
+              const float u = (t == k ? 0.f : p[q][t]) - f * sr[t];
+              p[q][t] = own ? sr[t] : u;
+            }
+          }
         }
       }
-      __syncthreads();
-      const int r = *s_prow;
-      for (int idx = tid; idx < NB * kb; idx += nthr) {
-        const int i = idx / kb, t = idx - i * kb;
-        float* m = M + i * LD + c0 + t;
-        *m = i == r ? srow[t] : (t == k ? 0.f : *m) - col[i] * srow[t];
+      // the panel's columns, and A = U (rows i, K index k)
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const int i = lane + 32 * q;
+        if (i < NB) {
+          const int mine = (int)(piv >> (5 * q) & 31u) - 1;
+#pragma unroll
+          for (int t = 0; t < BW; t += 4) {
+            float4 hi, lo;
+            float *h = &hi.x, *l = &lo.x;
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+              if (t + d < kb) M[i * LD + c0 + t + d] = p[q][t + d];
+              const float u = t + d < kb ? p[q][t + d] - (t + d == mine ? 1.f : 0.f) : 0.f;
+              split_tf32(u, h + d, l + d);
+            }
+            *reinterpret_cast<float4*>(Ahi + op_off(i, t)) = hi;
+            *reinterpret_cast<float4*>(Alo + op_off(i, t)) = lo;
+          }
+        }
       }
-      __syncthreads();
     }
-    // ---- operands: A = U (rows i, K index k), B = X^T (rows j, K index k) ----
-    for (int idx = tid; idx < NB * BW; idx += nthr) {
-      const int i = idx / BW, k = idx - i * BW;
-      float u = 0.f;
-      if (k < kb) u = M[i * LD + c0 + k] - (i == rows[k] ? 1.f : 0.f);
-      float hi, lo;
-      split_tf32(u, &hi, &lo);
-      const unsigned o = op_off(i, k);
-      *reinterpret_cast<float*>(Ahi + o) = hi;
-      *reinterpret_cast<float*>(Alo + o) = lo;
-    }
+    __syncthreads();
+    // ---- B = X^T (rows j, K index k) ----
     for (int idx = tid; idx < BW * NB; idx += nthr) {
       const int k = idx / NB, j = idx - k * NB;
       float x = 0.f;
@@ -211,7 +250,7 @@ __device__ bool invert(float* M, float* col, int* pr, unsigned char* scratch) {
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned ah = smem_u32(Ahi), al = smem_u32(Alo), bh = smem_u32(Bhi), bl = smem_u32(Blo);
 #pragma unroll

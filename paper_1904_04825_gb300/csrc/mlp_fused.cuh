@@ -70,11 +70,6 @@ __device__ __forceinline__ void arrive(unsigned long long* bar) {
 __device__ __forceinline__ bool warp_wait(unsigned long long* bar, unsigned parity) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, kWaitPolls));
 }
-__device__ __forceinline__ bool elect_one() {
-  unsigned p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
 // 16 accumulator columns of this thread's row
 __device__ __forceinline__ void tmem_ld16(unsigned (&v)[16], unsigned addr) {
   asm volatile(

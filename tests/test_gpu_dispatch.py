@@ -258,3 +258,29 @@ def test_network_inference_in_one_kernel_equals_the_layer_kernels(fr, n_in, n_h,
         inplace = even.clone()
         net.forward(inplace, inplace.view(-1)[:most * n_out].view(most, n_out), bf16=True)
         assert torch.equal(inplace.view(-1)[:most * n_out].view(torch.int32), want[:most].view(-1).view(torch.int32))
+
+
+@pytest.mark.parametrize("p,nx,ny", [(2, 3, 2), (3, 2, 5), (4, 3, 3)])
+@pytest.mark.parametrize("prec", [1, 2])
+def test_reduced_precision_block_inverse_against_the_fp64_blocks(fr, p, nx, ny, prec):
+    """36, 64 and 100-row blocks inverted in FP32 (panels of 16 columns in one warp's registers, the last
+    panel of 4 included): M^-1 r against FP64 blocks.  FP32 elimination of n rows loses at most about
+    n cond 2^-24, with cond below 1e2 at this shift: 100 * 1e2 * 6e-8 = 6e-4 < 1e-3; BF16 storage adds
+    2^-9 of each entry, times cond in the worst direction of r, a few 2^-9 for a random one: 2e-2."""
+    xe, ye = S.stretched_mesh(nx, ny, seed=p)
+    X, Y = S.point_coords(xe, ye, p)
+    U = S.smooth_random_state(X, Y, seed=nx, amp=0.05, base=(1.0, 0.7, -0.4, 2.0))
+    r = S.random_vector(U.shape, 3)
+    z = []
+    for q in (0, prec):
+        ctx = fr.Context(xe, ye, p, fr.default_opts(block_precision=q))
+        fr.ejacobi_factor(ctx, _t(U), None, 30.0)
+        out = ctx.empty()
+        fr.ejacobi_apply(ctx, _t(r), out)
+        z.append(out.cpu().numpy())
+    assert np.linalg.norm(z[1] - z[0]) < (1e-3 if prec == 1 else 2e-2) * np.linalg.norm(z[0])
+    U[1, 2, 3] = np.nan  # a NaN stays in its element's block
+    fr.ejacobi_factor(ctx, _t(U), None, 30.0)
+    fr.ejacobi_apply(ctx, _t(r), out)
+    z = out.cpu().numpy()
+    assert not np.isfinite(z[1]).all() and np.isfinite(z[nx * (ny // 2)]).all()
