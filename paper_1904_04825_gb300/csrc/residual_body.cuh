@@ -241,8 +241,12 @@ __device__ __forceinline__ void residual_body(const ResArgs& a, const double* z,
       qm[v] = pm[v * N];
       qp[v] = pp[v * N];
     }
+    // the caches' flux is subtracted from one at U + eps z and the difference divided by
+    // eps, which shows its last bits: it keeps one expression per direction, as those
+    // bits depend on how the compiler contracts it
     if (FAST) riemann_flux2(RM, qm, qp, dir, a.gam, fc);
-    else riemann_flux(RM, qm, qp, dir, a.gam, fc);
+    else if (dir == 0) riemann_flux(RM, qm, qp, 0, a.gam, fc);
+    else riemann_flux(RM, qm, qp, 1, a.gam, fc);
 #pragma unroll
     for (int v = 0; v < 4; ++v) dst[v * N] = fc[v];
     if (MODE == 3 && cache) {
