@@ -82,8 +82,6 @@ void free_ctx(fr_ctx* c) {
   }
   cudaFreeHost(c->h_stat);
   cudaFreeHost(c->h_scal);
-  cudaFreeHost(c->h_cyc);
-  cudaFree(c->cyc_bar);
   delete c;
 }
 
@@ -154,8 +152,8 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
   FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
-  FRK_TRY(dalloc(c, &c->cyc_bar, 32));
-  FRK_TRY(dalloc(c, &c->red.counter, 1));
+  FRK_TRY(dalloc(c, &c->red.counter, 64));
+  c->cyc_bar = c->red.counter + 32;  // a line of its own
   c->gd.ldh = m + 1;
   FRK_TRY(dalloc(c, &c->gd.H, (size_t)(m + 1) * m));
   FRK_TRY(dalloc(c, &c->gd.cs, m));
@@ -173,8 +171,8 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->kerr, 1));
   FRK_CUDA(c, cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_stat), (4 + kMaxVec) * sizeof(int)));
-  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double)));
-  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_cyc), sizeof(CycleStatus)));
+  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double) + sizeof(CycleStatus)));
+  c->h_cyc = reinterpret_cast<CycleStatus*>(c->h_scal + 8);
   for (cudaEvent_t& e : c->chunk_ev) FRK_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   FRK_CUDA(c, cudaDeviceSynchronize());
   return FR_OK;
@@ -242,8 +240,8 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
   FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
-  FRK_TRY(dalloc(c, &c->cyc_bar, 32));
-  FRK_TRY(dalloc(c, &c->red.counter, 1));
+  FRK_TRY(dalloc(c, &c->red.counter, 64));
+  c->cyc_bar = c->red.counter + 32;  // a line of its own
   c->gd.ldh = m + 1;
   FRK_TRY(dalloc(c, &c->gd.H, (size_t)(m + 1) * m));
   FRK_TRY(dalloc(c, &c->gd.cs, m));
@@ -261,8 +259,8 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->kerr, 1));
   FRK_CUDA(c, cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_stat), (4 + kMaxVec) * sizeof(int)));
-  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double)));
-  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_cyc), sizeof(CycleStatus)));
+  FRK_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_scal), 8 * sizeof(double) + sizeof(CycleStatus)));
+  c->h_cyc = reinterpret_cast<CycleStatus*>(c->h_scal + 8);
   for (cudaEvent_t& e : c->chunk_ev) FRK_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   FRK_CUDA(c, cudaDeviceSynchronize());
   return FR_OK;

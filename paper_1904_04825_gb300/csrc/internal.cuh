@@ -179,8 +179,8 @@ struct fr_ctx {
   int tile_variant = 0;      // element-tile shape of the Euler residual kernel (autotuned)
   frk::Reduce red{};
   frk::GmresDev gd{};
-  unsigned* cyc_bar = nullptr;             // one-launch solves: barrier counter
-  frk::CycleStatus* h_cyc = nullptr;       // pinned: how the last one ended
+  unsigned* cyc_bar = nullptr;             // one-launch solves: barrier counter (behind red.counter)
+  frk::CycleStatus* h_cyc = nullptr;       // pinned: how the last one ended (behind h_scal)
   int* h_stat = nullptr;     // pinned host mirror: done, k
   double* h_scal = nullptr;  // pinned host mirror of a few doubles
   frk::Prof prof;
