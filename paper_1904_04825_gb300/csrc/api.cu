@@ -151,7 +151,7 @@ int create(const fr_mesh_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->z, n));
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
-  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
+  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kMaxVec));
   FRK_TRY(dalloc(c, &c->red.counter, 64));
   c->cyc_bar = c->red.counter + 32;  // a line of its own
   c->gd.ldh = m + 1;
@@ -239,7 +239,7 @@ int create3d(const fr_mesh3d_desc* mesh, int p, const fr_opts* o, fr_ctx* c) {
   FRK_TRY(dalloc(c, &c->z, n));
   for (double*& b : c->buf) FRK_TRY(dalloc(c, &b, n));
   FRK_TRY(dalloc(c, &c->scal, S_COUNT));
-  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kCycleColumns));
+  FRK_TRY(dalloc(c, &c->red.partials, (size_t)kRedBlocks * kMaxVec));
   FRK_TRY(dalloc(c, &c->red.counter, 64));
   c->cyc_bar = c->red.counter + 32;  // a line of its own
   c->gd.ldh = m + 1;

@@ -29,9 +29,9 @@
 namespace frk {
 namespace cyc {
 
-constexpr int kColApply = kMaxVec, kColUpdate = kMaxVec + 1, kColU = kMaxVec + 2, kColB = kMaxVec + 3,
-              kColX = kMaxVec + 4;  // partial-sum columns beside the dot products'
-static_assert(kColX < kCycleColumns, "partial columns");
+constexpr int kColApply = kCycleDots, kColUpdate = kCycleDots + 1, kColU = kCycleDots + 2, kColB = kCycleDots + 3,
+              kColX = kCycleDots + 4;  // partial-sum columns beside the dot products'
+static_assert(kColX < kMaxVec, "partial columns");
 constexpr unsigned kBarrierPolls = 1u << 24;  // seconds; far above any phase
 
 // what a CTA keeps in shared memory beside the phase's buffer

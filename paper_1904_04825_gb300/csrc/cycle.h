@@ -7,7 +7,7 @@ namespace frk {
 
 constexpr int kCycleThreads = 256;         // the vector kernels' block size, whose blocks are the work items
 constexpr int kCyclePerSm = 2;             // resident CTAs per SM the kernel is compiled for
-constexpr int kCycleColumns = kMaxVec + 8; // columns of partial sums
+constexpr int kCycleDots = kMaxVec - 5;    // columns of partial sums for dot products; five more follow
 static_assert(kCycleThreads == kThreads, "a work item is one block of the vector kernels");
 
 enum { kCycleConverged = 0, kCycleNotConverged = 1, kCycleNonFinite = 2, kCycleTimeout = 3 };
@@ -26,7 +26,7 @@ struct CycleArgs {
   long long n, ne;
   const double* b;
   double* x;
-  Reduce red;              // kCycleColumns columns
+  Reduce red;
   GmresDev gd;
   double eta2, rtol;
   int m, max_restarts, vgrid, agrid;  // blocks of the vector kernels and of the apply

@@ -402,7 +402,7 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
 int gmres_impl(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b,
                double* x, int m, double rtol, int max_restarts, bool x_is_zero,
                fr_gmres_info* info, cudaStream_t s) {
-  if (cycle_supported(ctx))
+  if (m + 1 <= kCycleDots && cycle_supported(ctx))  // <V_i, w> of up to m vectors and <w, w>
     return gmres_one_launch(ctx, U, R0, shift, b, x, m, rtol, max_restarts, x_is_zero, info, s);
   const long long n = ctx->ndof;
   double* sc = ctx->scal;
