@@ -21,7 +21,7 @@
 // output.  The layers of one tile follow one another, each with an epilogue of
 // 1-2.5 us, and this chain (about 10 us a tile) bounds the kernel, not the MMAs
 // (3 us), the weights or X.
-// 73,728 rows of 300-256-256-100: 50 us, 157 us as four kernels; X and Y alone
+// 73,728 rows of 300-256-256-100: 51 us, 157 us as four kernels; X and Y alone
 // take 17 us at the HBM rate.
 // Every wait is bounded; a wait that gives up sets *err, and copies and MMAs that
 // were issued are waited for (bounded) before the tensor memory is freed.
