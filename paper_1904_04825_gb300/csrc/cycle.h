@@ -49,8 +49,10 @@ FRK_CYCLE_ENTRY(f32)
 FRK_CYCLE_ENTRY(bf16)
 #undef FRK_CYCLE_ENTRY
 
-// whether the context's solves run as one launch; the context's arguments; the grid
-bool cycle_supported(const fr_ctx* ctx);
+// whether a solve of restart length m runs as one launch (it then writes x whole
+// where the guess is zero; the separate launches add to the zeros they are given);
+// the context's arguments; the grid
+bool solves_in_one_launch(const fr_ctx* ctx, int m);
 int fill_cycle_args(fr_ctx* ctx, const double* U, const double* R0, double shift, double rtol, int m, int max_restarts,
                     CycleArgs* a);
 int launch_cycle(int prec, const CycleArgs& a, int nblocks, int riemann, cudaStream_t s);

@@ -318,8 +318,9 @@ int gmres_cycle_enqueue(fr_ctx* ctx, const double* U, const double* R0, double s
 // and four CTAs per SM win; the 14,400-unknown ROW2 step takes 2.9 against 5.2 ms.
 constexpr long long kCycleMaxDof = 200000;
 
-bool cycle_supported(const fr_ctx* ctx) {
-  return !ctx->dim3 && !ctx->viscous && ctx->opts.jv_precision == 0 && ctx->opts.precond && ctx->p >= 2 && ctx->p <= 4 &&
+bool solves_in_one_launch(const fr_ctx* ctx, int m) {
+  return m + 1 <= kCycleDots &&  // <V_i, w> of up to m vectors and <w, w>
+         !ctx->dim3 && !ctx->viscous && ctx->opts.jv_precision == 0 && ctx->opts.precond && ctx->p >= 2 && ctx->p <= 4 &&
          ctx->ndof <= kCycleMaxDof && ctx->prof.mask == 0 && !ctx->test_skip_copy && cycle_grid(ctx) > 0;
 }
 
@@ -402,7 +403,7 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
 int gmres_impl(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b,
                double* x, int m, double rtol, int max_restarts, bool x_is_zero,
                fr_gmres_info* info, cudaStream_t s) {
-  if (m + 1 <= kCycleDots && cycle_supported(ctx))  // <V_i, w> of up to m vectors and <w, w>
+  if (solves_in_one_launch(ctx, m))
     return gmres_one_launch(ctx, U, R0, shift, b, x, m, rtol, max_restarts, x_is_zero, info, s);
   const long long n = ctx->ndof;
   double* sc = ctx->scal;

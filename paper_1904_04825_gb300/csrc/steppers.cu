@@ -161,7 +161,7 @@ int read_scalar(fr_ctx* ctx, const double* dev, double* host, cudaStream_t s) {
 // Linear solve with zero initial guess: x = A^{-1} b at tolerance tol.
 int solve(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x,
           double tol, fr_step_stats* st, fr_gmres_info* info, cudaStream_t s) {
-  if (!cycle_supported(ctx)) FRK_TRY(launch_fill(ctx, x, 0.0, s));  // the one-launch solve writes x whole
+  if (!solves_in_one_launch(ctx, ctx->opts.gmres_m)) FRK_TRY(launch_fill(ctx, x, 0.0, s));
   const int rc = gmres_impl(ctx, U, R0, shift, b, x, ctx->opts.gmres_m, tol,
                             ctx->opts.gmres_max_restarts, true, info, s);
   st->gmres_iters += info->iters;

@@ -1,0 +1,64 @@
+"""Solves of small 2D Euler contexts that run as one launch: where they hand over to the
+separate launches, and how they end when a bounded wait gave up."""
+import numpy as np
+import pytest
+
+import synthetic as S
+from oracle.fr2d import Mesh
+from oracle.jfnk import Problem
+from oracle.steppers import PtcOpts, SolverOpts
+from oracle.steppers import step_bdf2 as o_bdf2
+from oracle.steppers import step_esdirk as o_esdirk
+from oracle.steppers import step_row as o_row
+from oracle.tableaus import ESDIRK, ROW
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fr():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    import paper_1904_04825_gb300 as mod
+    return mod
+
+
+def _t(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("m", [58, 59, 60, 63])
+@pytest.mark.parametrize("stepper", ["row", "esdirk", "bdf2"])
+def test_steps_around_the_longest_restart_of_one_launch(fr, m, stepper):
+    """One launch holds the partial sums of up to 58 basis vectors; longer restarts, the paper's 60
+    among them, take the separate launches, which add to the guess they are given.  The second and
+    later solves find the last solution in that buffer: steps against the oracle, at the tolerance
+    of the repository's stepper tests (1e-9 with solves to 1e-12)."""
+    p = 2
+    xe, ye = S.uniform_mesh(6)
+    X, Y = S.point_coords(xe, ye, p)
+    U0 = S.Vortex().state(X, Y)
+    prob = Problem(Mesh(xe, ye), p)
+    tight = SolverOpts(tol_lin=1e-12, m=m, max_restarts=40)
+    ctx = fr.Context(xe, ye, p, fr.default_opts(tol_lin=1e-12, m_max=m, gmres_m=m, gmres_max_restarts=40))
+    po, oo = fr.default_ptc_opts(tol_nl=1e-12, tol_lin=1e-3), PtcOpts(tol_nl=1e-12, tol_lin=1e-3)
+    U, Uo = _t(U0), U0.copy()
+    if stepper == "row":
+        for _ in range(2):
+            assert fr.step_row(ctx, 3, 0.1, U).converged
+            Uo, _s = o_row(prob, ROW[3](), 0.1, Uo, tight)
+    elif stepper == "esdirk":
+        assert fr.step_esdirk(ctx, 3, 0.1, U, po).converged
+        Uo, _s = o_esdirk(prob, ESDIRK[3](), 0.1, Uo, oo, tight)
+    else:
+        Up, Upo = ctx.empty(), None
+        for k in range(2):
+            assert fr.step_bdf2(ctx, 0.1, U, Up, k == 0, po).converged
+            Uo, Upo, _s = o_bdf2(prob, 0.1, Uo, Upo, k == 0, oo, tight)
+    assert _rel(U.cpu().numpy(), Uo) < 1e-9
+    ctx.close()
