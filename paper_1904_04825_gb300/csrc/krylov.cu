@@ -381,9 +381,11 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
   if (launch_cycle(ctx->opts.block_precision, a, cycle_grid(ctx), ctx->opts.riemann, s) !=
       FR_OK)
     return set_error(ctx, FR_ERR_CUDA, "launch of the solve failed: %s", cudaGetErrorString(cudaGetLastError()));
+  // the context's flag: a wait of this launch, or of an inversion or apply before it
+  FRK_CUDA(ctx, cudaMemcpyAsync(ctx->h_stat + 1, ctx->kerr, sizeof(int), cudaMemcpyDeviceToHost, s));
   FRK_CUDA(ctx, cudaStreamSynchronize(s));
   const CycleStatus& st = *ctx->h_cyc;
-  if (st.state == kCycleTimeout) return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
+  if (ctx->h_stat[1]) return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
   if (st.state == kCycleNonFinite) {
     if (info) *info = fr_gmres_info{};
     return set_error(ctx, FR_ERR_NONFINITE, "GMRES residual is not finite");

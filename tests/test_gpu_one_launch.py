@@ -62,3 +62,32 @@ def test_steps_around_the_longest_restart_of_one_launch(fr, m, stepper):
             Uo, Upo, _s = o_bdf2(prob, 0.1, Uo, Upo, k == 0, oo, tight)
     assert _rel(U.cpu().numpy(), Uo) < 1e-9
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_flag_of_an_earlier_wait_reaches_the_next_solve(fr, prec):
+    """A wait of the apply that gave up sets the context's flag: the next solve, and every later one
+    and every step, reports it, although their own waits end."""
+    import torch
+    p = 2
+    xe, ye = S.uniform_mesh(8)
+    X, Y = S.point_coords(xe, ye, p)
+    U = _t(S.Vortex().state(X, Y))
+    ctx = fr.Context(xe, ye, p, fr.default_opts(block_precision=prec))
+    R0, z = ctx.empty(), ctx.empty()
+    fr.fr_residual(ctx, U, R0)
+    fr.ejacobi_factor(ctx, U, R0, 20.0)
+    b = _t(S.random_vector(ctx.shape, 3))
+    assert fr.gmres_solve(ctx, U, R0, 20.0, b, torch.zeros_like(b)).converged
+    fr.fr_set_wait_test(ctx, polls=2000, skip_first_copy=True)
+    fr.ejacobi_apply(ctx, b, z)
+    fr.fr_set_wait_test(ctx)
+    for _ in range(2):
+        with pytest.raises(fr.FrError) as e:
+            fr.gmres_solve(ctx, U, R0, 20.0, b, torch.zeros_like(b))
+        assert e.value.code == fr.FR_ERR_TIMEOUT
+    with pytest.raises(fr.FrError) as e:
+        fr.step_row(ctx, 2, 0.05, U)
+    assert e.value.code == fr.FR_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    ctx.close()
