@@ -50,24 +50,27 @@ struct Grid {
   int bid, nblk;
   bool ok;
 };
-constexpr unsigned kDoneBit = 1u << 28;  // of the barrier counter: the cycle is done (set and cleared by the keeper)
+// The barrier counter: arrivals times two, which wrap at 2^32 (a solve may take any
+// number of barriers; the CTAs are never more than one barrier apart), and in bit 0
+// whether the cycle is done (set and cleared by the keeper).
+constexpr unsigned kDone = 1u, kArrival = 2u;
 
-// All CTAs of the instance arrive (this one adding `add` to the counter's high
-// bits), then all see what any of them wrote before.  s.flag: the done bit, which
+// All CTAs of the instance arrive (this one adding `add`, 0 or +-kDone, to the done
+// bit), then all see what any of them wrote before.  s.flag: the done bit, which
 // is settled at this barrier if the keeper changed it while arriving here or
 // earlier.  Returns false when the wait gave up.
 static __device__ __noinline__ bool barrier(Grid& g, Shared& s, unsigned add = 0u) {
-  g.target += (unsigned)g.nblk;
+  g.target += kArrival * (unsigned)g.nblk;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(g.counter, 1u + add);
+    atomicAdd(g.counter, kArrival + add);
     int flag = -1;
     for (unsigned it = 0; it < kBarrierPolls; ++it) {
       unsigned v;
       asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(g.counter) : "memory");
-      if ((v & (kDoneBit - 1u)) >= g.target) {
-        flag = v & kDoneBit ? 1 : 0;
+      if ((int)((v & ~kDone) - g.target) >= 0) {
+        flag = (int)(v & kDone);
         break;
       }
     }
@@ -300,7 +303,7 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
         }
         __syncthreads();
         const bool d = beta <= target;
-        done_add = d == done_set ? 0u : (d ? kDoneBit : 0u - kDoneBit);
+        done_add = d == done_set ? 0u : (d ? kDone : 0u - kDone);
         done_set = d;
       }
       double sc = beta > 0.0 ? 1.0 / beta : 0.0;
@@ -349,7 +352,7 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
           __syncthreads();
         }
         if (keeper && givens_phase(gd, j, nw2)) {
-          done_add = kDoneBit;
+          done_add = kDone;
           done_set = true;
         }
         const double hn = sqrt(nw2);
@@ -407,8 +410,8 @@ __device__ __forceinline__ void run(const CycleArgs& a, int bid, int nblk, Share
       atomicExch(a.err, 1);
       a.status->state = kCycleTimeout;
     }
-    const unsigned t = atomicAdd(a.bar, 1u) + 1u;
-    if ((t & (kDoneBit - 1u)) == g.target + (unsigned)nblk) atomicExch(a.bar, 0u);
+    const unsigned t = atomicAdd(a.bar, kArrival) + kArrival;
+    if ((t & ~kDone) == g.target + kArrival * (unsigned)nblk) atomicExch(a.bar, 0u);
   }
 }
 
