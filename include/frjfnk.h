@@ -505,7 +505,9 @@ enum {
  * runs out.  The CTA then flags the context, waits (bounded) for the copies
  * it did issue and leaves; the GMRES cycle that launched it returns
  * FR_ERR_TIMEOUT (as gmres_solve and the steppers do whenever a bounded wait
- * gave up).  Nothing faults.  A context that reported FR_ERR_TIMEOUT keeps
+ * gave up).  A solve that runs as one launch, which skip_first_copy turns into
+ * separate ones, waits at its grid barriers for up to four times polls.
+ * Nothing faults.  A context that reported FR_ERR_TIMEOUT keeps
  * reporting it: destroy it. */
 int fr_set_wait_test(fr_ctx* ctx, unsigned polls, int skip_first_copy);
 

@@ -32,7 +32,6 @@ namespace cyc {
 constexpr int kColApply = kCycleDots, kColUpdate = kCycleDots + 1, kColU = kCycleDots + 2, kColB = kCycleDots + 3,
               kColX = kCycleDots + 4;  // partial-sum columns beside the dot products'
 static_assert(kColX < kMaxVec, "partial columns");
-constexpr unsigned kBarrierPolls = 1u << 24;  // seconds; far above any phase
 
 // what a CTA keeps in shared memory beside the phase's buffer
 struct Shared {
@@ -46,7 +45,7 @@ struct Shared {
 
 struct Grid {
   unsigned* counter;
-  unsigned target;
+  unsigned target, polls;
   int bid, nblk;
   bool ok;
 };
@@ -58,7 +57,7 @@ constexpr unsigned kDone = 1u, kArrival = 2u;
 // All CTAs of the instance arrive (this one adding `add`, 0 or +-kDone, to the done
 // bit), then all see what any of them wrote before.  s.flag: the done bit, which
 // is settled at this barrier if the keeper changed it while arriving here or
-// earlier.  Returns false when the wait gave up.
+// earlier.  Returns false when the wait gave up after `polls` looks.
 static __device__ __noinline__ bool barrier(Grid& g, Shared& s, unsigned add = 0u) {
   g.target += kArrival * (unsigned)g.nblk;
   __syncthreads();
@@ -66,7 +65,7 @@ static __device__ __noinline__ bool barrier(Grid& g, Shared& s, unsigned add = 0
     __threadfence();
     atomicAdd(g.counter, kArrival + add);
     int flag = -1;
-    for (unsigned it = 0; it < kBarrierPolls; ++it) {
+    for (unsigned it = 0; it < g.polls; ++it) {
       unsigned v;
       asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(g.counter) : "memory");
       if ((int)((v & ~kDone) - g.target) >= 0) {
@@ -394,7 +393,7 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
 
 template <int RM, typename S, typename A>
 __device__ __forceinline__ void run(const CycleArgs& a, int bid, int nblk, Shared& s, unsigned char* smem) {
-  Grid g{a.bar, 0u, bid, nblk, true};
+  Grid g{a.bar, 0u, a.polls, bid, nblk, true};
   switch (a.p * 2 + (a.small_tile ? 1 : 0)) {
     case 4: solve<2, 0, RM, S, A>(a, g, s, smem); break;
     case 5: solve<2, 2, RM, S, A>(a, g, s, smem); break;
@@ -403,13 +402,11 @@ __device__ __forceinline__ void run(const CycleArgs& a, int bid, int nblk, Share
     case 8: solve<4, 0, RM, S, A>(a, g, s, smem); break;
     case 9: solve<4, 2, RM, S, A>(a, g, s, smem); break;
   }
-  // the last CTA to leave sets the counter back for the next launch
+  // the last CTA to leave sets the counter back for the next launch (after a wait
+  // that gave up the host does, which reads *err)
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (!g.ok) {
-      atomicExch(a.err, 1);
-      a.status->state = kCycleTimeout;
-    }
+    if (!g.ok) atomicExch(a.err, 1);
     const unsigned t = atomicAdd(a.bar, kArrival) + kArrival;
     if ((t & ~kDone) == g.target + kArrival * (unsigned)nblk) atomicExch(a.bar, 0u);
   }

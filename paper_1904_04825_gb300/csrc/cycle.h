@@ -10,7 +10,8 @@ constexpr int kCyclePerSm = 2;             // resident CTAs per SM the kernel is
 constexpr int kCycleDots = kMaxVec - 5;    // columns of partial sums for dot products; five more follow
 static_assert(kCycleThreads == kThreads, "a work item is one block of the vector kernels");
 
-enum { kCycleConverged = 0, kCycleNotConverged = 1, kCycleNonFinite = 2, kCycleTimeout = 3 };
+enum { kCycleConverged = 0, kCycleNotConverged = 1, kCycleNonFinite = 2 };
+// how a solve ended, if none of its waits gave up (CycleArgs::err)
 struct CycleStatus {
   int iters, restarts, state, pad;
   double relres;
@@ -31,8 +32,9 @@ struct CycleArgs {
   double eta2, rtol;
   int m, max_restarts, vgrid, agrid;  // blocks of the vector kernels and of the apply
   int x_zero;              // x is zero on entry (and need not be filled)
-  unsigned* bar;
-  int* err;
+  unsigned* bar;           // the grid barriers' counter, zero at the launch
+  unsigned polls;          // limit of every wait at a grid barrier
+  int* err;                // set when one gave up
   CycleStatus* status;     // pinned host memory
 };
 

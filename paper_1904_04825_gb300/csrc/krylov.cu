@@ -365,6 +365,7 @@ int fill_cycle_args(fr_ctx* ctx, const double* U, const double* R0, double shift
   a->vgrid = (int)vgrid(ctx, ctx->ndof);
   a->agrid = (int)apply_grid_of(ctx);
   a->bar = ctx->cyc_bar;
+  a->polls = ctx->wait_polls < 1u << 30 ? 4 * ctx->wait_polls : ~0u;  // phases are longer than copies
   a->err = ctx->kerr;
   a->status = ctx->h_cyc;
   return a->agrid > 0 ? FR_OK : FR_ERR_UNSUPPORTED;
@@ -385,7 +386,12 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
   FRK_CUDA(ctx, cudaMemcpyAsync(ctx->h_stat + 1, ctx->kerr, sizeof(int), cudaMemcpyDeviceToHost, s));
   FRK_CUDA(ctx, cudaStreamSynchronize(s));
   const CycleStatus& st = *ctx->h_cyc;
-  if (ctx->h_stat[1]) return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
+  if (ctx->h_stat[1]) {
+    // CTAs that left a barrier early leave its counter anywhere
+    FRK_CUDA(ctx, cudaMemsetAsync(ctx->cyc_bar, 0, sizeof(unsigned), s));
+    FRK_CUDA(ctx, cudaStreamSynchronize(s));
+    return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
+  }
   if (st.state == kCycleNonFinite) {
     if (info) *info = fr_gmres_info{};
     return set_error(ctx, FR_ERR_NONFINITE, "GMRES residual is not finite");

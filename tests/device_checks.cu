@@ -10,7 +10,7 @@ namespace {
 // with every third round and clears it with the next.
 __global__ void k_barrier_rounds(unsigned* counter, unsigned start, int* notes, int rounds, int* errors) {
   __shared__ frk::cyc::Shared s;
-  frk::cyc::Grid g{counter, start, (int)blockIdx.x, (int)gridDim.x, true};
+  frk::cyc::Grid g{counter, start, 1u << 22, (int)blockIdx.x, (int)gridDim.x, true};
   const bool keeper = g.bid == g.nblk - 1;
   for (int r = 0; r < rounds; ++r) {
     if (threadIdx.x == 0) *(volatile int*)(notes + g.bid) = r;

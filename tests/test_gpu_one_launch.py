@@ -91,3 +91,39 @@ def test_flag_of_an_earlier_wait_reaches_the_next_solve(fr, prec):
     assert e.value.code == fr.FR_ERR_TIMEOUT
     torch.cuda.synchronize()
     ctx.close()
+
+
+@pytest.mark.parametrize("prec,nx,ny", [(0, 61, 50), (2, 40, 11)])
+def test_grid_barrier_runs_out_and_the_context_keeps_saying_so(fr, prec, nx, ny):
+    """With a limit of a few looks the CTAs without a tile give up at the grid barrier: the solve
+    returns FR_ERR_TIMEOUT, and so does every later one of that context, with the default limit too.
+    Another context then solves as before."""
+    import torch
+    p = 3
+    xe, ye = S.uniform_mesh(nx)[0], S.uniform_mesh(ny)[1]
+    X, Y = S.point_coords(xe, ye, p)
+    U = _t(S.smooth_random_state(X, Y, seed=nx, amp=0.05))
+    b = _t(S.random_vector(U.shape, 3))
+
+    def context():
+        ctx = fr.Context(xe, ye, p, fr.default_opts(block_precision=prec))
+        R0 = ctx.empty()
+        fr.fr_residual(ctx, U, R0)
+        fr.ejacobi_factor(ctx, U, R0, 20.0)
+        return ctx, R0
+
+    ctx, R0 = context()
+    want = torch.zeros_like(b)
+    assert fr.gmres_solve(ctx, U, R0, 20.0, b, want).converged
+    for polls in (1, 0, 0):
+        fr.fr_set_wait_test(ctx, polls=polls)
+        with pytest.raises(fr.FrError) as e:
+            fr.gmres_solve(ctx, U, R0, 20.0, b, torch.zeros_like(b))
+        assert e.value.code == fr.FR_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    ctx.close()
+    ctx, R0 = context()
+    x = torch.zeros_like(b)
+    assert fr.gmres_solve(ctx, U, R0, 20.0, b, x).converged
+    assert torch.equal(x, want)
+    ctx.close()
