@@ -132,8 +132,8 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
       }
     }
     // ---- the panel back into M; U and x_P as integers ----
+    int ep = 0;  // largest exponent of the row's U, taken over its threads by whole warps
     if (mine) {
-      int e = 0;
 #pragma unroll
       for (int t = 0; t < CPT; ++t) {
         const int c = half * CPT + t;
@@ -143,12 +143,14 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
         } else {
           pv[t] = 0.0;
         }
-        e = max(e, fx::exponent(pv[t]));
+        ep = max(ep, fx::exponent(pv[t]));
       }
-      if (TPR == 2) e = max(e, __shfl_xor_sync(__activemask(), e, 1));
-      if (half == 0) eU[row] = e;
+    }
+    if (TPR == 2) ep = max(ep, __shfl_xor_sync(0xffffffffu, ep, 1));
+    if (mine) {
+      if (half == 0) eU[row] = ep;
 #pragma unroll
-      for (int t = 0; t < CPT; ++t) U[(half * CPT + t) * ROWS + row] = fx::split(pv[t], e);
+      for (int t = 0; t < CPT; ++t) U[(half * CPT + t) * ROWS + row] = fx::split(pv[t], ep);
     }
     for (int j = tid; j < NB; j += THREADS) {
       if (j >= c0 && j < c0 + kb) continue;

@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include "cycle.cuh"
+#include "gj_fx.cuh"
 
 namespace {
 
@@ -28,7 +29,57 @@ __global__ void k_barrier_rounds(unsigned* counter, unsigned start, int* notes, 
   }
 }
 
+// Inverse of the row-major n x n FP64 matrix M, one CTA, by gjfx::invert.
+template <int NB> struct InverseLayout {
+  static constexpr int LD = NB + 1, THREADS = NB <= 64 ? 128 : 256;
+  static constexpr size_t OFF_PIV = (size_t)NB * LD * sizeof(double);
+  static constexpr size_t OFF_SCRATCH = (OFF_PIV + NB * sizeof(int) + 127) / 128 * 128;
+  static constexpr size_t BYTES = OFF_SCRATCH + frk::gjfx::Shape<NB, THREADS>::BYTES;
+};
+template <int NB>
+__global__ void __launch_bounds__(InverseLayout<NB>::THREADS) k_inverse(const double* M, double* inv) {
+  using L = InverseLayout<NB>;
+  extern __shared__ __align__(128) unsigned char smem[];
+  double* A = reinterpret_cast<double*>(smem);
+  int* piv = reinterpret_cast<int*>(smem + L::OFF_PIV);
+  unsigned char* scratch = smem + L::OFF_SCRATCH;
+  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) A[i / NB * L::LD + i % NB] = M[i];
+  __syncthreads();
+  frk::gjfx::invert<NB, L::LD, L::THREADS>(A, piv, scratch);
+  const int* ipr = reinterpret_cast<const int*>(scratch + frk::gjfx::Shape<NB, L::THREADS>::OFF_IPR);
+  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) inv[i] = A[piv[i / NB] * L::LD + ipr[i % NB]];
+}
+template <int NB>
+int inverse(const double* M, double* inv) {
+  using L = InverseLayout<NB>;
+  const size_t bytes = sizeof(double) * NB * NB;
+  double* dev = nullptr;
+  if (cudaMalloc(&dev, 2 * bytes) != cudaSuccess) return -1;
+  int rc = -1;
+  if (cudaMemcpy(dev, M, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+      cudaFuncSetAttribute(k_inverse<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES) == cudaSuccess) {
+    k_inverse<NB><<<1, L::THREADS, L::BYTES>>>(dev, dev + NB * NB);
+    if (cudaGetLastError() == cudaSuccess && cudaMemcpy(inv, dev + NB * NB, bytes, cudaMemcpyDeviceToHost) == cudaSuccess)
+      rc = 0;
+  }
+  cudaFree(dev);
+  return rc;
+}
+
 }  // namespace
+
+// 0 and the inverse of the n x n matrix M (host, row-major), or -1.
+extern "C" int fp64_inverse(int n, const double* M, double* inv) {
+  switch (n) {
+    case 36: return inverse<36>(M, inv);
+    case 40: return inverse<40>(M, inv);
+    case 64: return inverse<64>(M, inv);
+    case 100: return inverse<100>(M, inv);
+    case 135: return inverse<135>(M, inv);
+    case 144: return inverse<144>(M, inv);
+    default: return -1;
+  }
+}
 
 // Errors of `rounds` rounds over nblk CTAs from the counter value `start`, or -1.
 extern "C" int check_barrier(int nblk, unsigned start, int rounds) {
