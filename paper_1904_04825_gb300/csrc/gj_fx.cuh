@@ -1,13 +1,23 @@
 // Gauss-Jordan inversion of one FP64 element block (the element-Jacobi
 // preconditioner of Sec. 4.5) with the trailing updates on the integer units.
 //
-// In-place Gauss-Jordan with partial pivoting in panels of BW = 16 columns, the
-// algorithm of gj_tc.cuh: a panel's pivots are found and eliminated on the panel's
+// In-place Gauss-Jordan with partial pivoting in panels of BW = 16 columns, like
+// gj_tc.cuh: a panel's pivots are found and eliminated on the panel's
 // columns alone in FP64 (the rows in registers, TPR threads a row), rows stay in
 // place (pr[c] = the pivot row of column c); then every other column takes
-//   M[:, j] += U x_P[:, j],  U = panel - unit vectors of the pivot rows,
-// a rank-16 update whose sums of 16 products are formed as integers (fx.cuh, one
-// exponent per row of U and per column of x_P) and added to M with one rounding.
+//   M[:, j] = (0 in the pivot rows, M[:, j] in the others) + U x_P[:, j],
+// U the panel after its pivots and x_P the pivot rows before them, a rank-16 update
+// whose sums of 16 products are formed as integers (fx.cuh) and added to M with one
+// rounding.  A pivot row is formed from the products alone: as M + (U - 1) x_P, a
+// difference of nearly equal numbers where the pivot is large, it kept only the
+// absolute accuracy of M, and one variable of the inverse lost 8 digits in SI units.
+// An operand keeps 57 bits below its group's largest value (groups: a row of U, a
+// column of x_P), so term k of the sums is scaled by 2^t_k, which leaves the products
+// as they are and evens the groups: t_k the largest exponent of row k of x_P, each
+// column's entries taken relative to its largest.  That takes out whatever units the
+// rows and columns have.  Worst variable of M^-1 r against the exact inverse, by
+// elimination one pivot at a time in FP64 / here: unit scaling 7e-16 / 4e-16, cells of
+// 1e-4 width 2e-14 / 2e-14, SI units (p = 2) 5e-13 / 2e-13.
 // The result is the inverse with permuted rows and columns:
 // inverse(a, b) = M[pr[a]][ipr[b]].
 //
@@ -15,7 +25,7 @@
 // NB^2 BW of them stay in the panels, and an updated entry costs 2 FP64
 // operations per panel instead of 16: at NB = 64 90 thousand instead of 262
 // thousand.  Formation and inversion of the 25,600 blocks of the 160 x 160, p = 3
-// mesh: 9.0 ms, 17.6 ms by rank-1 elimination in shared memory (five
+// mesh: 9.2 ms, 17.8 ms by rank-1 elimination in shared memory (five
 // barriers and an integer division per entry and pivot).  Panels of 8 or 32
 // columns would put more into the updates' roundings or the panels.
 #pragma once
@@ -35,7 +45,8 @@ struct Shape {
   static constexpr int ROWS = (NB + 3) / 4 * 4;          // U rows, whole quadruples
   static_assert(NB * TPR <= THREADS, "a thread per row");
   // scratch: U [BW][ROWS], X [BW][COLS] (int2, 16-byte aligned), exponents, the
-  // pivot column and scaled pivot row, candidates per warp, inverse permutation
+  // pivot column and scaled pivot row, candidates per warp, pivot rows, the terms'
+  // scales t_k, inverse permutation
   static constexpr size_t OFF_U = 0;
   static constexpr size_t OFF_X = OFF_U + (size_t)BW * ROWS * 8;
   static constexpr size_t OFF_COL = OFF_X + (size_t)BW * COLS * 8;
@@ -44,7 +55,8 @@ struct Shape {
   static constexpr size_t OFF_EX = OFF_EU + (size_t)ROWS * 4;
   static constexpr size_t OFF_CAND = OFF_EX + (size_t)COLS * 4;
   static constexpr size_t OFF_ROWS = OFF_CAND + 16 * 8;
-  static constexpr size_t OFF_IPR = OFF_ROWS + BW * 4;
+  static constexpr size_t OFF_T = OFF_ROWS + BW * 4;
+  static constexpr size_t OFF_IPR = OFF_T + BW * 4;
   static constexpr size_t BYTES = (OFF_IPR + (size_t)NB * 4 + 15) / 16 * 16;
 };
 
@@ -63,6 +75,7 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
   int* eX = reinterpret_cast<int*>(scratch + Sh::OFF_EX);
   uint2* cand = reinterpret_cast<uint2*>(scratch + Sh::OFF_CAND);
   int* rows = reinterpret_cast<int*>(scratch + Sh::OFF_ROWS);
+  int* ts = reinterpret_cast<int*>(scratch + Sh::OFF_T);
   int* ipr = reinterpret_cast<int*>(scratch + Sh::OFF_IPR);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row = tid / TPR, half = tid % TPR;  // this thread's row and columns [half CPT, ...) of a panel
@@ -75,7 +88,9 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
 
   for (int c0 = 0; c0 < NB; c0 += BW) {
     const int kb = NB - c0 < BW ? NB - c0 : BW;
+    if (tid < BW) ts[tid] = fx::kNone;
     // ---- the panel's pivots ----
+    bool pivot = false;  // this row is one of them
     double pv[CPT];
 #pragma unroll
     for (int t = 0; t < CPT; ++t) {
@@ -108,7 +123,7 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
       if (row == r) {
 #pragma unroll
         for (int t = 0; t < CPT; ++t) srow[half * CPT + t] = half == kh && t == kt ? 1.0 : pv[t];
-        used = true;
+        used = pivot = true;
         if (half == 0) {
           srow[BW] = rcp_fast(pc[r]);
           pr[c0 + k] = r;
@@ -131,42 +146,58 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
         }
       }
     }
-    // ---- the panel back into M; U and x_P as integers ----
-    int ep = 0;  // largest exponent of the row's U, taken over its threads by whole warps
+    // ---- the panel back into M; the scales of the terms from x_P ----
     if (mine) {
 #pragma unroll
-      for (int t = 0; t < CPT; ++t) {
-        const int c = half * CPT + t;
-        if (c < kb) {
-          M[row * LD + c0 + c] = pv[t];
-          if (row == rows[c]) pv[t] -= 1.0;
-        } else {
-          pv[t] = 0.0;
-        }
-        ep = max(ep, fx::exponent(pv[t]));
+      for (int t = 0; t < CPT; ++t)
+        if (half * CPT + t < kb) M[row * LD + c0 + half * CPT + t] = pv[t];
+        else pv[t] = 0.0;
+    }
+    const bool other = tid < NB && !(tid >= c0 && tid < c0 + kb);  // this thread's column of x_P
+    if (warp * 32 < NB) {
+      int ex[BW], top = 0, best = fx::kNone;
+#pragma unroll
+      for (int k = 0; k < BW; ++k) {
+        ex[k] = other && k < kb ? fx::exponent_of(M[rows[k] * LD + tid], 0) : fx::kNone;
+        top = max(top, ex[k]);
       }
+#pragma unroll
+      for (int k = 0; k < BW; ++k) {
+        const int m = __reduce_max_sync(0xffffffffu, ex[k] - top);
+        if (lane == k) best = m;
+      }
+      // (a row of zeros stays near kNone, and its column of U becomes zero too)
+      if (lane < BW) atomicMax(ts + lane, best);
+    }
+    __syncthreads();
+    // ---- U and x_P as integers ----
+    int ep = fx::kNone;  // largest exponent of the row's U, taken over its threads by whole warps
+    int tk[CPT];
+#pragma unroll
+    for (int t = 0; t < CPT; ++t) {
+      tk[t] = ts[half * CPT + t];
+      if (mine) ep = max(ep, fx::exponent_of(pv[t], tk[t]));
     }
     if (TPR == 2) ep = max(ep, __shfl_xor_sync(0xffffffffu, ep, 1));
     if (mine) {
-      if (half == 0) eU[row] = ep;
+      if (half == 0) eU[row] = 2 * ep + (pivot ? 1 : 0);
 #pragma unroll
-      for (int t = 0; t < CPT; ++t) U[(half * CPT + t) * ROWS + row] = fx::split(pv[t], ep);
+      for (int t = 0; t < CPT; ++t) U[(half * CPT + t) * ROWS + row] = fx::split(pv[t], tk[t], ep);
     }
-    for (int j = tid; j < NB; j += THREADS) {
-      if (j >= c0 && j < c0 + kb) continue;
-      int e = 0;
-      double x[BW];
+    if (other) {
+      int e = fx::kNone;
+      double x[BW];  // read again rather than held over the barrier: at 100 rows 122 registers, not 174
 #pragma unroll
       for (int k = 0; k < BW; ++k) {
-        x[k] = k < kb ? M[rows[k] * LD + j] : 0.0;
-        e = max(e, fx::exponent(x[k]));
+        x[k] = k < kb ? M[rows[k] * LD + tid] : 0.0;
+        e = max(e, fx::exponent_of(x[k], -ts[k]));
       }
-      eX[j] = e;
+      eX[tid] = e;
 #pragma unroll
-      for (int k = 0; k < BW; ++k) X[k * COLS + j] = fx::split(x[k], e);
+      for (int k = 0; k < BW; ++k) X[k * COLS + tid] = fx::split(x[k], -ts[k], e);
     }
     __syncthreads();
-    // ---- M[:, j] += U x_P[:, j], tiles of 4 rows x 2 columns per thread ----
+    // ---- M[:, j] = (M[:, j] or 0) + U x_P[:, j], tiles of 4 rows x 2 columns per thread ----
     constexpr int TJ = COLS / 2, TI = ROWS / 4;
     const bool first = kb == NB;
     for (int tile = tid; tile < TI * TJ && !first; tile += THREADS) {
@@ -194,7 +225,8 @@ __device__ void invert(double* M, int* pr, unsigned char* scratch) {
         for (int p = 0; p < 4; ++p)
           if (i + p < NB) {
             double* m = M + (i + p) * LD + jj;
-            *m = fma(fx::value(a[p][q]), fx::scale(eU[i + p], eX[jj]), *m);
+            const int eu = eU[i + p];  // exponent times two, and in bit 0 whether the row is a pivot row
+            *m = fma(fx::value(a[p][q]), fx::scale(eu >> 1, eX[jj]), eu & 1 ? 0.0 : *m);
           }
       }
     }

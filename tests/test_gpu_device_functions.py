@@ -7,6 +7,10 @@ import subprocess
 import numpy as np
 import pytest
 
+import synthetic as S
+from oracle.fr2d import Mesh
+from oracle.jfnk import Problem, element_blocks
+
 pytestmark = pytest.mark.gpu
 
 
@@ -50,6 +54,51 @@ def test_fp64_block_inverse_at_every_width(dev, n):
     M = 4.0 * np.eye(n) + np.random.default_rng(n).standard_normal((n, n)) / np.sqrt(n)
     want = _exact_inverse(M)
     assert np.abs(_inverse(dev, M) - want).max() < 1.6e-13 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("case", ["unit", "thin cells", "SI, shift 1e6", "SI, shift 1e4", "units far apart"])
+@pytest.mark.parametrize("p", [2, 3, 4, 5])
+def test_fp64_block_inverse_of_badly_scaled_blocks(dev, p, case):
+    """M^-1 r of the oracle's element blocks, variable by variable, against the exact inverse: cells 1e-4
+    thin, air in SI units on centimetre cells (density 1.2, speed of sound 340, energy 2e5), and variables
+    in units that differ by 2^27, 2^-17 and 2^40.  One-pivot-at-a-time elimination in FP64
+    with the same pivot rule, emulated on the CPU, leaves up to 5e-13 (SI, p = 2, where pivots fall
+    across variables): bound 1e-12.  Powers of two change no rounding but the choice of pivots (1e-11
+    in the emulation at p = 2): bound 1e-10 there."""
+    xe, ye = S.stretched_mesh(3, 2, seed=p)
+    base = dict(seed=3, amp=0.05, base=(1.0, 0.7, -0.4, 2.0))
+    if case == "thin cells":
+        X, Y = S.point_coords(xe, np.array([0.0, 1.0, 2.0]), p)
+        M = element_blocks(Problem(Mesh(xe, np.array([0.0, 1e-4, 2e-4])), p), S.smooth_random_state(X, Y, **base), 30.0)[0]
+    else:
+        X, Y = S.point_coords(xe, ye, p)
+        U = S.smooth_random_state(X, Y, **base)
+        if case.startswith("SI"):
+            U = U * (1.2 * np.array([1.0, 290.0, 290.0, 290.0**2]))[None, :, None]
+            M = element_blocks(Problem(Mesh(0.01 * xe, 0.01 * ye), p), U, float(case.split()[-1]))[0]
+        else:
+            M = element_blocks(Problem(Mesh(xe, ye), p), U, 30.0)[0]
+    n, npt = len(M), (p + 1) ** 2
+    rng = np.random.default_rng(p)
+    if case == "units far apart":
+        d = np.repeat(np.exp2([0, 27, -17, 40]), npt)
+        M = d[:, None] * M / d
+    want, got = _exact_inverse(M), _inverse(dev, M)
+    size = [float(np.median(np.abs(want[v * npt:(v + 1) * npt, v * npt:(v + 1) * npt]))) for v in range(4)]
+    for _ in range(4):
+        r = rng.standard_normal(n) / np.repeat(size, npt)
+        z, err = want @ r, (got - want) @ r
+        for v in range(4):
+            k = slice(v * npt, (v + 1) * npt)
+            assert np.linalg.norm(err[k]) < (1e-10 if case == "units far apart" else 1e-12) * np.linalg.norm(z[k])
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_fp64_block_inverse_of_non_finite_blocks(dev, bad):
+    """A non-finite entry spreads over the inverse instead of vanishing in an integer."""
+    M = 4.0 * np.eye(64) + np.random.default_rng(1).standard_normal((64, 64)) / 8.0
+    M[17, 40] = bad
+    assert not np.isfinite(_inverse(dev, M)).all()
 
 
 @pytest.mark.parametrize("nblk", [1, 2, 19, 32])
