@@ -402,13 +402,18 @@ __device__ __forceinline__ void run(const CycleArgs& a, int bid, int nblk, Share
     case 8: solve<4, 0, RM, S, A>(a, g, s, smem); break;
     case 9: solve<4, 2, RM, S, A>(a, g, s, smem); break;
   }
-  // the last CTA to leave sets the counter back for the next launch (after a wait
-  // that gave up the host does, which reads *err)
+  // the last CTA to leave sets the counter back for the next launch and passes the
+  // context's flag on (after a wait that gave up the host clears the counter)
   __syncthreads();
   if (threadIdx.x == 0) {
     if (!g.ok) atomicExch(a.err, 1);
+    __threadfence();  // the flag before the arrival
     const unsigned t = atomicAdd(a.bar, kArrival) + kArrival;
-    if ((t & ~kDone) == g.target + kArrival * (unsigned)nblk) atomicExch(a.bar, 0u);
+    if ((t & ~kDone) == g.target + kArrival * (unsigned)nblk) {
+      __threadfence();
+      a.status->err = *(volatile const int*)a.err;
+      atomicExch(a.bar, 0u);
+    }
   }
 }
 

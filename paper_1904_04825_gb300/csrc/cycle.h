@@ -11,9 +11,10 @@ constexpr int kCycleDots = kMaxVec - 5;    // columns of partial sums for dot pr
 static_assert(kCycleThreads == kThreads, "a work item is one block of the vector kernels");
 
 enum { kCycleConverged = 0, kCycleNotConverged = 1, kCycleNonFinite = 2 };
-// how a solve ended, if none of its waits gave up (CycleArgs::err)
+// how a solve ended
 struct CycleStatus {
-  int iters, restarts, state, pad;
+  int iters, restarts, state;
+  int err;                 // the context's flag as the last CTA left; 1 (the host's) if none saw itself as the last
   double relres;
 };
 

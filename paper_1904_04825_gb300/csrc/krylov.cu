@@ -379,14 +379,13 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
   a.b = b;
   a.x = x;
   a.x_zero = x_is_zero;
+  ctx->h_cyc->err = 1;
   if (launch_cycle(ctx->opts.block_precision, a, cycle_grid(ctx), ctx->opts.riemann, s) !=
       FR_OK)
     return set_error(ctx, FR_ERR_CUDA, "launch of the solve failed: %s", cudaGetErrorString(cudaGetLastError()));
-  // the context's flag: a wait of this launch, or of an inversion or apply before it
-  FRK_CUDA(ctx, cudaMemcpyAsync(ctx->h_stat + 1, ctx->kerr, sizeof(int), cudaMemcpyDeviceToHost, s));
   FRK_CUDA(ctx, cudaStreamSynchronize(s));
   const CycleStatus& st = *ctx->h_cyc;
-  if (ctx->h_stat[1]) {
+  if (st.err) {  // a wait of this launch, or of an inversion or apply before it
     // CTAs that left a barrier early leave its counter anywhere
     FRK_CUDA(ctx, cudaMemsetAsync(ctx->cyc_bar, 0, sizeof(unsigned), s));
     FRK_CUDA(ctx, cudaStreamSynchronize(s));
