@@ -21,6 +21,8 @@
 // bounded, and a wait that gives up sets *err and ends the CTA.
 #pragma once
 
+#include <atomic>
+
 #include "apply_body.cuh"
 #include "cycle.h"
 #include "krylov_body.cuh"
@@ -454,21 +456,23 @@ int launch(const CycleArgs& a, int nblocks, int riemann, cudaStream_t s) {
              : FR_ERR_CUDA;
 }
 
-// resident CTAs per SM, found once per process (with the shared-memory attribute)
+// resident CTAs per SM, found once per device (with the shared-memory attribute) by
+// whichever threads ask first; they find the same
 template <typename S, typename A>
-int resident(int riemann) {
-  static int occ[2] = {-1, -1};
-  if (occ[riemann] < 0) {
-    const void* f = kernel_of<S, A>(riemann);
-    int o = 0;
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cycle_smem<S, A>()) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, f, kCycleThreads, cycle_smem<S, A>()) != cudaSuccess) {
-      (void)cudaGetLastError();
-      o = 0;
-    }
-    occ[riemann] = o;
+int resident(int riemann, int device) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][2];  // one more than the number; 0: not yet known
+  std::atomic<int>* slot = device >= 0 && device < kDevices ? &known[device][riemann] : nullptr;
+  int o = slot ? slot->load(std::memory_order_relaxed) - 1 : -1;
+  if (o >= 0) return o;
+  const void* f = kernel_of<S, A>(riemann);
+  if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cycle_smem<S, A>()) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, f, kCycleThreads, cycle_smem<S, A>()) != cudaSuccess) {
+    (void)cudaGetLastError();
+    o = 0;
   }
-  return occ[riemann];
+  if (slot) slot->store(o + 1, std::memory_order_relaxed);
+  return o;
 }
 
 }  // namespace cyc

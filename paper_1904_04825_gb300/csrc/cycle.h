@@ -46,7 +46,7 @@ bool residual_small_tile(const fr_ctx* ctx);
 // by the block precision: the launch, and the resident CTAs per SM (0: cannot run)
 #define FRK_CYCLE_ENTRY(name)                                                          \
   int launch_cycle_##name(const CycleArgs& a, int nblocks, int riemann, cudaStream_t s); \
-  int resident_cycle_##name(int riemann);
+  int resident_cycle_##name(int riemann, int device);
 FRK_CYCLE_ENTRY(f64)
 FRK_CYCLE_ENTRY(f32)
 FRK_CYCLE_ENTRY(bf16)

@@ -329,9 +329,9 @@ bool solves_in_one_launch(const fr_ctx* ctx, int m) {
 int cycle_grid(const fr_ctx* ctx) {
   int occ = 0;
   switch (ctx->opts.block_precision) {
-    case 1: occ = resident_cycle_f32(ctx->opts.riemann); break;
-    case 2: occ = resident_cycle_bf16(ctx->opts.riemann); break;
-    default: occ = resident_cycle_f64(ctx->opts.riemann); break;
+    case 1: occ = resident_cycle_f32(ctx->opts.riemann, ctx->device); break;
+    case 2: occ = resident_cycle_bf16(ctx->opts.riemann, ctx->device); break;
+    default: occ = resident_cycle_f64(ctx->opts.riemann, ctx->device); break;
   }
   const int want = ctx->ndof <= 60000 ? 1 : 2;
   return (occ < want ? occ : want) * ctx->num_sms;

@@ -127,3 +127,44 @@ def test_grid_barrier_runs_out_and_the_context_keeps_saying_so(fr, prec, nx, ny)
     assert fr.gmres_solve(ctx, U, R0, 20.0, b, x).converged
     assert torch.equal(x, want)
     ctx.close()
+
+
+_FIRST_SOLVES = """
+import hashlib, sys, threading
+sys.path.insert(0, sys.argv[1])
+import torch
+import paper_1904_04825_gb300 as fr
+import synthetic as S
+cs = []
+for k in range(6):
+    xe, ye = S.uniform_mesh(10 + k)
+    U = torch.from_numpy(S.Vortex().state(*S.point_coords(xe, ye, 3))).cuda()
+    cs.append((fr.Context(xe, ye, 3, fr.default_opts(block_precision=k % 3, riemann=k // 3)), U, torch.cuda.Stream()))
+torch.cuda.synchronize()
+gate = threading.Barrier(6)
+def work(ctx, U, s):
+    gate.wait()
+    fr.step_row(ctx, 3, 0.05, U, stream=s.cuda_stream)
+if sys.argv[2] == "threads":
+    ts = [threading.Thread(target=work, args=c) for c in cs]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+else:
+    for ctx, U, s in cs:
+        fr.step_row(ctx, 3, 0.05, U, stream=s.cuda_stream)
+torch.cuda.synchronize()
+print([hashlib.sha1(U.cpu().numpy().tobytes()).hexdigest() for _, U, _ in cs])
+"""
+
+
+def test_first_solves_of_a_process_on_several_threads():
+    """The grid's size is found by the first solve of a process: six threads that solve first, together,
+    end with the bits of one thread after another."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = [subprocess.run([sys.executable, "-c", _FIRST_SOLVES, root, how], capture_output=True, text=True, timeout=300)
+           for how in ("threads", "in turn")]
+    assert out[0].returncode == 0 and out[1].returncode == 0, out[0].stderr + out[1].stderr
+    assert out[0].stdout == out[1].stdout
