@@ -261,7 +261,9 @@ int launch_solution_update(fr_ctx* ctx, double* x, cudaStream_t s);
 // krylov.cu
 int launch_sumsq(fr_ctx* ctx, const double* x, double* out, cudaStream_t s, bool with_eps = false);
 EpsArgs eps_args(fr_ctx* ctx, bool on);
-// ||U||^2, ||z||^2 and the FD step of the product A z in one launch
+// ||U||^2, ||z||^2 and the FD step of the product A z in one launch, which sums
+// kNormValues values (the partials it needs: kNormValues columns of kRedBlocks)
+constexpr int kNormValues = 2;
 int launch_norms_eps(fr_ctx* ctx, const double* U, const double* z, cudaStream_t s);
 int launch_lincomb(fr_ctx* ctx, double* out, int nterms, const double* const* xs,
                    const double* coefs, double* sumsq, cudaStream_t s);

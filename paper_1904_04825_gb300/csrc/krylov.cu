@@ -44,7 +44,8 @@ __global__ void k_sumsq2(const double* __restrict__ x, const double* __restrict_
     red.value(1)[blockIdx.x] = by;
   }
   if (last_block(red.counter)) {
-    finish_sums(red, 2, out);
+    static_assert(kNormValues == 2, "the scratch of fr_jv_noalloc holds the columns written here");
+    finish_sums(red, kNormValues, out);
     __syncthreads();
     if (threadIdx.x == 0) write_eps(ea, out[1]);
   }

@@ -19,7 +19,7 @@ constexpr size_t kOffYE = kOffXE + kNoAllocMaxCells + 1;         // y edges (ny+
 constexpr size_t kOffSX = kOffYE + kNoAllocMaxCells + 1;         // 2 / width (nx)
 constexpr size_t kOffSY = kOffSX + kNoAllocMaxCells;             // 2 / height (ny)
 constexpr size_t kOffPart = kOffSY + kNoAllocMaxCells;           // reduction partials
-constexpr size_t kOffScal = kOffPart + (size_t)kVecBlocks * kMaxVec;
+constexpr size_t kOffScal = kOffPart + (size_t)kNormValues * kRedBlocks;
 constexpr size_t kOffCount = kOffScal + S_COUNT;                 // completion counter
 constexpr size_t kScratchDoubles = ((kOffCount + 1 + 31) / 32) * 32;
 
