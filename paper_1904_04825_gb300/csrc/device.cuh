@@ -63,18 +63,28 @@ __device__ __forceinline__ void euler_fluxes(const double q[4], double gam, doub
   g[3] = v * (q[3] + p);
 }
 
-// Normal flux along +x (dir 0) or +y (dir 1), plus |u_n| + c.
-template <bool FR = false, bool FS = FR>
-__device__ __forceinline__ double normal_flux(const double q[4], int dir, double gam, double f[4]) {
+// Normal flux along +x (dir 0) or +y (dir 1) of mass and momentum, the factors
+// un, h of the energy's un h, and |u_n| + c.
+template <bool FR, bool FS>
+__device__ __forceinline__ double normal_flux_parts(const double q[4], int dir, double gam, double f[3], double* un_,
+                                                    double* h) {
   const double rinv = rcp_of<FR>(q[0]);
   const double u = q[1] * rinv, v = q[2] * rinv;
   const double p = (gam - 1.0) * (q[3] - 0.5 * (q[1] * u + q[2] * v));
   const double un = dir == 0 ? u : v;
-  f[0] = q[1 + dir];
+  f[0] = dir == 0 ? q[1] : q[2];
   f[1] = q[1] * un + (dir == 0 ? p : 0.0);
   f[2] = q[2] * un + (dir == 1 ? p : 0.0);
-  f[3] = un * (q[3] + p);
+  *un_ = un;
+  *h = q[3] + p;
   return fabs(un) + sqrt_of<FS>(gam * p * rinv);
+}
+template <bool FR = false, bool FS = FR>
+__device__ __forceinline__ double normal_flux(const double q[4], int dir, double gam, double f[4]) {
+  double un, h;
+  const double a = normal_flux_parts<FR, FS>(q, dir, gam, f, &un, &h);
+  f[3] = un * h;
+  return a;
 }
 
 // Rusanov common flux f_n = (f(qm)+f(qp))/2 - lam/2 (qp - qm),
@@ -89,18 +99,31 @@ __device__ __forceinline__ void rusanov(const double qm[4], const double qp[4], 
   for (int v = 0; v < 4; ++v) out[v] = 0.5 * (fm[v] + fp[v]) - 0.5 * lam * (qp[v] - qm[v]);
 }
 
+// Sum of two sides' normal fluxes; the energy's products are summed with one rounding
+// of one of them, which left to the compiler rounds both (errors of R against 64 bits
+// 1.003 to 1.02 times those of the flux halved side by side).
+template <bool FR, bool FS>
+__device__ __forceinline__ void flux_sum(const double qm[4], const double qp[4], int dir, double gam, double s[4],
+                                         double* am, double* ap) {
+  double fm[3], fp[3], um, up, hm, hp;
+  *am = normal_flux_parts<FR, FS>(qm, dir, gam, fm, &um, &hm);
+  *ap = normal_flux_parts<FR, FS>(qp, dir, gam, fp, &up, &hp);
+#pragma unroll
+  for (int v = 0; v < 3; ++v) s[v] = fm[v] + fp[v];
+  s[3] = fma(um, hm, up * hp);
+}
+
 // Twice the Rusanov flux (the caller's coefficients carry the 1/2): 3 FP64
 // operations per variable instead of 4.  FR: the fast reciprocal (the root is
 // always the fast one; it only scales the jump).
 template <bool FR>
 __device__ __forceinline__ void rusanov2(const double qm[4], const double qp[4], int dir, double gam,
                                          double out[4]) {
-  double fm[4], fp[4];
-  const double am = normal_flux<FR, true>(qm, dir, gam, fm);
-  const double ap = normal_flux<FR, true>(qp, dir, gam, fp);
+  double s[4], am, ap;
+  flux_sum<FR, true>(qm, qp, dir, gam, s, &am, &ap);
   const double lam = max_nonneg(am, ap);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) out[v] = fma(-lam, qp[v] - qm[v], fm[v] + fp[v]);
+  for (int v = 0; v < 4; ++v) out[v] = fma(-lam, qp[v] - qm[v], s[v]);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -216,9 +239,14 @@ __device__ __forceinline__ void write_eps(const EpsArgs& ea, double nz2) {
 template <bool FAST = false>
 __device__ __forceinline__ void roe(const double qm[4], const double qp[4], int dir, double gam,
                                     double out[4]) {
-  double fm[4], fp[4];
-  (void)normal_flux<FAST>(qm, dir, gam, fm);
-  (void)normal_flux<FAST>(qp, dir, gam, fp);
+  double fm[4], fp[4], fs[4];
+  if (FAST) {
+    double am, ap;
+    flux_sum<FAST, FAST>(qm, qp, dir, gam, fs, &am, &ap);
+  } else {
+    (void)normal_flux<FAST>(qm, dir, gam, fm);
+    (void)normal_flux<FAST>(qp, dir, gam, fp);
+  }
   const double rim = rcp_of<FAST>(qm[0]), rip = rcp_of<FAST>(qp[0]);
   const double um = qm[1] * rim, vm = qm[2] * rim, up = qp[1] * rip, vp = qp[2] * rip;
   const double pm = (gam - 1.0) * (qm[3] - 0.5 * (qm[1] * um + qm[2] * vm));
@@ -252,7 +280,7 @@ __device__ __forceinline__ void roe(const double qm[4], const double qp[4], int 
     d[3] = l1 * (H - v * a) + l2 * k2 + l3 * u + l4 * (H + v * a);
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) out[k] = FAST ? (fm[k] + fp[k]) - d[k] : 0.5 * (fm[k] + fp[k]) - 0.5 * d[k];
+  for (int k = 0; k < 4; ++k) out[k] = FAST ? fs[k] - d[k] : 0.5 * (fm[k] + fp[k]) - 0.5 * d[k];
 }
 
 // the common inviscid flux selected by fr_opts.riemann (0 Rusanov, 1 Roe)

@@ -29,6 +29,19 @@ __global__ void k_barrier_rounds(unsigned* counter, unsigned start, int* notes, 
   }
 }
 
+// The common fluxes of n pairs of states, qm and qp [n][4], along direction dir:
+// by the operations of R(U) and A z, which give twice the flux, and by those of the
+// element blocks.
+__global__ void k_fluxes(int n, const double* qm, const double* qp, int kind, int dir, double* fast, double* full) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double a[4];
+  frk::riemann_flux2(kind, qm + 4 * i, qp + 4 * i, dir, 1.4, a);
+  for (int v = 0; v < 4; ++v) fast[4 * i + v] = 0.5 * a[v];
+  frk::riemann_flux(kind, qm + 4 * i, qp + 4 * i, dir, 1.4, a);
+  for (int v = 0; v < 4; ++v) full[4 * i + v] = a[v];
+}
+
 // Inverse of the row-major n x n FP64 matrix M, one CTA, by gjfx::invert.
 template <int NB> struct InverseLayout {
   static constexpr int LD = NB + 1, THREADS = NB <= 64 ? 128 : 256;
@@ -79,6 +92,23 @@ extern "C" int fp64_inverse(int n, const double* M, double* inv) {
     case 144: return inverse<144>(M, inv);
     default: return -1;
   }
+}
+
+// 0 and the fluxes (k_fluxes; host arrays), or -1.
+extern "C" int fluxes(int n, const double* qm, const double* qp, int kind, int dir, double* fast, double* full) {
+  const size_t bytes = (size_t)n * 4 * sizeof(double);
+  double* d = nullptr;
+  if (n < 1 || cudaMalloc(&d, 4 * bytes) != cudaSuccess) return -1;
+  int rc = -1;
+  if (cudaMemcpy(d, qm, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+      cudaMemcpy(d + 4 * n, qp, bytes, cudaMemcpyHostToDevice) == cudaSuccess) {
+    k_fluxes<<<(n + 255) / 256, 256>>>(n, d, d + 4 * n, kind, dir, d + 8 * n, d + 12 * n);
+    if (cudaGetLastError() == cudaSuccess && cudaMemcpy(fast, d + 8 * n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess &&
+        cudaMemcpy(full, d + 12 * n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess)
+      rc = 0;
+  }
+  cudaFree(d);
+  return rc;
 }
 
 // Errors of `rounds` rounds over nblk CTAs from the counter value `start`, or -1.

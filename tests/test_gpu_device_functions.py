@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 import synthetic as S
-from oracle.fr2d import Mesh
+from oracle.fr2d import Mesh, roe, rusanov
 from oracle.jfnk import Problem, element_blocks
 
 pytestmark = pytest.mark.gpu
@@ -26,10 +26,14 @@ def dev(tmp_path_factory):
     return ctypes.CDLL(out)
 
 
+def _dp(a):
+    assert a.dtype == np.float64 and a.flags.c_contiguous
+    return a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+
+
 def _inverse(dev, M):
-    out = np.empty_like(M)
-    D = ctypes.POINTER(ctypes.c_double)
-    assert dev.fp64_inverse(len(M), np.ascontiguousarray(M).ctypes.data_as(D), out.ctypes.data_as(D)) == 0
+    M, out = np.ascontiguousarray(M), np.empty(M.shape)
+    assert dev.fp64_inverse(len(M), _dp(M), _dp(out)) == 0
     return out
 
 
@@ -108,3 +112,25 @@ def test_grid_barrier_over_the_wrap_of_its_counter(dev, nblk):
     carry the done bit."""
     for start in (0, 2**32 - 40 * nblk, 2**31 - 40 * nblk):
         assert dev.check_barrier(nblk, ctypes.c_uint(start), 60) == 0
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("direction", [0, 1])
+@pytest.mark.parametrize("jump", [0.3, 1e-3])
+def test_common_flux_is_as_accurate_as_with_the_full_operations(dev, kind, direction, jump):
+    """The common flux of R(U) and A z (reciprocals and roots by one step from the approximate units,
+    both sides' fluxes summed undivided) against the extended-precision flux: per variable, its rms error
+    is no larger than that of the IEEE form of the element blocks.  The two share most of their roundings;
+    the ratio of two rms errors over n samples scatters by less than 1 / sqrt(2 n) = 0.16 % for n = 2e5:
+    bound 1 + 3 * 0.0016."""
+    n = 200_000
+    rng = np.random.default_rng(7)
+    rho, u, v, p = rng.uniform(0.5, 2.0, n), rng.normal(0, 1.0, n), rng.normal(0, 1.0, n), rng.uniform(0.5, 6.0, n)
+    qm = S.conserved(rho, u, v, p)
+    d = jump * rng.uniform(-1.0, 1.0, (4, n))
+    qp = S.conserved(rho * (1.0 + d[0]), u + d[1], v + d[2], p * (1.0 + d[3]))
+    fast, full = np.empty_like(qm), np.empty_like(qm)
+    assert dev.fluxes(n, _dp(qm), _dp(qp), kind, direction, _dp(fast), _dp(full)) == 0
+    exact = (roe if kind else rusanov)(qm.T.astype(np.longdouble), qp.T.astype(np.longdouble), direction, np.longdouble(1.4))
+    rms = [np.sqrt(np.mean((f.T - exact) ** 2, axis=1)) for f in (fast, full)]
+    assert (rms[0] <= 1.005 * rms[1]).all(), rms[0] / rms[1]
