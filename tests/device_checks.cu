@@ -42,6 +42,38 @@ __global__ void k_fluxes(int n, const double* qm, const double* qp, int kind, in
   for (int v = 0; v < 4; ++v) full[4 * i + v] = a[v];
 }
 
+// rcp_fast and sqrt_fast against the correctly rounded operations at n arguments of
+// every exponent that the fast forms take: out[0], out[2] the largest difference in
+// units in the last place, out[1], out[3] how many differ.
+__global__ void k_rcp_sqrt(unsigned n, unsigned long long* out) {
+  const auto bits = [](double x) { return __double_as_longlong(x); };
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    unsigned long long h = (i + 1) * 0x9e3779b97f4a7c15ull;  // a mixed counter: mantissa and exponent
+    h = (h ^ (h >> 30)) * 0xbf58476d1ce4e5b9ull;
+    h = (h ^ (h >> 27)) * 0x94d049bb133111ebull;
+    h ^= h >> 31;
+    const unsigned long long e = 0x030 + (h >> 52) % 0x790;
+    const double x = __longlong_as_double((long long)(e << 52 | (h & 0xfffffffffffffull)));
+    const unsigned long long a = llabs(bits(frk::rcp_fast(x)) - bits(1.0 / x)), b = llabs(bits(frk::sqrt_fast(x)) - bits(sqrt(x)));
+    if (a) {
+      atomicMax(out, a);
+      atomicAdd(out + 1, 1ull);
+    }
+    if (b) {
+      atomicMax(out + 2, b);
+      atomicAdd(out + 3, 1ull);
+    }
+  }
+}
+// both at given arguments, out [2][n]
+__global__ void k_rcp_sqrt_at(int n, const double* x, double* out) {
+  const int i = threadIdx.x;
+  if (i < n) {
+    out[i] = frk::rcp_fast(x[i]);
+    out[n + i] = frk::sqrt_fast(x[i]);
+  }
+}
+
 // Inverse of the row-major n x n FP64 matrix M, one CTA, by gjfx::invert.
 template <int NB> struct InverseLayout {
   static constexpr int LD = NB + 1, THREADS = NB <= 64 ? 128 : 256;
@@ -105,6 +137,31 @@ extern "C" int fluxes(int n, const double* qm, const double* qp, int kind, int d
     k_fluxes<<<(n + 255) / 256, 256>>>(n, d, d + 4 * n, kind, dir, d + 8 * n, d + 12 * n);
     if (cudaGetLastError() == cudaSuccess && cudaMemcpy(fast, d + 8 * n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess &&
         cudaMemcpy(full, d + 12 * n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess)
+      rc = 0;
+  }
+  cudaFree(d);
+  return rc;
+}
+
+extern "C" int rcp_sqrt(unsigned n, unsigned long long* out) {
+  unsigned long long* d = nullptr;
+  if (cudaMalloc(&d, 4 * sizeof(*out)) != cudaSuccess) return -1;
+  int rc = -1;
+  if (cudaMemset(d, 0, 4 * sizeof(*out)) == cudaSuccess) {
+    k_rcp_sqrt<<<608, 256>>>(n, d);
+    if (cudaGetLastError() == cudaSuccess && cudaMemcpy(out, d, 4 * sizeof(*out), cudaMemcpyDeviceToHost) == cudaSuccess)
+      rc = 0;
+  }
+  cudaFree(d);
+  return rc;
+}
+extern "C" int rcp_sqrt_at(int n, const double* x, double* out) {
+  double* d = nullptr;
+  if (n < 1 || n > 64 || cudaMalloc(&d, 3 * n * sizeof(double)) != cudaSuccess) return -1;
+  int rc = -1;
+  if (cudaMemcpy(d, x, n * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess) {
+    k_rcp_sqrt_at<<<1, 64>>>(n, d, d + n);
+    if (cudaGetLastError() == cudaSuccess && cudaMemcpy(out, d + n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost) == cudaSuccess)
       rc = 0;
   }
   cudaFree(d);

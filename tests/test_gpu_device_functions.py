@@ -134,3 +134,24 @@ def test_common_flux_is_as_accurate_as_with_the_full_operations(dev, kind, direc
     exact = (roe if kind else rusanov)(qm.T.astype(np.longdouble), qp.T.astype(np.longdouble), direction, np.longdouble(1.4))
     rms = [np.sqrt(np.mean((f.T - exact) ** 2, axis=1)) for f in (fast, full)]
     assert (rms[0] <= 1.005 * rms[1]).all(), rms[0] / rms[1]
+
+
+def test_fast_reciprocal_and_root(dev):
+    """One step of third order from the approximate units.  1 / x: the approximation is within 2^-19.9, the
+    step leaves 2^-59.7 of x, so the rounding is right except within 1/100 of the last place of a tie:
+    one unit at most, in fewer than 1e-3 of the arguments.  The root starts from a rounded x r, whose error
+    enters with half its size: at most 1/2 + 1/4 units and the step's 2^-59, so one unit at most, less
+    often than in a quarter.  Arguments at the ends of the range and beyond take the full operations."""
+    n = 1 << 24
+    out = (ctypes.c_ulonglong * 4)()
+    assert dev.rcp_sqrt(n, out) == 0
+    assert out[0] <= 1 and out[1] <= 1e-3 * n
+    assert out[2] <= 1 and out[3] <= 0.25 * n
+    tiny, big = np.finfo(np.float64).tiny, np.finfo(np.float64).max
+    x = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, tiny / 2, tiny, big, -big, -1.0, -tiny, 2.0**-974, 2.0**962,
+                  2.0**-975, 2.0**961])
+    got = np.empty((2, x.size))
+    assert dev.rcp_sqrt_at(x.size, _dp(x), _dp(got)) == 0
+    with np.errstate(divide="ignore", invalid="ignore", over="ignore"):
+        assert np.array_equal(got[0], 1.0 / x, equal_nan=True)
+        assert np.array_equal(got[1], np.sqrt(x), equal_nan=True)
