@@ -34,9 +34,12 @@ __device__ __forceinline__ double sqrt_fast(double x) {
   return fma(g, fma(e, 0.375, 0.5) * e, g);
 }
 // The larger of two non-negative values by their bit patterns (fmax takes 2.3
-// FP64 slots); a NaN wins.
+// FP64 slots).  The offset brings the patterns of a NaN of either sign below
+// those of zero to infinity, so the number wins over a NaN, as in fmax: a side
+// of a face without a speed of sound takes the other's.
 __device__ __forceinline__ double max_nonneg(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+  constexpr unsigned long long kOff = 0x800fffffffffffffull;
+  return (unsigned long long)__double_as_longlong(a) + kOff > (unsigned long long)__double_as_longlong(b) + kOff ? a : b;
 }
 // FAST selects them.  The finite-difference element blocks and the FP32-linear-
 // parts products keep the correctly rounded operations: they subtract fluxes

@@ -74,6 +74,10 @@ __global__ void k_rcp_sqrt_at(int n, const double* x, double* out) {
   }
 }
 
+__global__ void k_max_nonneg(int n, const double* a, const double* b, double* out) {
+  if ((int)threadIdx.x < n) out[threadIdx.x] = frk::max_nonneg(a[threadIdx.x], b[threadIdx.x]);
+}
+
 // Inverse of the row-major n x n FP64 matrix M, one CTA, by gjfx::invert.
 template <int NB> struct InverseLayout {
   static constexpr int LD = NB + 1, THREADS = NB <= 64 ? 128 : 256;
@@ -163,6 +167,20 @@ extern "C" int rcp_sqrt_at(int n, const double* x, double* out) {
     k_rcp_sqrt_at<<<1, 64>>>(n, d, d + n);
     if (cudaGetLastError() == cudaSuccess && cudaMemcpy(out, d + n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost) == cudaSuccess)
       rc = 0;
+  }
+  cudaFree(d);
+  return rc;
+}
+
+extern "C" int max_nonneg(int n, const double* a, const double* b, double* out) {
+  double* d = nullptr;
+  const size_t bytes = n * sizeof(double);
+  if (n < 1 || n > 256 || cudaMalloc(&d, 3 * bytes) != cudaSuccess) return -1;
+  int rc = -1;
+  if (cudaMemcpy(d, a, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+      cudaMemcpy(d + n, b, bytes, cudaMemcpyHostToDevice) == cudaSuccess) {
+    k_max_nonneg<<<1, 256>>>(n, d, d + n, d + 2 * n);
+    if (cudaGetLastError() == cudaSuccess && cudaMemcpy(out, d + 2 * n, bytes, cudaMemcpyDeviceToHost) == cudaSuccess) rc = 0;
   }
   cudaFree(d);
   return rc;

@@ -155,3 +155,44 @@ def test_fast_reciprocal_and_root(dev):
     with np.errstate(divide="ignore", invalid="ignore", over="ignore"):
         assert np.array_equal(got[0], 1.0 / x, equal_nan=True)
         assert np.array_equal(got[1], np.sqrt(x), equal_nan=True)
+
+
+def test_larger_wave_speed_ignores_a_nan_of_either_sign(dev):
+    """The larger of two non-negative values by their bit patterns gives what fmax gives, whatever the
+    sign bit of a NaN (the root of a negative pressure comes with it set)."""
+    neg_nan = np.copysign(np.nan, -1.0)
+    v = [0.0, 5e-324, 1e-300, 1.0, np.nextafter(1.0, 2.0), 3.5, 1e300, np.inf, np.nan, neg_nan]
+    a, b = (np.ascontiguousarray(m.ravel()) for m in np.meshgrid(np.array(v), np.array(v)))
+    out = np.empty_like(a)
+    assert dev.max_nonneg(a.size, _dp(a), _dp(b), _dp(out)) == 0
+    assert np.array_equal(out, np.fmax(a, b), equal_nan=True)
+
+
+@pytest.mark.parametrize("p", [2, 3])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_negative_pressure_on_one_side_of_a_face(monkeypatch, dim, p):
+    """An element whose pressure is negative has no speed of sound; the faces to its neighbours take the
+    neighbours' wave speed, as fmax does: R(U) equals the oracle's with fmax, to its 1e-12."""
+    import torch
+    import oracle.fr3d
+    import paper_1904_04825_gb300 as fr
+    opts = fr.default_opts(precond=0, m_max=1, gmres_m=1)
+    if dim == 2:
+        xe, ye = S.stretched_mesh(5, 4, seed=p)
+        U = S.smooth_random_state(*S.point_coords(xe, ye, p), seed=1, amp=0.05)
+        ctx = fr.Context(xe, ye, p, opts)
+    else:
+        e = S.stretched_mesh3d(4, 3, 5, seed=p)
+        U = S.TaylorGreen().state(*S.point_coords3d(*e, p))
+        ctx = fr.Context3D(*e, p, opts)
+    kin = 0.5 * (U[7, 1:-1] ** 2).sum(0) / U[7, 0]
+    U[7, -1] = kin - 0.3 * (U[7, -1] - kin)  # pressure times -0.3
+    R = ctx.empty()
+    fr.fr_residual(ctx, torch.from_numpy(U).cuda(), R)
+    R = R.cpu().numpy()
+    with monkeypatch.context() as m, np.errstate(invalid="ignore"):
+        m.setattr(np, "maximum", np.fmax)  # the oracle's wave speed
+        want = (Problem(Mesh(xe, ye), p).R(U) if dim == 2 else
+                oracle.fr3d.residual3d(U, oracle.fr3d.Mesh3D(*e), p, oracle.fr3d.Gas3D(mu=0.0)))
+    assert np.isfinite(want).all()
+    assert np.linalg.norm(R - want) < 1e-12 * np.linalg.norm(want)
