@@ -473,7 +473,9 @@ int fr_batch_step_bdf2(fr_batch* batch, double dt, double* const* U, double* con
  * another vec_blocks changes their rounding order. */
 int fr_set_launch_config(fr_ctx* ctx, int vec_blocks, int tile_variant);
 int fr_get_launch_config(const fr_ctx* ctx, int* vec_blocks, int* tile_variant);
-/* Time full GMRES(gmres_m) cycles of A = shift I - dR/dU at U (device) for
+/* Time full GMRES(gmres_m) cycles of A = shift I - dR/dU at U (device), in the
+ * form the context's solves take (one launch on small 2D Euler contexts,
+ * separate launches elsewhere and on a batch's instances), for
  * vec_blocks in {152, 304, 456, 608, 912, 1216} x both tile variants and
  * keep the fastest; ms_best / ms_default (host, may be NULL) = time of one
  * cycle with the chosen / the configuration found on entry.  Overwrites the

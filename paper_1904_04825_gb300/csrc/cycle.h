@@ -59,6 +59,9 @@ bool solves_in_one_launch(const fr_ctx* ctx, int m);
 int fill_cycle_args(fr_ctx* ctx, const double* U, const double* R0, double shift, double rtol, int m, int max_restarts,
                     CycleArgs* a);
 int launch_cycle(int prec, const CycleArgs& a, int nblocks, int riemann, cudaStream_t s);
+// one solve in one launch on the stream; its status lies in ctx->h_cyc when it is done
+int launch_solve(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x, int m,
+                 double rtol, int max_restarts, bool x_is_zero, cudaStream_t s);
 // CTAs of a solve
 int cycle_grid(const fr_ctx* ctx);
 

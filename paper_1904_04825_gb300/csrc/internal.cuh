@@ -176,6 +176,7 @@ struct fr_ctx {
   unsigned wait_polls = 1u << 22;  // poll limit of the element-Jacobi apply's bounded waits
   int test_skip_copy = 0;    // test hook: the apply leaves one copy unissued (see fr_set_wait_test)
   int vec_blocks = frk::kVecBlocks;  // grid of the streaming vector kernels (autotuned)
+  int in_batch = 0;          // a batch's instance (its ROW cycles replay separate launches)
   int tile_variant = 0;      // element-tile shape of the Euler residual kernel (autotuned)
   frk::Reduce red{};
   frk::GmresDev gd{};

@@ -372,18 +372,24 @@ int fill_cycle_args(fr_ctx* ctx, const double* U, const double* R0, double shift
   return a->agrid > 0 ? FR_OK : FR_ERR_UNSUPPORTED;
 }
 
-namespace {
-int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x, int m,
-                     double rtol, int max_restarts, bool x_is_zero, fr_gmres_info* info, cudaStream_t s) {
+int launch_solve(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x, int m,
+                 double rtol, int max_restarts, bool x_is_zero, cudaStream_t s) {
   CycleArgs a;
   FRK_TRY(fill_cycle_args(ctx, U, R0, shift, rtol, m, max_restarts, &a));
   a.b = b;
   a.x = x;
   a.x_zero = x_is_zero;
-  ctx->h_cyc->err = 1;
   if (launch_cycle(ctx->opts.block_precision, a, cycle_grid(ctx), ctx->opts.riemann, s) !=
       FR_OK)
     return set_error(ctx, FR_ERR_CUDA, "launch of the solve failed: %s", cudaGetErrorString(cudaGetLastError()));
+  return FR_OK;
+}
+
+namespace {
+int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shift, const double* b, double* x, int m,
+                     double rtol, int max_restarts, bool x_is_zero, fr_gmres_info* info, cudaStream_t s) {
+  ctx->h_cyc->err = 1;
+  FRK_TRY(launch_solve(ctx, U, R0, shift, b, x, m, rtol, max_restarts, x_is_zero, s));
   FRK_CUDA(ctx, cudaStreamSynchronize(s));
   const CycleStatus& st = *ctx->h_cyc;
   if (st.err) {  // a wait of this launch, or of an inversion or apply before it

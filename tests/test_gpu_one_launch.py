@@ -168,3 +168,22 @@ def test_first_solves_of_a_process_on_several_threads():
            for how in ("threads", "in turn")]
     assert out[0].returncode == 0 and out[1].returncode == 0, out[0].stderr + out[1].stderr
     assert out[0].stdout == out[1].stdout
+
+
+def test_autotune_times_the_form_that_solves_take(fr):
+    """Thirteen configurations of two cycles: two launches each and a few where the solves run as one
+    launch; with a restart length that does not fit, and on a batch's instance, dozens per cycle."""
+    p, m = 2, 30
+    xe, ye = S.uniform_mesh(12)
+    U = _t(S.Vortex().state(*S.point_coords(xe, ye, p)))
+
+    def launches(ctx):
+        n = fr.fr_kernel_launches()
+        vb, tv, best, default = fr.autotune(ctx, U, 20.0, reps=1)
+        assert 0.0 < best <= default
+        return fr.fr_kernel_launches() - n
+
+    assert 13 * 2 <= launches(fr.Context(xe, ye, p, fr.default_opts(gmres_m=m))) <= 13 * 2 + 10
+    assert launches(fr.Context(xe, ye, p, fr.default_opts(m_max=60, gmres_m=60))) > 13 * 2 * 60
+    B = fr.Batch([(xe, ye)], [p], fr.default_opts(gmres_m=m))
+    assert launches(B.members[0]) > 13 * 2 * m
