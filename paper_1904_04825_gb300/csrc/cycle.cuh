@@ -250,7 +250,7 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
   const bool keeper = g.bid == g.nblk - 1;  // the CTA that keeps the Hessenberg column
   bool x_zero = a.x_zero != 0;
   int iters = 0, iterated = 0, state = kCycleNotConverged;
-  double res = 0.0, target = 0.0;
+  double res = 0.0, target = 0.0, relres = 0.0;
   unsigned done_add = 0u;  // keeper's thread 0: what its next arrival adds
   bool done_set = false;   // ... and whether the done bit is set
 
@@ -370,12 +370,14 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
         backsub(gd, k, reinterpret_cast<double*>(smem), s.ys);
         solution_phase<NB, S, A>(a, x, k, s.ys, x_zero && cycle == 0, g, smem);
       }
-      iters += k;
-      if (k > 0) ++iterated;
-      if (!isfinite(res) || !isfinite(bn)) {
+      if (!isfinite(res) || !isfinite(bn)) {  // the cycles before this one are reported
         state = kCycleNonFinite;
+        if (k > 0) ++iterated;
         break;
       }
+      iters += k;
+      if (k > 0) ++iterated;
+      relres = res / bn;
       if (res <= target) {
         state = kCycleConverged;
         break;
@@ -389,7 +391,7 @@ __device__ __noinline__ void solve(const CycleArgs& a, Grid& g, Shared& s, unsig
     st->iters = iters;
     st->restarts = iterated > 0 ? iterated - 1 : 0;
     st->state = state;
-    st->relres = nb2 == 0.0 ? 0.0 : res / bn;
+    st->relres = relres;
   }
 }
 

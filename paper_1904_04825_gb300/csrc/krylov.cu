@@ -398,15 +398,15 @@ int gmres_one_launch(fr_ctx* ctx, const double* U, const double* R0, double shif
     FRK_CUDA(ctx, cudaStreamSynchronize(s));
     return set_error(ctx, FR_ERR_TIMEOUT, "a kernel's bounded wait gave up");
   }
-  if (st.state == kCycleNonFinite) {
-    if (info) *info = fr_gmres_info{};
-    return set_error(ctx, FR_ERR_NONFINITE, "GMRES residual is not finite");
-  }
   fr_gmres_info loc{};
   loc.iters = st.iters;
+  loc.relres = st.relres;
+  if (st.state == kCycleNonFinite) {
+    if (info) *info = loc;
+    return set_error(ctx, FR_ERR_NONFINITE, "GMRES residual is not finite");
+  }
   loc.restarts = st.restarts;
   loc.converged = st.state == kCycleConverged;
-  loc.relres = st.relres;
   if (info) *info = loc;
   if (!loc.converged)
     return set_error(ctx, FR_ERR_NOT_CONVERGED, "GMRES stopped after %d iterations at relres %.3e", loc.iters, loc.relres);

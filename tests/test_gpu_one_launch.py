@@ -187,3 +187,33 @@ def test_autotune_times_the_form_that_solves_take(fr):
     assert launches(fr.Context(xe, ye, p, fr.default_opts(m_max=60, gmres_m=60))) > 13 * 2 * 60
     B = fr.Batch([(xe, ye)], [p], fr.default_opts(gmres_m=m))
     assert launches(B.members[0]) > 13 * 2 * m
+
+
+def test_solve_that_turns_non_finite_in_a_later_cycle_reports_the_earlier_ones(fr):
+    """On cells 1e100 wide ||x||^2 overflows, so the second cycle's difference step is zero and its
+    residual b - shift x, 1.10 ||b|| here (by the oracle); with ||b|| = 1.28e154, whose square is below
+    1.8e308, that one's square is not: one launch reports what the separate launches do, the first
+    cycle's iterations and residual."""
+    import ctypes
+    import torch
+    p, m, scale = 2, 10, 1e100
+    xe, ye = S.uniform_mesh(6)
+    U = _t(S.Vortex().state(*S.point_coords(xe, ye, p)))
+    ctx = fr.Context(xe * scale, ye * scale, p)
+    R0 = ctx.empty()
+    fr.fr_residual(ctx, U, R0)
+    fr.ejacobi_factor(ctx, U, R0, 1.0 / scale)
+    b = S.random_vector(tuple(U.shape), 1)
+    b = _t(b * (1.28e154 / np.linalg.norm(b)))
+    infos = []
+    for timed in (False, True):
+        if timed:
+            fr.fr_profile_begin(ctx, ["dots"])
+        x, info = torch.zeros_like(b), fr.fr_gmres_info()
+        rc = fr.lib.gmres_solve(ctx.handle, U.data_ptr(), R0.data_ptr(), 1.0 / scale, b.data_ptr(), x.data_ptr(), m, 1e-12,
+                                5, ctypes.byref(info), None)
+        assert rc == fr.FR_ERR_NONFINITE
+        infos.append((info.iters, info.restarts, info.converged, info.relres))
+    fr.fr_profile_end(ctx)
+    assert infos[0] == infos[1] and infos[0][0] == m
+    ctx.close()
