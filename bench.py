@@ -810,7 +810,7 @@ def kernel_arm(args):
     out = {"kernel": args.kernel, "workload": args.workload, "ndof": ctx.ndof,
            "block_precision": args.block_precision, "jv_precision": args.jv_precision}
     out.update(summary(prof[args.kernel]))
-    if args.kernel == "factor" and prof["invert"]["launches"]:
+    if args.kernel == "factor" and "invert" in prof:  # viscous and 3D contexts
         out["invert"] = summary(prof["invert"])
     print(json.dumps(out))
     return 0
