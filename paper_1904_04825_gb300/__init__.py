@@ -407,7 +407,7 @@ def step_ssprk3(ctx: Context, dt: float, U, stream=None):
 
 
 def fr_set_wait_test(ctx: Context, polls: int = 0, skip_first_copy: bool = False):
-    """Test hook for the element-Jacobi apply's bounded waits (see the C header)."""
+    """Test hook for the bounded waits of the element-Jacobi apply and of the one-launch solve (see the C header)."""
     return ctx.check(lib.fr_set_wait_test(ctx.handle, int(polls), int(bool(skip_first_copy))))
 
 

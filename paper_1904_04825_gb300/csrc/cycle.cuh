@@ -1,4 +1,4 @@
-// Restarted GMRES(m) of one linear solve (or of a batch of them) in one launch.
+// Restarted GMRES(m) of one linear solve in one launch.
 //
 // The launches of krylov.cu take seven kernels per Arnoldi iteration, and on a
 // small mesh each of them is latency (5 us of host time to launch, 5 to 20 us to

@@ -1,5 +1,5 @@
 // The guess network's whole BF16 inference in one kernel: Y = W3 relu(W2 relu(W1 x
-// + b1) + b2) + b3 for 128-row tiles of X, hidden activations in shared memory.
+// + b1) + b2) + b3 for 128-row tiles of X, hidden activations in tensor memory.
 //
 // Layer by layer (umma_ws.cuh) the activations cross memory three times as BF16
 // after a conversion pass; here X is read once in FP32 and Y written once, and

@@ -13,7 +13,7 @@
 //    solution points, the corrected divergence with the four faces' common
 //    fluxes, the body-force source and the output.  Both elements of a face
 //    read the same stored flux, so conservation holds to round-off.
-// Bound: FP64 issue.  R + A z at 256 x 128, p = 3: 660 us; 963 us when all
+// Bound: FP64 issue.  R + A z at 256 x 128, p = 3: 655 us; 963 us when all
 // three derivatives were traced from both sides, both viscous fluxes formed on
 // every face, q_com - q subtracted at every point, a third of the face threads
 // kept for walls, and 2 / h divided out by every thread.

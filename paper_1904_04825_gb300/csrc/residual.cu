@@ -14,7 +14,7 @@
 // into Dt, which removes their extrapolation from the flop count).
 //
 // Bound: FP64 issue (two operations per clock and SM).  At 512^2, p = 3, R and
-// A z with its two norms take 2241 us together; with IEEE divisions, roots and
+// A z with its two norms take 2114 us together; with IEEE divisions, roots and
 // fmax in the fluxes, two divisions per thread for the metric and one load in
 // flight in the norms they took 2718 us.
 #include "residual_body.cuh"
